@@ -49,6 +49,7 @@ struct geo_batch_s {
     int64_t max_end = 0;
     int32_t segs = 0;
     int32_t vox = 0;            // a volume has a uniform grid
+    int32_t max_nf = 0;         // filter entries of the largest volume
     int64_t* d_idx = nullptr;   // track indices of packed tiles
     VolView* d_vols = nullptr;
     BatchTile* d_tiles = nullptr;
@@ -335,6 +336,8 @@ bool make_rec32(const geo_placed_shape& s, double grow, double delta, ShapeRec32
         r.e[4] = float_up(ro * ro);
         r.e[5] = hole && ri > 0 ? float_down(ri * ri) : 0.f;
         r.e[6] = float_up(dz + delta);
+        r.e[7] = float(rmax);
+        r.e[8] = hole ? float(rmin) : 0.f;
     } else {
         const double dz = p[0], dzg = dz + g;
         if (!(dzg > 0)) return false;
@@ -369,6 +372,94 @@ bool make_rec32(const geo_placed_shape& s, double grow, double delta, ShapeRec32
     r.brad = float(bounding_radius(s) * (1.0 + 1e-6) + std::max(g, 0.0));
     r.brad2 = float_up(double(r.brad) * double(r.brad));
     return true;
+}
+
+bool needs_segs_code(const geo_placed_shape& s);
+
+// The filter's tables (layout in geo_internal.h) from the daughters `in` and
+// their FP32 copies: sorted by class, the daughters of a class in index order.
+void make_filter(const geo_placed_shape* in, const std::vector<ShapeRec32>& d, std::vector<FiltSph>& sph,
+                 std::vector<FiltHvy>& hvy, int32_t& nq1, int32_t& nq) {
+    const int nd = int(d.size());
+    std::vector<int32_t> order;   // -1: a filling entry
+    auto append = [&](auto&& wanted) {
+        for (int j = 0; j < nd; ++j)
+            if (wanted(d[j])) order.push_back(j);
+    };
+    auto even = [&] {
+        if (order.size() % 2) order.push_back(-1);
+    };
+    append([](const ShapeRec32& r) { return r.kind != KBOX && (r.flags & kRec32Identity); });
+    even();
+    nq1 = int32_t(order.size());
+    append([](const ShapeRec32& r) { return r.kind != KBOX && !(r.flags & kRec32Identity); });
+    nq = int32_t(order.size());
+    append([](const ShapeRec32& r) { return r.kind == KBOX; });
+    even();
+    const int nf = int(order.size());
+    sph.resize(static_cast<size_t>(nf));
+    hvy.resize(static_cast<size_t>(nf));
+    for (int k = 0; k < nf; ++k) {
+        FiltSph& s = sph[k];
+        FiltHvy& h = hvy[k];
+        std::memset(&h, 0, sizeof h);
+        if (order[k] < 0) {   // an annulus of negative radius; an empty sphere (below)
+            s.a = make_float4(0.f, 0.f, 0.f, 1.f);
+            s.b = make_float4(0.f, -1.f, -1.f, 0.f);
+            continue;
+        }
+        const ShapeRec32& r = d[order[k]];
+        std::memcpy(h.t, r.t, sizeof h.t);
+        std::memcpy(h.R, r.R, sizeof h.R);
+        h.delta = r.delta;
+        h.id = order[k];
+        h.flags = (r.flags & kRec32Identity) ? kFiltIdentity : 0;
+        if (r.kind == KBOX) {
+            std::memcpy(h.e, r.e, 3 * sizeof(float));
+            continue;
+        }
+        float hi[2], lo[2];   // squared acceptance limits of the end annuli at -dz, +dz
+        if (r.kind == KTUBE) {
+            const float e[5] = {r.e[2], r.e[7], 0.f, r.e[8], 0.f};
+            std::memcpy(h.e, e, sizeof e);
+            h.h = r.e[6];
+            hi[0] = hi[1] = r.e[4];
+            lo[0] = lo[1] = r.e[5];
+            if (r.e[3] != 0.f) h.flags |= kFiltHole;
+        } else {
+            std::memcpy(h.e, r.e, 5 * sizeof(float));
+            h.h = r.e[14];
+            hi[0] = r.e[10]; hi[1] = r.e[11];
+            lo[0] = r.e[12]; lo[1] = r.e[13];
+            if (r.e[5] != 0.f) h.flags |= kFiltHole;
+        }
+        h.e[5] = hi[0]; h.e[6] = hi[1]; h.e[7] = lo[0]; h.e[8] = lo[1];
+        const double slope = std::max(std::fabs(double(h.e[2])), std::fabs(double(h.e[4])));
+        h.g = float_up(4.0 * double(r.delta) * std::sqrt(1.0 + slope * slope));
+        const geo_placed_shape& sh = in[order[k]];
+        const bool has_hole = sh.kind == GEO_TUBE ? sh.p[0] > 0 : (sh.kind == GEO_CONE && (sh.p[1] > 0 || sh.p[3] > 0));
+        if (needs_segs_code(sh) || (has_hole && !(h.flags & kFiltHole))) h.flags |= kFiltLoose;
+        if (k < nq1) {
+            const bool axis = k % 32 == 0 || r.t[0] != sph[k - 1].a.x || r.t[1] != sph[k - 1].a.y;
+            s.a = make_float4(r.t[0], r.t[1], r.t[2], axis ? 1.f : 0.f);
+            s.b = make_float4(0.f, float_up(std::sqrt(double(std::max(hi[0], hi[1])))),
+                              float_down(std::sqrt(double(std::min(lo[0], lo[1])))), h.h);
+        }
+    }
+    for (int k = nq1; k < nf; k += 2) {
+        float t[2][3] = {}, b2[2] = {-1.f, -1.f}, br[2] = {};
+        for (int q = 0; q < 2; ++q) {
+            if (order[k + q] < 0) continue;
+            const ShapeRec32& r = d[order[k + q]];
+            for (int c = 0; c < 3; ++c) t[q][c] = -r.t[c];
+            b2[q] = r.brad2;
+            br[q] = r.brad;
+        }
+        sph[k].a = make_float4(t[0][0], t[1][0], t[0][1], t[1][1]);
+        sph[k].b = make_float4(t[0][2], t[1][2], b2[0], b2[1]);
+        sph[k + 1].a = make_float4(br[0], br[1], 0.f, 0.f);
+        sph[k + 1].b = make_float4(0.f, 0.f, 0.f, 0.f);
+    }
 }
 
 // Extent of the mother: an upper bound of |p| for every point inside it.
@@ -647,8 +738,14 @@ geo_status geo_build_volume(const geo_placed_shape* mother, const geo_placed_sha
         if (needs_segs_code(daughters[j])) vw.segs = 1;
 
     const size_t b64 = sizeof(ShapeRec64) * size_t(std::max(n_daughters, 1));
+    std::vector<FiltSph> hsph;
+    std::vector<FiltHvy> hhvy;
+    make_filter(daughters, h32, hsph, hhvy, vw.nq1, vw.nq);
+    // the FP32 records, then the filter's two tables
     const size_t b32 = sizeof(ShapeRec32) * size_t(std::max(n_daughters, 1));
-    if ((e = lib_malloc(&v->d64, b64)) != cudaSuccess || (e = lib_malloc(&v->d32, b32)) != cudaSuccess ||
+    vw.nf = int32_t(hsph.size());
+    const size_t bsph = sizeof(FiltSph) * hsph.size(), bhvy = sizeof(FiltHvy) * hhvy.size();
+    if ((e = lib_malloc(&v->d64, b64)) != cudaSuccess || (e = lib_malloc(&v->d32, b32 + bsph + bhvy)) != cudaSuccess ||
         (e = lib_malloc(&v->status, sizeof(unsigned int))) != cudaSuccess) {
         geo_destroy_volume(v);
         return cuda_status(e);
@@ -663,7 +760,11 @@ geo_status geo_build_volume(const geo_placed_shape* mother, const geo_placed_sha
         if ((e = cudaMemcpyAsync(v->d64, h64.data(), sizeof(ShapeRec64) * n_daughters, cudaMemcpyHostToDevice, s)) !=
                 cudaSuccess ||
             (e = cudaMemcpyAsync(v->d32, h32.data(), sizeof(ShapeRec32) * n_daughters, cudaMemcpyHostToDevice, s)) !=
-                cudaSuccess) {
+                cudaSuccess ||
+            (e = cudaMemcpyAsync(reinterpret_cast<char*>(v->d32) + b32, hsph.data(), bsph, cudaMemcpyHostToDevice, s)) !=
+                cudaSuccess ||
+            (e = cudaMemcpyAsync(reinterpret_cast<char*>(v->d32) + b32 + bsph, hhvy.data(), bhvy, cudaMemcpyHostToDevice,
+                                 s)) != cudaSuccess) {
             geo_destroy_volume(v);
             return cuda_status(e);
         }
@@ -675,6 +776,8 @@ geo_status geo_build_volume(const geo_placed_shape* mother, const geo_placed_sha
     }
     vw.d64 = v->d64;
     vw.d32 = v->d32;
+    vw.fsph = reinterpret_cast<const FiltSph*>(reinterpret_cast<char*>(v->d32) + b32);
+    vw.fhvy = reinterpret_cast<const FiltHvy*>(reinterpret_cast<char*>(v->d32) + b32 + bsph);
     vw.status = v->status;
     v->h64 = std::move(h64);
     if (opts && opts->voxelize) {
@@ -687,13 +790,13 @@ geo_status geo_build_volume(const geo_placed_shape* mother, const geo_placed_sha
     vw.smem64 = (int64_t(n_daughters) * int64_t(sizeof(ShapeRec64)) <= smem_budget(dev)) ? 1 : 0;
     // the refine kernel wants two blocks per SM: its staged tables get what
     // half of an SM's shared memory leaves beside its two stage buffers (less
-    // the per-block reservation and static shared memory); larger tables are
-    // read through L1 from global memory
+    // the per-block reservation and static shared memory); tables that do not
+    // fit are read through L1 from global memory, the FP64 records first (a
+    // track reads one of them, the filter reads all of its own)
     const int64_t stages = int64_t(refine_stage_bytes());
-    vw.smem_refine = (int64_t(n_daughters) * int64_t(sizeof(ShapeRec64) + sizeof(ShapeRec32)) <=
-                      std::min(int64_t(smem_budget(dev)) - stages, int64_t(sm_smem(dev)) / 2 - 2048 - stages))
-                         ? 1
-                         : 0;
+    const int64_t room = std::min(int64_t(smem_budget(dev)) - stages, int64_t(sm_smem(dev)) / 2 - 2048 - stages);
+    const int64_t filt = int64_t(vw.nf) * int64_t(sizeof(FiltSph) + sizeof(FiltHvy));
+    vw.smem_refine = filt + int64_t(n_daughters) * int64_t(sizeof(ShapeRec64)) <= room ? 2 : (filt <= room ? 1 : 0);
     *out = v;
     return GEO_OK;
 }
@@ -968,6 +1071,7 @@ geo_status geo_build_batch(const geo_volume* vols, int32_t n_vols, const geo_bas
     for (int i = 0; i < n_vols; ++i) {
         b->segs = b->segs || vols[i]->view.segs;
         b->vox = b->vox || vols[i]->view.voxelized;
+        b->max_nf = std::max(b->max_nf, vols[i]->view.nf);
     }
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     cudaError_t e;
@@ -1028,7 +1132,7 @@ geo_status geo_dist_to_boundary_batched(geo_batch b, const double* x, const doub
     bv.segs = b->segs;
     bv.nvols = b->n_vols;
     bv.vox = b->vox;
-    bv.pad_ = 0;
+    bv.max_nf = b->max_nf;
     bv.idx = b->d_idx;
     const Basket bk{x, y, z, dx, dy, dz, n_total};
     return cuda_status(

@@ -82,6 +82,44 @@ struct __align__(16) ShapeRec32 {
 };
 static_assert(sizeof(ShapeRec32) == 128, "ShapeRec32 layout");
 
+// The filter's own tables (filter_pass.cuh), one entry per daughter, sorted by
+// class: unrotated quadrics (tube or cone copies), rotated ones, boxes.
+// The unrotated quadrics are filled up to an even number, and the whole table
+// too, with entries that no track meets.
+//  FiltSph, read by all lanes together:
+//   unrotated quadric: a = (t, 1 where its axis differs from the entry before
+//     or its index is a multiple of 32, else 0), b = (-, Rmax, Rmin,
+//     half-length) of its bounding annulus: the inflated copy plus delta
+//   rotated quadrics and boxes by pairs (indices 2i, 2i + 1): a = (-t_x of
+//     both, -t_y of both), b = (-t_z of both, brad^2 of both); the second
+//     entry's a = (brad of both)
+//  FiltHvy, gathered per lane (112 B: seven 16-byte words, an odd number, so
+//  that gathers of different entries meet few bank conflicts):
+//   t, delta; R (9); flags, daughter index (int bits); h, e by kind:
+//   quadric: h = zl (dz' + delta); e = dz', a_out', b_out, a_in', b_in, the
+//     acceptance limits of the end annuli (hi at -dz, hi at +dz, lo at -dz, lo
+//     at +dz; see ShapeRec32); g = 4 delta sqrt(1 + the larger slope squared)
+//   box: e[0..2] = h + delta
+// kFiltLoose: the copy bounds another solid (a tube segment, a polycone, a hole
+// narrower than delta, a cone with an apex on an end plane), so that no
+// surface of it is surely the solid's.
+constexpr int32_t kFiltIdentity = 1, kFiltHole = 2, kFiltLoose = 4;
+struct __align__(16) FiltSph {
+    float4 a, b;
+};
+struct __align__(16) FiltHvy {
+    float t[3];
+    float delta;
+    float R[9];
+    int32_t flags;
+    int32_t id;
+    float h;
+    float e[9];
+    float g;
+    float pad[2];
+};
+static_assert(sizeof(FiltSph) == 32 && sizeof(FiltHvy) == 112, "filter table layout");
+
 // Everything a kernel needs about one volume, passed by value (or copied
 // from a device array of views by the batched kernel).
 struct __align__(16) VolView {
@@ -90,13 +128,19 @@ struct __align__(16) VolView {
     ShapeRec32 m32u;           // mother, FP32 inflated (upper bound of the exit)
     const ShapeRec64* d64;     // [nd] device
     const ShapeRec32* d32;     // [nd] device
+    const FiltSph* fsph;       // [nf] device, in the filter's order
+    const FiltHvy* fhvy;       // [nf] device, likewise
+    int32_t nq1;               // unrotated quadrics of the filter's order
+    int32_t nq;                // quadrics of the filter's order
+    int32_t nf;                // entries of the filter's tables
     int32_t nd;
     int32_t smem64;            // 1 if the FP64 table fits the shared-memory budget
-    int32_t smem_refine;       // 1 if the FP32 + FP64 tables fit it together
+    int32_t smem_refine;       // tables the refine kernel stages: 0 none, 1 the filter's, 2 the FP64 records too
     // voxel grid (uniform over the mother's bounding box)
     int32_t voxelized;
     int32_t grid[3];
     int32_t segs;              // 1 if the mother or a daughter is a tube segment or a polycone
+    int32_t pad_;
     double lo[3];
     double cell[3];
     double inv_cell[3];
@@ -129,7 +173,7 @@ struct BatchView {
     int32_t segs;             // 1 if a volume holds a tube segment or a polycone
     int32_t nvols;            // entries of vols
     int32_t vox;              // 1 if a volume has a uniform grid
-    int32_t pad_;
+    int32_t max_nf;           // filter entries of the largest volume
     const int64_t* idx;       // track indices of packed tiles (count < 0), or null
 };
 
@@ -151,6 +195,10 @@ cudaError_t launch_dist_refine_latency(const VolView& v, const Basket& b, double
 bool split_basket(const VolView& v, int64_t n, int num_sms);
 cudaError_t launch_dist_refine_split(const VolView& v, const Basket& b, double* step, int32_t* hit, double* bpoint,
                                      int32_t* nref, cudaStream_t s);
+
+// one thread per track (volumes without segments and polycones)
+cudaError_t launch_dist_direct(const VolView& v, const Basket& b, double* step, int32_t* hit, double* bpoint,
+                               int32_t* nref, cudaStream_t s, int num_sms);
 
 // launchers (host), each returns cudaGetLastError() of its launch
 cudaError_t launch_dist_fp64(const VolView& v, const Basket& b, double* step, int32_t* hit,

@@ -1,20 +1,23 @@
 // nav_refine.cu -- the navigator step of Fig. 1b with an FP32 filter and FP64
-// refinement (GEO_FP32_REFINE).
+// refinement (GEO_FP32_REFINE): dispatch, the batched launch.
 //
-// Pass 1 (FP32, every daughter): bounding-sphere cull against an upper bound
-// U of the mother exit, master->local transform in a frame shifted to the
-// track's closest approach to the daughter's origin, and a LOWER bound L_j of
-// DistFromOutside from the daughter's inflated FP32 copy (shapes32.cuh).  The
-// kCand = 2 smallest bounds are kept in registers, sorted.
-// Pass 2 (FP64, few solids): candidates are refined in ascending order of
-// their bounds, the mother (bound L_m of its exit) taking its place in that
-// order, with the same FP64 routines as the plain kernel; refinement stops as
-// soon as the next bound exceeds the best FP64 step.  Ties resolve as in the
-// sequential algorithm of Fig. 1a (mother, then lowest index).  If a bound
-// that had to be dropped from the list could still win, the track falls back
-// to the full FP64 loop.  Every track therefore gets exactly the plain FP64
-// kernel's answer.
+// Pass 1 (FP32, every daughter; filter_pass.cuh): a LOWER bound L_j of
+// DistFromOutside from each daughter's inflated FP32 copy that the track comes
+// near before the mother's exit (upper bound U), and where it is certain the
+// surface the track enters through.  The kCand = 2 smallest bounds are kept in
+// registers, sorted.
+// Pass 2 (FP64, one surface or few solids): candidates are refined in ascending
+// order of their bounds, the mother (bound L_m of its exit) taking its place in
+// that order, with the operations of the plain kernel's routines; refinement
+// stops as soon as the next bound exceeds the best FP64 step.  Ties resolve as
+// in the sequential algorithm of Fig. 1a (mother, then lowest index).  If a
+// bound that had to be dropped from the list could still win, the track falls
+// back to the full FP64 loop.  Every track therefore gets exactly the plain
+// FP64 kernel's answer.
 #include <cuda_runtime.h>
+
+#include <algorithm>
+
 #include "geo_internal.h"
 #include "launch.cuh"
 #include "nav_common.cuh"
@@ -30,11 +33,19 @@ size_t refine_stage_bytes() { return 2 * (sizeof(Stage<kProd>) + sizeof(Answers<
 // Batched persistent launch: tiles of many logical volumes, claimed in order
 // from a device counter (largest estimated cost first when the host sorted
 // them so), with the same producer / consumer pipeline.  The tile header of a
-// stage carries a copy of the tile's volume view; the solid tables are read
-// from global memory through L1 (a table change per tile would otherwise
-// need a restage while the other stage still uses the previous one).  A
-// packed tile (negative count) lists its tracks' indices in bv.idx from its
-// base on (the ragged tails of a volume's baskets gathered into full tiles).
+// stage carries a copy of the tile's volume view.  The filter's tables of a
+// tile's volume are copied to shared memory (bulk copy): the lanes gather
+// records of different solids from them, which through L1 costs a tag lookup
+// for each (64 volumes, 4 to 200 daughters, 2^22 tracks: 1277 us with the tables
+// read through L1 and every bound run for the union of a warp's lanes, 675 us
+// so).  The
+// tables of even tiles sit at the bottom of the table area, those of odd tiles
+// at its top; the next tile is claimed, and its tables are copied, while the
+// current one is bounded when both fit side by side, and otherwise once every
+// producer is done with the current tables.  The FP64 records are read through
+// L1 (each track reads one).  A packed tile (negative count) lists its
+// tracks' indices in bv.idx from its base on (the ragged tails of a volume's
+// baskets gathered into full tiles).
 struct __align__(16) TileHdr {
     VolView vol;
     int64_t base;
@@ -44,18 +55,31 @@ struct __align__(16) TileHdr {
     int pad[3];
 };
 
+// the next tile, as claimed by producer thread 0
+struct NextTile {
+    int64_t base;
+    int tile, count, vol_index;
+    uint32_t bytes;      // of its filter tables
+    int pending;         // 1: their copy is not issued yet
+    const void* src;
+};
+
 // SEGS = false: no volume of the batch holds a tube segment or a polycone.
-// VOX = false: no volume has a uniform grid, and the kernel carries only the
-// all-daughter FP32 pass (10 % faster on the 64-volume batch than with the
-// grid walk's code beside it).  P producer threads (one track each of a tile
-// of P) and C consumer threads.
-template <bool SEGS, bool VOX, int P, int C>
+// GLOB = false: no volume has a uniform grid and every volume's filter tables
+// fit the table area (`room` bytes); the kernel carries only the all-daughter
+// FP32 pass over staged tables (10 % faster on the 64-volume batch than with
+// the grid walk's code beside it).  GLOB = true: the tables are read from
+// global memory, a volume's grid is walked where it has one.  P producer
+// threads (one track each of a tile of P) and C consumer threads.
+template <bool SEGS, bool GLOB, int P, int C>
 __global__ void __launch_bounds__(P + C, 2) k_dist_batched(BatchView bv, Basket b, double* __restrict__ step,
-                                                              int32_t* __restrict__ hit) {
+                                                              int32_t* __restrict__ hit, uint32_t room) {
     extern __shared__ __align__(128) unsigned char smem_raw[];
-    __shared__ uint64_t full[2], done[2];
+    __shared__ uint64_t full[2], done[2], tabs[2];
+    __shared__ NextTile N;
     Stage<P>* S = reinterpret_cast<Stage<P>*>(smem_raw);
     TileHdr* H = reinterpret_cast<TileHdr*>(smem_raw + 2 * sizeof(Stage<P>));
+    unsigned char* area = smem_raw + 2 * (sizeof(Stage<P>) + sizeof(TileHdr));
     const int t = threadIdx.x;
     const int lane = t & 31;
     bool healthy = true;
@@ -64,12 +88,51 @@ __global__ void __launch_bounds__(P + C, 2) k_dist_batched(BatchView bv, Basket 
         mbar_init(&full[1], P / 32);
         mbar_init(&done[0], C / 32);
         mbar_init(&done[1], C / 32);
+        mbar_init(&tabs[0], 1);
+        mbar_init(&tabs[1], 1);
     }
     __syncthreads();
     constexpr int kWords = int(sizeof(VolView) / sizeof(int4));
 
     if (t < P) {
         // ------------------------------------------------------ producers --
+        // thread 0: copy of N's tables for tile k of this block
+        auto copy_tables = [&](int k) {
+            unsigned char* dst = (k & 1) ? area + (room - N.bytes) : area;
+            if (N.bytes == 0) {
+                mbar_arrive(&tabs[k & 1]);
+            } else {
+                mbar_expect_tx(&tabs[k & 1], N.bytes);
+                for (uint32_t off = 0; off < N.bytes; off += kChunk)
+                    bulk_g2s(dst + off, static_cast<const unsigned char*>(N.src) + off, min(kChunk, N.bytes - off),
+                             &tabs[k & 1]);
+            }
+            N.pending = 0;
+        };
+        // thread 0: claims this block's tile k; its tables are copied now when
+        // they fit beside the `used` bytes of the tile before
+        auto claim = [&](int k, uint32_t used) {
+            const unsigned q = atomicAdd(bv.counter, 1u);
+            N.pending = 0;
+            N.bytes = 0;
+            if (int64_t(q) < bv.ntiles) {
+                const BatchTile tl = bv.tiles[q];
+                N.tile = int(q);
+                N.base = tl.base;
+                N.count = tl.count;
+                N.vol_index = tl.vol;
+                if (!GLOB) {
+                    const VolView& nv = bv.vols[tl.vol];
+                    N.bytes = uint32_t(nv.nf) * uint32_t(sizeof(FiltSph) + sizeof(FiltHvy));
+                    N.src = nv.fsph;
+                    if (used + N.bytes <= room) copy_tables(k);
+                    else N.pending = 1;
+                }
+            } else {
+                N.tile = -1;
+            }
+        };
+        if (t == 0) claim(0, 0);
         for (int k = 0;; ++k) {
             Stage<P>& st_ = S[k & 1];
             TileHdr& hd = H[k & 1];
@@ -77,17 +140,12 @@ __global__ void __launch_bounds__(P + C, 2) k_dist_batched(BatchView bv, Basket 
             // have finished
             if (k >= 2) mbar_wait_bounded(&done[k & 1], uint32_t(((k - 2) >> 1) & 1), bv.status, healthy);
             if (t == 0) {
-                const unsigned q = atomicAdd(bv.counter, 1u);
-                if (int64_t(q) < bv.ntiles) {
-                    const BatchTile tl = bv.tiles[q];
-                    hd.tile = int(q);
-                    hd.base = tl.base;
-                    hd.count = tl.count;
-                    hd.vol_index = tl.vol;
-                } else {
-                    hd.tile = -1;
-                }
-                st_.cnt[0] = st_.cnt[1] = st_.cnt[2] = st_.cnt[3] = 0;
+                hd.tile = N.tile;
+                hd.base = N.base;
+                hd.count = N.count;
+                hd.vol_index = N.vol_index;
+#pragma unroll
+                for (int q = 0; q < kTaskBins; ++q) st_.cnt[q] = 0;
                 st_.next = 0;
             }
             producer_barrier<P>();
@@ -98,8 +156,21 @@ __global__ void __launch_bounds__(P + C, 2) k_dist_batched(BatchView bv, Basket 
                 const int64_t base = hd.base;
                 const bool packed = hd.count < 0;
                 const int count = packed ? -hd.count : hd.count;
+                if (t == 0) claim(k + 1, N.bytes);
                 producer_barrier<P>();
                 const VolView& v = hd.vol;
+                FiltTab f = {v.fsph, v.fhvy, v.nq1, v.nq, v.nf};
+                if (!GLOB) {
+                    // every tile's copy is waited for, so none is in flight when the block ends
+                    if (!mbar_wait_limited(&tabs[k & 1], uint32_t((k >> 1) & 1), kWaitLimit)) {
+                        atomicOr(bv.status, ST_TMA_TIMEOUT);
+                        healthy = false;
+                    }
+                    const unsigned char* tab =
+                        (k & 1) ? area + (room - uint32_t(v.nf) * uint32_t(sizeof(FiltSph) + sizeof(FiltHvy))) : area;
+                    f.sph = reinterpret_cast<const FiltSph*>(tab);
+                    f.hvy = reinterpret_cast<const FiltHvy*>(tab + size_t(v.nf) * sizeof(FiltSph));
+                }
                 bool live = t < count;
                 int64_t i = live ? (packed ? bv.idx[base + t] : base + t) : 0;
                 if (live && (i < 0 || i >= b.n)) {   // a stale or corrupt tile list: skip, and say so
@@ -115,18 +186,22 @@ __global__ void __launch_bounds__(P + C, 2) k_dist_batched(BatchView bv, Basket 
                 }
                 st_.pd[0][t] = px; st_.pd[1][t] = py; st_.pd[2][t] = pz;
                 st_.pd[3][t] = qx; st_.pd[4][t] = qy; st_.pd[5][t] = qz;
+                asm volatile("" ::: "memory");   // the FP64 paths of the FP32 pass read the stage again
                 RefineState rs;
                 double best = 0.0;
                 int h = -2, nev = 0;
                 rs.status = 1;
-                if (live) refine_pass1<VOX ? 2 : 0>(v, v.d32, v.d64, px, py, pz, qx, qy, qz, rs, best, h, nev);
+                if (live)
+                    refine_pass1<GLOB ? kTravEither : kTravAll, SEGS>(v, f, v.d64, px, py, pz, qx, qy, qz,
+                                                                [&](int c) { return st_.pd[c][t]; }, rs, best, h, nev);
                 int task = 0, bin = -1;
                 if (rs.status == 0) {
                     task = first_task(rs);
-                    bin = task < 0 ? 0 : kind_bin(v.d64[task].kind);
+                    bin = task_bin<SEGS || GLOB>(rs.tag, task, v.d64);
                 }
                 const int slot = bin >= 0 ? atomicAdd(&st_.cnt[bin], 1) : 0;
                 producer_barrier<P>();
+                if (!GLOB && t == 0 && N.pending) copy_tables(k + 1);   // nobody reads the current tables any more
                 if (bin >= 0) st_.task[bin_start(st_.cnt, bin) + slot] = t | ((task + 1) << kOwnerBits);
                 pad_bins<P>(st_, t);
                 if (rs.status == 0) {
@@ -137,7 +212,7 @@ __global__ void __launch_bounds__(P + C, 2) k_dist_batched(BatchView bv, Basket 
                     }
                     st_.Lm[t] = rs.Lm;
                     st_.dropped[t] = rs.c.dropped;
-                    st_.n[t] = rs.c.n;
+                    st_.n[t] = rs.c.n | rs.tag << 8;
                 } else if (live) {
                     store_result(i, b.n, best, h, px, py, pz, qx, qy, qz, step, hit, nullptr);
                 }
@@ -160,7 +235,7 @@ __global__ void __launch_bounds__(P + C, 2) k_dist_batched(BatchView bv, Basket 
             const int64_t* idx = bv.idx;
             // the outputs are in device memory: each track is stored as it is
             // finished (staging the tile's answers was 4 % slower here)
-            drain_tasks<SEGS, P, false>(v, v.d64, st_, nullptr, [=](int o) { return packed ? idx[base + o] : base + o; },
+            drain_tasks<SEGS, P, false>(v, v.d64, v.m64, st_, nullptr, [=](int o) { return packed ? idx[base + o] : base + o; },
                                         b.n, step, hit);
             __syncwarp();
             if (lane == 0) mbar_arrive(&done[k & 1]);
@@ -190,36 +265,61 @@ cudaError_t launch_wait_selftest(unsigned int* status, uint32_t polls, cudaStrea
     return cudaGetLastError();
 }
 
-template <bool SEGS, bool VOX, int P, int C>
-static int batched_blocks_per_sm() {
-    static int cached = 0;
-    if (cached == 0) {
-        const int smem = 2 * int(sizeof(Stage<P>) + sizeof(TileHdr));
-        int per_sm = 0;
-        if (cudaFuncSetAttribute(k_dist_batched<SEGS, VOX, P, C>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) !=
-                cudaSuccess ||
-            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_dist_batched<SEGS, VOX, P, C>, P + C, smem) !=
-                cudaSuccess ||
-            per_sm < 1) {
-            cudaGetLastError();
-            per_sm = 1;
-        }
-        cached = per_sm;
+// shared memory of one SM and of one block
+static void smem_limits(int* per_sm, int* per_block) {
+    int dev = 0, a = 0, c = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&a, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&c, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess) {
+        cudaGetLastError();
+        a = c = 48 * 1024;
     }
-    return cached;
+    *per_sm = a;
+    *per_block = c;
 }
 
-template <bool SEGS, bool VOX, int P, int C>
+// The table area of a batch: two tables of its largest volume, or what half an
+// SM's shared memory leaves beside the stages (two blocks per SM); 0 when that
+// does not hold the largest volume's.
+template <int P>
+static uint32_t table_room(int max_nf) {
+    const int fixed = 2 * int(sizeof(Stage<P>) + sizeof(TileHdr));
+    int per_sm, per_block;
+    smem_limits(&per_sm, &per_block);
+    const int64_t avail = std::min(per_sm / 2 - 2048, per_block - 1024) - fixed;
+    const int64_t one = int64_t(max_nf) * int64_t(sizeof(FiltSph) + sizeof(FiltHvy));
+    if (one > avail) return 0;
+    return uint32_t(std::max<int64_t>(std::min(2 * one, avail) & ~int64_t(15), 16));
+}
+
+template <bool SEGS, bool GLOB, int P, int C>
 static cudaError_t launch_batched(const BatchView& bv, const Basket& b, double* step, int32_t* hit, int blocks_per_sm,
-                                  cudaStream_t s, int num_sms) {
-    const int smem = 2 * int(sizeof(Stage<P>) + sizeof(TileHdr));
-    const int maxb = batched_blocks_per_sm<SEGS, VOX, P, C>();
-    const int per_sm = (blocks_per_sm <= 0 || blocks_per_sm > maxb) ? maxb : blocks_per_sm;
+                                  uint32_t room, cudaStream_t s, int num_sms) {
+    const int smem = 2 * int(sizeof(Stage<P>) + sizeof(TileHdr)) + (GLOB ? 0 : int(room));
     cudaError_t e =
-        cudaFuncSetAttribute(k_dist_batched<SEGS, VOX, P, C>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        cudaFuncSetAttribute(k_dist_batched<SEGS, GLOB, P, C>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
-    k_dist_batched<SEGS, VOX, P, C><<<per_sm * num_sms, P + C, smem, s>>>(bv, b, step, hit);
+    int maxb = 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&maxb, k_dist_batched<SEGS, GLOB, P, C>, P + C, smem) !=
+            cudaSuccess ||
+        maxb < 1) {
+        cudaGetLastError();
+        maxb = 1;
+    }
+    const int per_sm = (blocks_per_sm <= 0 || blocks_per_sm > maxb) ? maxb : blocks_per_sm;
+    k_dist_batched<SEGS, GLOB, P, C><<<per_sm * num_sms, P + C, smem, s>>>(bv, b, step, hit, room);
     return cudaGetLastError();
+}
+
+template <int P, int C>
+static cudaError_t launch_batched_shape(const BatchView& bv, const Basket& b, double* step, int32_t* hit,
+                                        int blocks_per_sm, cudaStream_t s, int num_sms) {
+    const uint32_t room = bv.vox ? 0 : table_room<P>(bv.max_nf);
+    if (room == 0)
+        return bv.segs ? launch_batched<true, true, P, C>(bv, b, step, hit, blocks_per_sm, room, s, num_sms)
+                       : launch_batched<false, true, P, C>(bv, b, step, hit, blocks_per_sm, room, s, num_sms);
+    return bv.segs ? launch_batched<true, false, P, C>(bv, b, step, hit, blocks_per_sm, room, s, num_sms)
+                   : launch_batched<false, false, P, C>(bv, b, step, hit, blocks_per_sm, room, s, num_sms);
 }
 
 // Two tile shapes, the autotuner's choice per batch: tiles of kTileTracks =
@@ -227,33 +327,23 @@ static cudaError_t launch_batched(const BatchView& bv, const Basket& b, double* 
 cudaError_t launch_dist_batched(const BatchView& bv, const Basket& b, double* step, int32_t* hit, int blocks_per_sm,
                                 int tile_tracks, cudaStream_t s, int num_sms) {
     static_assert(sizeof(TileHdr) % 16 == 0 && sizeof(VolView) % 16 == 0, "16-byte copies");
-    const int code = (bv.segs ? 1 : 0) + (bv.vox ? 2 : 0);
-    if (tile_tracks == kLatProd) {
-        switch (code) {
-            case 0: return launch_batched<false, false, kLatProd, kLatCons>(bv, b, step, hit, blocks_per_sm, s, num_sms);
-            case 1: return launch_batched<true, false, kLatProd, kLatCons>(bv, b, step, hit, blocks_per_sm, s, num_sms);
-            case 2: return launch_batched<false, true, kLatProd, kLatCons>(bv, b, step, hit, blocks_per_sm, s, num_sms);
-            default: return launch_batched<true, true, kLatProd, kLatCons>(bv, b, step, hit, blocks_per_sm, s, num_sms);
-        }
-    }
-    switch (code) {
-        case 0: return launch_batched<false, false, kProd, kCons>(bv, b, step, hit, blocks_per_sm, s, num_sms);
-        case 1: return launch_batched<true, false, kProd, kCons>(bv, b, step, hit, blocks_per_sm, s, num_sms);
-        case 2: return launch_batched<false, true, kProd, kCons>(bv, b, step, hit, blocks_per_sm, s, num_sms);
-        default: return launch_batched<true, true, kProd, kCons>(bv, b, step, hit, blocks_per_sm, s, num_sms);
-    }
+    if (tile_tracks == kLatProd)
+        return launch_batched_shape<kLatProd, kLatCons>(bv, b, step, hit, blocks_per_sm, s, num_sms);
+    return launch_batched_shape<kProd, kCons>(bv, b, step, hit, blocks_per_sm, s, num_sms);
 }
 
 // A small basket in a volume of many daughters takes the split kernel
-// (split_basket()); otherwise a basket of at most two tiles of 256 tracks per
-// resident block (two blocks per SM) takes the latency configuration, larger
-// ones the throughput configuration (toy detector, one call: 65536 tracks
-// 43.8 us instead of 59.1 us, 131072 tracks 66.5 us instead of 78.5 us; from
-// 196608 tracks on the two are equal, and at 2^20 the throughput
-// configuration is 13 % faster).
+// (split_basket()); otherwise volumes of boxes, tubes and cones without a grid
+// take the direct kernel whatever the size (per call against the pipelined
+// kernel: toy detector 19457 tracks 29.1 -> 21.8 us, 2^20 218 -> 140 us), and
+// the others the pipelined one: its latency configuration for a basket of at
+// most two tiles of 256 tracks per resident block (two blocks per SM), else its
+// throughput configuration (measured on the toy detector, when it took this
+// kernel: 65536 tracks 43.8 us instead of 59.1 us, from 196608 tracks on equal).
 cudaError_t launch_dist_refine_stats(const VolView& v, const Basket& b, double* step, int32_t* hit,
                                      double* bpoint, int32_t* nref, cudaStream_t s, int num_sms) {
     if (split_basket(v, b.n, num_sms)) return launch_dist_refine_split(v, b, step, hit, bpoint, nref, s);
+    if (!v.segs && !v.voxelized) return launch_dist_direct(v, b, step, hit, bpoint, nref, s, num_sms);
     if (b.n <= int64_t(4) * num_sms * kLatProd)
         return launch_dist_refine_latency(v, b, step, hit, bpoint, nref, s, num_sms);
     return launch_refine_cfg<kProd, kCons>(v, b, step, hit, bpoint, nref, s, num_sms);

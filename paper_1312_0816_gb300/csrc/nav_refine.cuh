@@ -2,6 +2,7 @@
 // navigator (see nav_refine.cu for the scheme).  Shared by every kernel that
 // navigates with the filter.
 #pragma once
+#include "filter_pass.cuh"
 #include "geo_internal.h"
 #include "nav_common.cuh"
 #include "shapes32.cuh"
@@ -9,78 +10,34 @@
 
 namespace geonav {
 
-// Candidates kept per track: the kCand smallest FP32 bounds, and the least
-// bound evicted.  Two suffice: on every test scene, random and adversarial
-// rays, no track falls back to the full FP64 loop, and the list's registers
-// and insertion work are what the FP32 pass can least afford (toy detector:
-// 0.283 ms with two, 0.298 with three, 0.312 with four, 0.408 with five).
-constexpr int kCand = 2;
-
-struct Cands {
-    float L[kCand];
-    int j[kCand];
-    int n;
-    float dropped;   // smallest bound evicted from the list
-};
-
-__device__ __forceinline__ void cand_insert(Cands& c, float L, int j) {
-    float Lc = L;
-    int jc = j;
-#pragma unroll
-    for (int k = 0; k < kCand; ++k) {
-        if (k < c.n) {
-            if (Lc < c.L[k]) {
-                const float tL = c.L[k];
-                const int tj = c.j[k];
-                c.L[k] = Lc;
-                c.j[k] = jc;
-                Lc = tL;
-                jc = tj;
-            }
-        } else if (k == c.n) {
-            c.L[k] = Lc;
-            c.j[k] = jc;
-            Lc = f_inf();
-        }
-    }
-    if (c.n < kCand) ++c.n;
-    else c.dropped = fminf(c.dropped, Lc);
-}
-
-// lower the FP32 parameter t by its rounding allowance
-__device__ __forceinline__ float lower_bound(float t, float delta, float inv_dn) {
-    return t - (16.f * kEps32f * fabsf(t) + delta * inv_dn);
-}
-
 // FP32 lower bound of one daughter's DistFromOutside (bounding-sphere test,
 // transform in the frame shifted to the closest approach, inflated solid),
-// inserted into the candidate list when it can beat the mother's exit.
-__device__ __forceinline__ void bound_daughter(const ShapeRec32& r, int j, const float* p32, const float* d32,
-                                               float inv_dd, float inv_dn, float Um, Cands& c) {
+// inserted into the candidate list when it can beat the mother's exit.  For
+// lanes that visit the same daughter together.
+__device__ __forceinline__ void bound_daughter(const ShapeRec32& r, int j, const Ray32& ray, float Um, Cands& c) {
     const float4 tb = *reinterpret_cast<const float4*>(r.t);   // t and brad^2
-    const float w0 = p32[0] - tb.x, w1 = p32[1] - tb.y, w2 = p32[2] - tb.z;
-    const float s0 = -fmaf(w0, d32[0], fmaf(w1, d32[1], w2 * d32[2])) * inv_dd;
-    const float q0 = fmaf(s0, d32[0], w0), q1 = fmaf(s0, d32[1], w1), q2 = fmaf(s0, d32[2], w2);
-    const float perp2 = fmaf(q0, q0, fmaf(q1, q1, q2 * q2));
+    float s0, q[3];
+    to_shifted(tb, ray, s0, q);
+    const float perp2 = fmaf(q[0], q[0], fmaf(q[1], q[1], q[2] * q[2]));
     if (perp2 > tb.w) return;
-    const float half = r.brad * inv_dn;
+    const float half = r.brad * ray.inv_dn;
     if (s0 + half < 0.f || s0 - half > Um) return;
     float x[3], u[3];
     if (r.flags & kRec32Identity) {   // warp-uniform: every lane visits solid j together
-        x[0] = q0; x[1] = q1; x[2] = q2;
-        u[0] = d32[0]; u[1] = d32[1]; u[2] = d32[2];
+        x[0] = q[0]; x[1] = q[1]; x[2] = q[2];
+        u[0] = ray.d[0]; u[1] = ray.d[1]; u[2] = ray.d[2];
     } else {
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
-            x[k] = fmaf(r.R[6 + k], q2, fmaf(r.R[3 + k], q1, r.R[k] * q0));
-            u[k] = fmaf(r.R[6 + k], d32[2], fmaf(r.R[3 + k], d32[1], r.R[k] * d32[0]));
+            x[k] = fmaf(r.R[6 + k], q[2], fmaf(r.R[3 + k], q[1], r.R[k] * q[0]));
+            u[k] = fmaf(r.R[6 + k], ray.d[2], fmaf(r.R[3 + k], ray.d[1], r.R[k] * ray.d[0]));
         }
     }
     const float tp = enter32(r, x, u, -s0);
     if (!(tp < f_inf())) return;
-    const float L = lower_bound(s0 + tp, r.delta, inv_dn);
+    const float L = lower_bound(s0 + tp, r.delta, ray.inv_dn);
     if (L > Um) return;
-    cand_insert(c, L, j);
+    cand_put(c, L, j);
 }
 
 // Walk of the uniform grid (3D-DDA) along the FP32 ray from its start to the
@@ -139,6 +96,22 @@ __device__ __forceinline__ void vox_walk32(const VolView& v, const float* p, con
     }
 }
 
+// The daughters listed in the cells the track crosses before the mother's
+// exit (upper bound Um); a daughter met again is skipped (4-entry mailbox,
+// then the candidate list).
+__device__ __forceinline__ void bound_grid(const VolView& v, const Ray32& r, float Um, Cands& c) {
+    int mb0 = -1, mb1 = -1, mb2 = -1, mb3 = -1;
+    vox_walk32(v, r.p, r.d, Um, [&](int j) {
+        if (j == mb0 || j == mb1 || j == mb2 || j == mb3) return;
+        mb3 = mb2; mb2 = mb1; mb1 = mb0; mb0 = j;
+#pragma unroll
+        for (int k = 0; k < kCand; ++k)
+            if (c.L[k] < f_inf() && c.j[k] == j) return;
+        bound_daughter(v.d32[j], j, r, Um, c);
+    });
+    cands_count(c);
+}
+
 // The filter's cold FP64 paths (a direction magnitude outside the FP32
 // range, a start between the mother's shrunk copy and the mother, a bound
 // evicted from the list that could still win), out of line: inlined, their
@@ -161,88 +134,158 @@ static __device__ __noinline__ bool contains64_cold(const ShapeRec64& m, double 
 struct RefineState {
     Cands c;
     float Lm;       // lower bound of the mother's exit
+    int tag;        // the surface the first task is surely decided by (kTagNone: not certain)
     int status;     // 0: refine, 1: result already final (invalid / outside / fallback)
 };
 
-// FP32 pass: bounds of the mother and of every daughter.  When status == 1
-// on return, best/h already hold the final answer.  TRAVERSAL: 0 = every
-// daughter, 1 = the uniform grid, 2 = chosen per volume at run time.
-// (TRAVERSAL 0 only) j_first, j_step: bound daughters j_first, j_first +
-// j_step, ... alone (a share of the volume's daughters).
-template <int TRAVERSAL, bool SEGS = true>
-__device__ __forceinline__ void refine_pass1(const VolView& v, const ShapeRec32* __restrict__ tab32,
-                                             const ShapeRec64* __restrict__ tab64, double px, double py,
-                                             double pz, double qx, double qy, double qz, RefineState& st,
-                                             double& best, int& h, int& nev, int j_first = 0, int j_step = 1) {
+// The first solid to refine: the mother (-1) when its bound comes first or
+// there is no candidate, else candidate 0.
+__device__ __forceinline__ int first_task(const RefineState& st) {
+    return (st.c.n == 0 || st.Lm <= st.c.L[0]) ? -1 : st.c.j[0];
+}
+
+// The mother's exit: the shrunk copy gives "surely inside" and a lower bound,
+// the grown copy an upper bound, and both together the surface the exact exit
+// crosses when that is certain: its exit from the grown copy comes before every
+// other surface's exit from the shrunk one.
+struct MotherExit {
+    float lo, hi;
+    bool in;    // inside the shrunk copy
+    int tag;    // kTagPlane / kTagOuter / kTagInner, a box's kTagAxis + k, kTagNone: not certain
+};
+
+__device__ __forceinline__ MotherExit mother_exit32(const VolView& v, const Ray32& r) {
+    const float *el = v.m32.e, *eh = v.m32u.e, *x = r.p, *u = r.d;
+    MotherExit m;
+    float second = f_inf(), thi = f_inf();
+    m.lo = m.hi = f_inf();
+    m.tag = kTagNone;
+    auto take = [&](float lo, float hi, int tag) {
+        const bool first = lo < m.lo;
+        second = first ? m.lo : fminf(second, lo);
+        m.tag = first ? tag : m.tag;
+        thi = first ? hi : thi;
+        m.lo = fminf(m.lo, lo);
+        m.hi = fminf(m.hi, hi);
+    };
+    auto plane = [&](int k, float hl, float hh, int tag) {
+        if (u[k] != 0.f) take(fdiv(copysignf(hl, u[k]) - x[k], u[k]), fdiv(copysignf(hh, u[k]) - x[k], u[k]), tag);
+    };
+    const int kind = v.m32.kind;
+    if (kind == KBOX) {
+        m.in = fabsf(x[0]) <= el[0] && fabsf(x[1]) <= el[1] && fabsf(x[2]) <= el[2];
+#pragma unroll
+        for (int k = 0; k < 3; ++k) plane(k, el[k], eh[k], kTagAxis + k);
+    } else {
+        const float rho2 = fmaf(x[0], x[0], x[1] * x[1]);
+        const float A0 = fmaf(u[0], u[0], u[1] * u[1]);
+        const float B0 = fmaf(x[0], u[0], x[1] * u[1]);
+        if (kind == KTUBE) {
+            m.in = fabsf(x[2]) <= el[2] && rho2 <= el[1] && (el[3] == 0.f || rho2 >= el[0]);
+            plane(2, el[2], eh[2], kTagPlane);
+            float lo = root_rising32(A0, B0, rho2 - el[1]), hi = root_rising32(A0, B0, rho2 - eh[1]);
+            take(lo >= 0.f ? lo : f_inf(), hi >= 0.f ? hi : f_inf(), kTagOuter);
+            if (el[3] != 0.f) {
+                lo = root_falling32(A0, B0, rho2 - el[0]);
+                hi = eh[3] != 0.f ? root_falling32(A0, B0, rho2 - eh[0]) : f_inf();
+                take(lo >= 0.f ? lo : f_inf(), hi >= 0.f ? hi : f_inf(), kTagInner);
+            }
+        } else {
+            // inside test on the same rounded constants as the roots, so that a
+            // point counted inside never sees a root behind it
+            auto cone = [&](const float* e, int a, float& A, float& B, float& C) {
+                const float r0 = fmaf(e[a + 1], x[2], e[a]), rs = e[a + 1] * u[2];
+                A = fmaf(-rs, rs, A0);
+                B = fmaf(-r0, rs, B0);
+                C = fmaf(-r0, r0, rho2);
+            };
+            float A, B, C, Ch;
+            cone(el, 1, A, B, C);
+            m.in = fabsf(x[2]) <= el[0] && C <= 0.f;
+            plane(2, el[0], eh[0], kTagPlane);
+            float lo = root_rising32(A, B, C);
+            cone(eh, 1, A, B, Ch);
+            float hi = root_rising32(A, B, Ch);
+            take(lo >= 0.f ? lo : f_inf(), hi >= 0.f ? hi : f_inf(), kTagOuter);
+            if (el[5] != 0.f) {
+                cone(el, 3, A, B, C);
+                m.in = m.in && C >= 0.f;
+                lo = root_falling32(A, B, C);
+                cone(eh, 3, A, B, Ch);
+                hi = eh[5] != 0.f ? root_falling32(A, B, Ch) : f_inf();
+                take(lo >= 0.f ? lo : f_inf(), hi >= 0.f ? hi : f_inf(), kTagInner);
+            }
+        }
+    }
+    m.lo = fmaxf(m.lo, 0.f);
+    m.hi = fmaxf(m.hi, 0.f);
+    const float dt = 4.f * v.m32u.delta * r.inv_dn;
+    if (!(m.in && m.lo > dt && fmaf(thi, 1.f + 32.f * kEps32f, dt) < second * (1.f - 32.f * kEps32f))) m.tag = kTagNone;
+    return m;
+}
+
+// Which daughters the FP32 pass bounds: every daughter (filter_daughters),
+// the uniform grid's walk, either one by the volume, or the daughters j_first,
+// j_first + j_step, ... of the volume's own order (a share of them).
+enum : int { kTravAll = 0, kTravGrid = 1, kTravEither = 2, kTravShare = 3 };
+
+// FP32 pass: bounds of the mother and of the daughters.  When status == 1 on
+// return, best/h already hold the final answer.  The FP64 track is taken from
+// `src` (src(k): x, y, z, dx, dy, dz) where the rare FP64 paths need it again, so
+// that a caller that holds it in shared memory need not keep it in registers.
+template <int TRAV, bool SEGS = true, class Src>
+__device__ __forceinline__ void refine_pass1(const VolView& v, const FiltTab& f, const ShapeRec64* __restrict__ tab64,
+                                             double px, double py, double pz, double qx, double qy, double qz, Src src,
+                                             RefineState& st, double& best, int& h, int& nev, int j_first = 0,
+                                             int j_step = 1) {
     nev = 0;
     st.status = 1;
-    st.c.n = 0;
-    st.c.dropped = f_inf();
-#pragma unroll
-    for (int k = 0; k < kCand; ++k) {
-        st.c.L[k] = f_inf();
-        st.c.j[k] = 0;
-    }
+    cands_clear(st.c);
     st.Lm = 0.f;
     if (!valid_track(px, py, pz, qx, qy, qz)) {
         best = d_nan();
         h = -2;
         return;
     }
-    const float p32[3] = {f64_to_f32_trunc(px), f64_to_f32_trunc(py), f64_to_f32_trunc(pz)};
-    const float d32[3] = {f64_to_f32_trunc(qx), f64_to_f32_trunc(qy), f64_to_f32_trunc(qz)};
-    const float dd = fmaf(d32[0], d32[0], fmaf(d32[1], d32[1], d32[2] * d32[2]));
+    Ray32 r;
+    r.p[0] = f64_to_f32_trunc(px); r.p[1] = f64_to_f32_trunc(py); r.p[2] = f64_to_f32_trunc(pz);
+    r.d[0] = f64_to_f32_trunc(qx); r.d[1] = f64_to_f32_trunc(qy); r.d[2] = f64_to_f32_trunc(qz);
+    const float dd = fmaf(r.d[0], r.d[0], fmaf(r.d[1], r.d[1], r.d[2] * r.d[2]));
     if (!(dd > 1e-30f && dd < 1e30f)) {
         // direction magnitude outside the range the FP32 bounds assume
-        const double p[3] = {px, py, pz};
-        if (contains64<SEGS>(v.m64, p)) nav_all64_cold<SEGS>(v.m64, tab64, v.nd, px, py, pz, qx, qy, qz, best, h);
+        const double p[3] = {src(0), src(1), src(2)};
+        if (contains64<SEGS>(v.m64, p))
+            nav_all64_cold<SEGS>(v.m64, tab64, v.nd, p[0], p[1], p[2], src(3), src(4), src(5), best, h);
         else { best = 0.0; h = -2; }
         nev = 1000;
         return;
     }
     const float inv_dd = __frcp_rn(dd);
-    const float inv_dn = rsqrtf(dd) * (1.f + 4.f * kEps32f);
-    // mother: the shrunk copy gives "surely inside" and a lower bound of the
-    // exit, the grown copy an upper bound
-    bool in_shrunk;
-    const float e_lo = exit32(v.m32, p32, d32, in_shrunk);
-    bool inside = in_shrunk;
-    if (!in_shrunk) {
-        inside = contains64_cold<SEGS>(v.m64, px, py, pz);
-    }
-    if (!inside) {
-        best = 0.0;
-        h = -2;
-        return;
-    }
-    st.Lm = in_shrunk ? fmaxf(lower_bound(e_lo, v.m32.delta, inv_dn), 0.f) : 0.f;
-    bool dummy;
-    const float e_hi = exit32(v.m32u, p32, d32, dummy);
-    const float Um = e_hi + 16.f * kEps32f * e_hi + v.m32u.delta * inv_dn;
-    const bool grid = TRAVERSAL == 1 || (TRAVERSAL == 2 && v.voxelized);
-    if (!grid) {
-        for (int j = j_first; j < v.nd; j += j_step) bound_daughter(tab32[j], j, p32, d32, inv_dd, inv_dn, Um, st.c);
-    } else {
-        // only daughters listed in the cells the track crosses before the
-        // mother's exit (upper bound Um); a daughter met again is skipped
-        // (4-entry mailbox, then the candidate list)
-        int mb0 = -1, mb1 = -1, mb2 = -1, mb3 = -1;
-        vox_walk32(v, p32, d32, Um, [&](int j) {
-            if (j == mb0 || j == mb1 || j == mb2 || j == mb3) return;
-            mb3 = mb2; mb2 = mb1; mb1 = mb0; mb0 = j;
+    r.inv_dn = rsqrtf(dd) * (1.f + 4.f * kEps32f);
 #pragma unroll
-            for (int k = 0; k < kCand; ++k)
-                if (k < st.c.n && st.c.j[k] == j) return;
-            bound_daughter(tab32[j], j, p32, d32, inv_dd, inv_dn, Um, st.c);
-        });
+    for (int k = 0; k < 3; ++k) r.e[k] = -r.d[k] * inv_dd;
+    const MotherExit m = mother_exit32(v, r);
+    if (!m.in) {
+        if (!contains64_cold<SEGS>(v.m64, src(0), src(1), src(2))) {
+            best = 0.0;
+            h = -2;
+            return;
+        }
     }
+    st.Lm = m.in ? fmaxf(lower_bound(m.lo, v.m32.delta, r.inv_dn), 0.f) : 0.f;
+    const float Um = m.hi + 16.f * kEps32f * m.hi + v.m32u.delta * r.inv_dn;
+    if (TRAV == kTravShare) {
+        for (int j = j_first; j < v.nd; j += j_step) bound_daughter(v.d32[j], j, r, Um, st.c);
+        cands_count(st.c);
+    } else if (TRAV == kTravGrid || (TRAV == kTravEither && v.voxelized)) {
+        bound_grid(v, r, Um, st.c);
+    } else {
+        filter_daughters(f, r, Um, st.c);
+    }
+    st.tag = first_task(st) < 0 ? (v.m64.kind >= KTUBS ? kTagNone : m.tag) : st.c.j[0] >> kTagShift;
+#pragma unroll
+    for (int k = 0; k < kCand; ++k) st.c.j[k] &= kIdMask;
     st.status = 0;
-}
-
-// The first solid to refine: the mother (-1) when its bound comes first or
-// there is no candidate, else candidate 0.
-__device__ __forceinline__ int first_task(const RefineState& st) {
-    return (st.c.n == 0 || st.Lm <= st.c.L[0]) ? -1 : st.c.j[0];
 }
 
 // FP64 evaluation of one solid for one track (the mother's DistFromInside or
@@ -258,6 +301,73 @@ __device__ __forceinline__ double eval64(const VolView& v, const ShapeRec64* __r
     double x[3], u[3];
     to_local64(r, px, py, pz, qx, qy, qz, x, u);
     return dist_out64<false, SEGS>(r, x, u);
+}
+
+// The FP64 step of solid r to the surface it is surely entered (a daughter) or
+// left (the mother: `exit`) through: that surface's part of dist_out64 /
+// dist_in64 with operations that round alike, so the same bits.  Planes and
+// quadrics, tubes and cones run one code path with one division, so that the
+// lanes of a warp need not be ordered by surface: an FP64 instruction costs a
+// warp 64 cycles of its unit however few lanes take part, and a plane adds no
+// instruction to a quadric's.
+//  * A tube is a cone of slope 0 whose C = rho^2 - R^2 keeps the rounded R^2
+//    (FMA(-1, R^2, rho^2); the other terms of slope 0 vanish exactly).
+//  * The rising root of F = A s^2 + 2 B s + C is the falling root of -F (every
+//    operation of a root commutes with the change of all signs).
+//  * A plane needs one local coordinate; it is formed where a quadric forms its
+//    first.
+__device__ __forceinline__ double surface64(const ShapeRec64& r, int tag, bool exit, double px, double py, double pz,
+                                            double qx, double qy, double qz) {
+    const double* d = r.d;
+    const bool quad = tag == kTagOuter || tag == kTagInner, inner = tag == kTagInner;
+    const int k = quad ? 0 : (tag >= kTagAxis ? tag - kTagAxis : 2);
+    const double w0 = SUB(px, r.t[0]), w1 = SUB(py, r.t[1]), w2 = SUB(pz, r.t[2]);
+    double xk, uk, x1 = w1, u1 = qy, x2 = w2, u2 = qz;
+    if (r.flags & kRec64Identity) {
+        xk = k == 0 ? w0 : (k == 1 ? w1 : w2);
+        uk = k == 0 ? qx : (k == 1 ? qy : qz);
+    } else {
+        xk = FMA(r.R[6 + k], w2, FMA(r.R[3 + k], w1, MUL(r.R[k], w0)));
+        uk = FMA(r.R[6 + k], qz, FMA(r.R[3 + k], qy, MUL(r.R[k], qx)));
+        if (quad) {
+            x1 = FMA(r.R[7], w2, FMA(r.R[4], w1, MUL(r.R[1], w0)));
+            u1 = FMA(r.R[7], qz, FMA(r.R[4], qy, MUL(r.R[1], qx)));
+            x2 = FMA(r.R[8], w2, FMA(r.R[5], w1, MUL(r.R[2], w0)));
+            u2 = FMA(r.R[8], qz, FMA(r.R[5], qy, MUL(r.R[2], qx)));
+        }
+    }
+    double num, den;
+    bool ok = true;
+    if (quad) {
+        const bool tube = r.kind == KTUBE;
+        const double b = tube ? 0.0 : (inner ? d[4] : d[2]);
+        const double rho2 = DOT2(xk, xk, x1, x1);
+        const double r0 = FMA(b, x2, tube ? 1.0 : (inner ? d[3] : d[1])), rs = MUL(b, u2);
+        double A = FMA(-rs, rs, DOT2(uk, uk, u1, u1)), B = FMA(-r0, rs, DOT2(xk, uk, x1, u1));
+        double C = FMA(-r0, tube ? (inner ? d[3] : d[4]) : r0, rho2);
+        if (inner != exit) {   // rising
+            A = -A;
+            B = -B;
+            C = -C;
+        }
+        const double D = FMA(B, B, -MUL(A, C));   // root_falling(A, B, C)
+        const bool real = NONNEG(D);
+        const bool bneg = IS_NEG(B);
+        const double t = ADD(SQRT(real ? D : 1.0), fabs(B));
+        num = bneg ? C : -t;
+        den = bneg ? t : A;
+        ok = real && (bneg || IS_NEG(A));
+    } else {   // the face of axis k ahead (exit) or met first (entry)
+        const double h = r.kind == KBOX ? d[k] : (r.kind == KTUBE ? d[2] : d[0]);
+        const double c = copysign(h, uk);
+        num = SUB(exit ? c : -c, xk);
+        den = uk;
+    }
+    // one division for both kinds of lane (the empty statement keeps the
+    // compiler from moving a copy of it into each branch)
+    asm volatile("" : "+d"(num), "+d"(den));
+    const double s = DIV(ok ? num : 1.0, ok ? den : 1.0);
+    return ok ? s : d_inf();
 }
 
 // The answer of refine_rest() when no further FP64 evaluation can change it
@@ -349,19 +459,6 @@ static __device__ __noinline__ void refine_rest(const VolView& v, const ShapeRec
         nav_all64_cold<SEGS>(v.m64, tab64, v.nd, px, py, pz, qx, qy, qz, best, h);
         nev += 1000;   // marks a fallback in the statistics
     }
-}
-
-// One track, all in this thread (used where no block-level compaction is
-// available).  Same answers as nav_all64 with the mother prologue.
-__device__ __forceinline__ void refine_track(const VolView& v, const ShapeRec32* __restrict__ tab32,
-                                             const ShapeRec64* __restrict__ tab64, double px, double py,
-                                             double pz, double qx, double qy, double qz, double& best, int& h,
-                                             int& nev) {
-    RefineState st;
-    refine_pass1<2>(v, tab32, tab64, px, py, pz, qx, qy, qz, st, best, h, nev);
-    if (st.status) return;
-    const double s1 = eval64(v, tab64, first_task(st), px, py, pz, qx, qy, qz);
-    refine_rest(v, tab64, st, s1, px, py, pz, qx, qy, qz, best, h, nev);
 }
 
 }  // namespace geonav

@@ -63,7 +63,11 @@ __global__ void __launch_bounds__(kSplitWarps * 32, kSplitBlocksPerSm)
         }
         double best = 0.0;
         int h = -2, nev = 0;
-        if (live) refine_pass1<0, SEGS>(v, v.d32, v.d64, px, py, pz, qx, qy, qz, rs, best, h, nev, w, kSplitWarps);
+        if (live) {
+            const double tr[6] = {px, py, pz, qx, qy, qz};
+            refine_pass1<kTravShare, SEGS>(v, FiltTab{}, v.d64, px, py, pz, qx, qy, qz, [&](int k) { return tr[k]; }, rs,
+                                           best, h, nev, w, kSplitWarps);
+        }
 #pragma unroll
         for (int q = 0; q < kCand; ++q) {
             sh.L[w][q][lane] = rs.c.L[q];
@@ -106,9 +110,10 @@ __global__ void __launch_bounds__(kSplitWarps * 32, kSplitBlocksPerSm)
         const int nu = sh.n[u][lane];
 #pragma unroll
         for (int q = 0; q < kCand; ++q)
-            if (q < nu) cand_insert(rs.c, sh.L[u][q][lane], sh.j[u][q][lane]);
+            if (q < nu) cand_put(rs.c, sh.L[u][q][lane], sh.j[u][q][lane]);
         rs.c.dropped = fminf(rs.c.dropped, sh.dropped[u][lane]);
     }
+    cands_count(rs.c);
     const int task = first_task(rs);
     if ((task < 0 ? 0 : kind_bin(v.d64[task].kind)) != w) return;
     const double s_first = eval64<SEGS>(v, v.d64, task, px, py, pz, qx, qy, qz);

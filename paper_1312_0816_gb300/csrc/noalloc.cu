@@ -138,11 +138,12 @@ extern "C" geo_status geo_dist_to_boundary_batched_noalloc(const geo_volume* vol
     bv.segs = 0;
     bv.nvols = n_vols;
     bv.vox = 0;
-    bv.pad_ = 0;
+    bv.max_nf = 0;
     bv.idx = nullptr;   // plain tiles only
     for (int i = 0; i < n_vols; ++i) {
         bv.segs = bv.segs || volume_view(vols[i])->segs;
         bv.vox = bv.vox || volume_view(vols[i])->voxelized;
+        bv.max_nf = std::max(bv.max_nf, volume_view(vols[i])->nf);
     }
     const Basket bk{x, y, z, dx, dy, dz, n_total};
     e = launch_dist_batched(bv, bk, step, hit, 0, kTileTracks, s, sm_count(dev));

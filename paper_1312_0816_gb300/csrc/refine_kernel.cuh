@@ -19,14 +19,15 @@ namespace geonav {
 // instruction every 64 cycles; a dependent FP64 chain takes about 76 cycles
 // per step, and the square roots, divisions and comparisons between them
 // leave gaps, so one warp cannot keep its unit busy and two do better.
-// Measured on the toy detector (2^20 tracks): 12 + 4 warps 0.242 ms, 12 + 2
-// warps at 72 registers 0.257 ms, 11 + 3 0.248, 10 + 4 0.254, 9 + 3 at 80
-// registers 0.264, 8 + 4 0.265; the producers alone (FP64 evaluations
-// skipped) take 0.207 ms and the consumers alone (each track's winner given)
-// 0.160 ms, so the FP32 pass sets the pace.
+// This kernel serves volumes with tube segments or polycones, whose tracks need
+// whole solids of differing kinds in FP64, and volumes with a uniform grid;
+// nav_refine_direct.cu serves the others.  (While it served those too, the toy
+// detector's 2^20 tracks took 0.222 ms with 12 + 4 warps, 0.257 with 12 + 2 at 72
+// registers, 0.248 with 11 + 3, 0.264 with 9 + 3 at 80 registers.)
 //  producers: wait done[k%2] (the stage's previous tile, k-2, finished), FP32
-//             pass of tile k, bin each track's first FP64 task by solid kind
-//             (mother, box, tube, cone) into stage k%2, arrive on full[k%2].
+//             pass of tile k, bin each track's first FP64 task (a sure plane
+//             or quadric, or a whole solid by its kind) into stage k%2, arrive
+//             on full[k%2].
 //  consumers: wait full[k%2], evaluate the binned tasks of tile k in FP64 (a
 //             warp claims chunks of 32 consecutive tasks, all of one kind:
 //             the bins start on multiples of 32) and finish their tracks
@@ -51,6 +52,19 @@ constexpr int kOwnerBits = 9;   // binned task: owner | (solid + 1) << kOwnerBit
 static_assert(kProd <= (1 << kOwnerBits) && kProd % 32 == 0 && kLatProd % 32 == 0 && kLatProd >= 128,
               "task encoding, bin padding");
 
+// FP64 task bins: 0 a plane (a box's axis, an end plane), 1 a quadric, of a
+// solid whose surface the FP32 pass is certain of; 2 to 5 whole solids: the mother, box, tube
+// (and tube segment), cone (and polycone).
+constexpr int kTaskBins = 6;
+__device__ __forceinline__ int kind_bin(int kind) { return kind == KTUBS ? 2 : (kind == KPCON ? 3 : 1 + kind); }
+// KINDS = false: whole solids are rare and share one bin (the all-daughter pass
+// in volumes without segments and polycones).
+template <bool KINDS>
+__device__ __forceinline__ int task_bin(int tag, int task, const ShapeRec64* __restrict__ tab64) {
+    if (tag != kTagNone) return tag == kTagOuter || tag == kTagInner ? 1 : 0;
+    return !KINDS || task < 0 ? 2 : 2 + kind_bin(tab64[task].kind);
+}
+
 template <int P>
 struct Stage {
     double pd[6][P];        // the tile's positions and directions (FP64)
@@ -58,11 +72,11 @@ struct Stage {
     int j[kCand][P];        //   that finishes the track (tracks with an FP64 task)
     float Lm[P];
     float dropped[P];
-    int n[P];               // candidate count
-    int task[P + 128];      // binned tasks: owner | (solid + 1) << kOwnerBits; -1 pads
-    int cnt[4];
+    int n[P];               // candidate count | the first task's surface tag << 8
+    int task[P + 32 * kTaskBins];   // binned tasks: owner | (solid + 1) << kOwnerBits; -1 pads
+    int cnt[kTaskBins];
     int next;               // the next chunk of 32 tasks to claim
-    int pad_[3];
+    int pad_[1];
 };
 
 // The answers of one tile, gathered for stores by consecutive lanes (the
@@ -80,15 +94,16 @@ struct Answers {
 __device__ __forceinline__ int bin_start(const int* cnt, int bin) {
     int start = 0;
 #pragma unroll
-    for (int q = 0; q < 4; ++q)
+    for (int q = 0; q < kTaskBins; ++q)
         if (q < bin) start += (cnt[q] + 31) & ~31;
     return start;
 }
 
-// After the counts are final: thread t < 128 pads bin t / 32 (P >= 128).
+// After the counts are final: thread t < 32 kTaskBins pads bin t / 32 (P >= 192).
 template <int P>
 __device__ __forceinline__ void pad_bins(Stage<P>& st, int t) {
-    if (t < 128) {
+    static_assert(P >= 32 * kTaskBins, "one thread per pad slot");
+    if (t < 32 * kTaskBins) {
         const int b = t >> 5, c = st.cnt[b];
         if ((t & 31) < ((c + 31) & ~31) - c) st.task[bin_start(st.cnt, b) + c + (t & 31)] = -1;
     }
@@ -119,10 +134,6 @@ __device__ __forceinline__ void mbar_wait_bounded(uint64_t* bar, uint32_t parity
     healthy = false;
 }
 
-// FP64 task bins: 0 the mother, then box, tube (and tube segment), cone (and
-// polycone)
-__device__ __forceinline__ int kind_bin(int kind) { return kind == KTUBS ? 2 : (kind == KPCON ? 3 : 1 + kind); }
-
 // A consumer's whole share of one track: the FP64 value of its first task
 // jj, then the refinement's end (nearly always refine_fast: no other bound
 // can win or tie).  The answer goes to the tile's answer buffer (STAGED),
@@ -132,13 +143,20 @@ __device__ __forceinline__ int kind_bin(int kind) { return kind == KTUBS ? 2 : (
 // link pay for); or it is stored right away to index(o).
 template <bool SEGS, int P, bool STAGED, typename Index>
 __device__ __forceinline__ void finish_track(const VolView& v, const ShapeRec64* __restrict__ tab64,
-                                             const Stage<P>& st, Answers<P>* ans, int o, int jj, Index index,
+                                             const ShapeRec64& m64, const Stage<P>& st, Answers<P>* ans, int o, int jj, Index index,
                                              int64_t n, double* __restrict__ step, int32_t* __restrict__ hit) {
-    const double s_first =
-        eval64<SEGS>(v, tab64, jj, st.pd[0][o], st.pd[1][o], st.pd[2][o], st.pd[3][o], st.pd[4][o], st.pd[5][o]);
+    const int nt = st.n[o], tag = nt >> 8;
+    double s_first;
+    if (tag == kTagNone) {
+        s_first =
+            eval64<SEGS>(v, tab64, jj, st.pd[0][o], st.pd[1][o], st.pd[2][o], st.pd[3][o], st.pd[4][o], st.pd[5][o]);
+    } else {
+        s_first = surface64(jj < 0 ? m64 : tab64[jj], tag, jj < 0, st.pd[0][o], st.pd[1][o], st.pd[2][o], st.pd[3][o],
+                            st.pd[4][o], st.pd[5][o]);
+    }
     RefineState rs;
     rs.status = 0;
-    rs.c.n = st.n[o];
+    rs.c.n = nt & 255;
 #pragma unroll
     for (int q = 0; q < kCand; ++q) {
         rs.c.L[q] = st.L[q][o];
@@ -183,10 +201,11 @@ __device__ __forceinline__ void store_tile(const Stage<P>& st, const Answers<P>&
 // bin-aligned chunk, so one solid kind) from the stage's counter until none
 // is left, and finishes their tracks.  Every lane of the warp takes part.
 template <bool SEGS, int P, bool STAGED, typename Index>
-__device__ __forceinline__ void drain_tasks(const VolView& v, const ShapeRec64* __restrict__ tab64, Stage<P>& st,
+__device__ __forceinline__ void drain_tasks(const VolView& v, const ShapeRec64* __restrict__ tab64,
+                                            const ShapeRec64& m64, Stage<P>& st,
                                             Answers<P>* ans, Index index, int64_t n, double* __restrict__ step,
                                             int32_t* __restrict__ hit) {
-    const int total = bin_start(st.cnt, 4);   // a multiple of 32
+    const int total = bin_start(st.cnt, kTaskBins);   // a multiple of 32
     const int lane = threadIdx.x & 31;
     for (;;) {
         int q0 = 0;
@@ -196,7 +215,7 @@ __device__ __forceinline__ void drain_tasks(const VolView& v, const ShapeRec64* 
         const int e = st.task[q0 + lane];
         if (e >= 0) {
             const int o = e & ((1 << kOwnerBits) - 1), jj = (e >> kOwnerBits) - 1;
-            finish_track<SEGS, P, STAGED>(v, tab64, st, ans, o, jj, index, n, step, hit);
+            finish_track<SEGS, P, STAGED>(v, tab64, m64, st, ans, o, jj, index, n, step, hit);
         }
     }
 }
@@ -206,8 +225,8 @@ __device__ __forceinline__ void producer_barrier() { asm volatile("bar.sync 1, %
 template <int C>
 __device__ __forceinline__ void consumer_barrier() { asm volatile("bar.sync 2, %0;" ::"r"(C) : "memory"); }
 
-template <int P, int C, bool SMEM, int TRAV, bool SEGS>
-__global__ void __launch_bounds__(P + C, 2) k_dist_refine(VolView v, Basket b, double* __restrict__ step,
+template <int P, int C, int SMEM, int TRAV, bool SEGS>
+__global__ void __launch_bounds__(P + C, 2) k_dist_refine(const __grid_constant__ VolView v, Basket b, double* __restrict__ step,
                                                              int32_t* __restrict__ hit,
                                                              double* __restrict__ bpoint,
                                                              int32_t* __restrict__ nref) {
@@ -218,17 +237,23 @@ __global__ void __launch_bounds__(P + C, 2) k_dist_refine(VolView v, Basket b, d
     Stage<P>* S = reinterpret_cast<Stage<P>*>(smem_raw);
     Answers<P>* A = reinterpret_cast<Answers<P>*>(smem_raw + 2 * sizeof(Stage<P>));
     unsigned char* tables = smem_raw + 2 * (sizeof(Stage<P>) + sizeof(Answers<P>));
-    const ShapeRec32* tab32 = v.d32;
+    FiltTab f = {v.fsph, v.fhvy, v.nq1, v.nq, v.nf};
     const ShapeRec64* tab64 = v.d64;
     if (SMEM) {
-        const uint32_t b32 = uint32_t(v.nd) * sizeof(ShapeRec32);
-        if (!stage_tables(tables, v.d32, b32, tables + b32, v.d64, uint32_t(v.nd) * sizeof(ShapeRec64), &bar,
-                          v.status))
+        // the filter's two tables (consecutive in device memory), then the FP64 records
+        const uint32_t bf = uint32_t(v.nf) * uint32_t(sizeof(FiltSph) + sizeof(FiltHvy));
+        if (!stage_tables(tables, v.fsph, bf, tables + bf, v.d64, SMEM == 2 ? uint32_t(v.nd) * uint32_t(sizeof(ShapeRec64)) : 0,
+                          &bar, v.status))
             return;
-        tab32 = reinterpret_cast<const ShapeRec32*>(tables);
-        tab64 = reinterpret_cast<const ShapeRec64*>(tables + b32);
+        f.sph = reinterpret_cast<const FiltSph*>(tables);
+        f.hvy = reinterpret_cast<const FiltHvy*>(tables + size_t(v.nf) * sizeof(FiltSph));
+        if (SMEM == 2) tab64 = reinterpret_cast<const ShapeRec64*>(tables + bf);
     }
     const int t = threadIdx.x;
+    // the mother's FP64 record beside the daughters', for tasks of either kind
+    __shared__ ShapeRec64 m64;
+    if (t < int(sizeof(ShapeRec64) / sizeof(double)))
+        reinterpret_cast<double*>(&m64)[t] = reinterpret_cast<const double*>(&v.m64)[t];
     if (t == 0) {
         mbar_init(&full[0], P / 32);
         mbar_init(&full[1], P / 32);
@@ -256,18 +281,21 @@ __global__ void __launch_bounds__(P + C, 2) k_dist_refine(VolView v, Basket b, d
             }
             st_.pd[0][t] = px; st_.pd[1][t] = py; st_.pd[2][t] = pz;
             st_.pd[3][t] = qx; st_.pd[4][t] = qy; st_.pd[5][t] = qz;
+            asm volatile("" ::: "memory");   // the FP64 paths of the FP32 pass read the stage again
             RefineState rs;
             double best = 0.0;
             int h = -2, nev = 0;
             rs.status = 1;
-            if (live) refine_pass1<TRAV, SEGS>(v, tab32, tab64, px, py, pz, qx, qy, qz, rs, best, h, nev);
+            if (live)
+                refine_pass1<TRAV, SEGS>(v, f, tab64, px, py, pz, qx, qy, qz, [&](int c) { return st_.pd[c][t]; }, rs, best,
+                                         h, nev);
             int task = 0, bin = -1;
             if (rs.status == 0) {
                 task = first_task(rs);
-                bin = task < 0 ? 0 : kind_bin(tab64[task].kind);
+                bin = task_bin<SEGS || TRAV == kTravGrid>(rs.tag, task, tab64);
             }
-            if (t < 4) st_.cnt[t] = 0;
-            if (t == 4) st_.next = 0;
+            if (t < kTaskBins) st_.cnt[t] = 0;
+            if (t == kTaskBins) st_.next = 0;
             producer_barrier<P>();
             const int slot = bin >= 0 ? atomicAdd(&st_.cnt[bin], 1) : 0;
             producer_barrier<P>();
@@ -283,7 +311,7 @@ __global__ void __launch_bounds__(P + C, 2) k_dist_refine(VolView v, Basket b, d
                 }
                 st_.Lm[t] = rs.Lm;
                 st_.dropped[t] = rs.c.dropped;
-                st_.n[t] = rs.c.n;
+                st_.n[t] = rs.c.n | rs.tag << 8;
             } else {   // a final answer, or no track
                 A[k & 1].best[t] = best;
                 A[k & 1].h[t] = live ? h : kNoStore;
@@ -300,7 +328,7 @@ __global__ void __launch_bounds__(P + C, 2) k_dist_refine(VolView v, Basket b, d
             const int64_t base = (int64_t(blockIdx.x) + int64_t(k) * gridDim.x) * P;
             const bool ok = __all_sync(0xffffffffu, healthy);   // a stage never filled is not read
             auto index = [base](int o) { return base + o; };
-            if (ok) drain_tasks<SEGS, P, true>(v, tab64, S[k & 1], &A[k & 1], index, b.n, step, hit);
+            if (ok) drain_tasks<SEGS, P, true>(v, tab64, m64, S[k & 1], &A[k & 1], index, b.n, step, hit);
             consumer_barrier<C>();   // every answer of the tile is in its answer buffer
             if (ok) store_tile<P, C>(S[k & 1], A[k & 1], c, index, b.n, step, hit, bpoint, nref);
             __syncwarp();
@@ -336,31 +364,26 @@ template <int P, int C>
 static cudaError_t launch_refine_cfg(const VolView& v, const Basket& b, double* step, int32_t* hit, double* bpoint,
                                      int32_t* nref, cudaStream_t s, int num_sms) {
     static_assert(sizeof(Stage<P>) % 16 == 0 && sizeof(Answers<P>) % 16 == 0, "the tables stay 16-byte aligned");
-    const int smem = 2 * int(sizeof(Stage<P>) + sizeof(Answers<P>)) +
-                     (v.smem_refine ? v.nd * int(sizeof(ShapeRec64) + sizeof(ShapeRec32)) : 0);
+    const int stages = 2 * int(sizeof(Stage<P>) + sizeof(Answers<P>));
+    const int filt = v.nf * int(sizeof(FiltSph) + sizeof(FiltHvy));
     if (v.voxelized) {
         // the grid walk needs registers: 12 + 2 warps at 72 registers beat
         // 12 + 4 at 64 (7.0 against 7.4 ms for 2^24 tracks in 512 daughters)
         constexpr int CV = P == kProd ? kVoxCons : C;
-        const int smem_v = 2 * int(sizeof(Stage<P>) + sizeof(Answers<P>));
         if (v.segs)
-            return launch_refine<P, CV>(k_dist_refine<P, CV, false, 1, true>, smem_v, v, b, step, hit, bpoint, nref,
+            return launch_refine<P, CV>(k_dist_refine<P, CV, 0, kTravGrid, true>, stages, v, b, step, hit, bpoint, nref,
                                         s, num_sms);
-        return launch_refine<P, CV>(k_dist_refine<P, CV, false, 1, false>, smem_v, v, b, step, hit, bpoint, nref, s,
+        return launch_refine<P, CV>(k_dist_refine<P, CV, 0, kTravGrid, false>, stages, v, b, step, hit, bpoint, nref, s,
                                     num_sms);
     }
-    if (v.smem_refine) {
-        if (v.segs)
-            return launch_refine<P, C>(k_dist_refine<P, C, true, 0, true>, smem, v, b, step, hit, bpoint, nref, s,
-                                       num_sms);
-        return launch_refine<P, C>(k_dist_refine<P, C, true, 0, false>, smem, v, b, step, hit, bpoint, nref, s,
+    // volumes without segments and polycones take the direct kernel
+    if (v.smem_refine == 2)
+        return launch_refine<P, C>(k_dist_refine<P, C, 2, kTravAll, true>, stages + filt + v.nd * int(sizeof(ShapeRec64)), v,
+                                   b, step, hit, bpoint, nref, s, num_sms);
+    if (v.smem_refine == 1)
+        return launch_refine<P, C>(k_dist_refine<P, C, 1, kTravAll, true>, stages + filt, v, b, step, hit, bpoint, nref, s,
                                    num_sms);
-    }
-    if (v.segs)
-        return launch_refine<P, C>(k_dist_refine<P, C, false, 0, true>, smem, v, b, step, hit, bpoint, nref, s,
-                                   num_sms);
-    return launch_refine<P, C>(k_dist_refine<P, C, false, 0, false>, smem, v, b, step, hit, bpoint, nref, s,
-                               num_sms);
+    return launch_refine<P, C>(k_dist_refine<P, C, 0, kTravAll, true>, stages, v, b, step, hit, bpoint, nref, s, num_sms);
 }
 
 }  // namespace geonav

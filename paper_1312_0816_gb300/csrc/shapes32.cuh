@@ -32,21 +32,41 @@ constexpr float kEps32f = 5.9604645e-08f;
 
 __device__ __forceinline__ float f_inf() { return __int_as_float(0x7f800000); }
 
-// Approximate division and square root (a few ulp): the filter's margins
-// (16 eps32 |t| relative, plus the inflation delta) absorb them.
-__device__ __forceinline__ float fdiv(float a, float b) { return __fdividef(a, b); }
-__device__ __forceinline__ float fsqrt(float a) { return a > 0.f ? a * rsqrtf(a) : 0.f; }
+// Approximate division and square roots (a few ulp): the filter's margins
+// (16 eps32 |t| relative, plus the inflation delta) absorb them.  The forms that
+// flush subnormal operands to zero are one instruction each (the others test
+// and rescale their operand); a subnormal divisor then gives an infinity
+// and a subnormal square root 0, both within the margins: the filter's
+// lengths are at least delta and its directions at least 1e-15 long.
+__device__ __forceinline__ float frcp(float a) {
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(a));
+    return r;
+}
+__device__ __forceinline__ float frsqrt(float a) {
+    float r;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(a));
+    return r;
+}
+__device__ __forceinline__ float fsqrt(float a) {   // a >= 0
+    float r;
+    asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(a));
+    return r;
+}
+__device__ __forceinline__ float fdiv(float a, float b) { return a * frcp(b); }
 
-// FP64 -> FP32 by truncating the significand (integer operations only, so the
-// FP64 pipe stays free).  Relative error below 2^-23, which the inflation
-// covers.  Magnitudes outside the normal FP32 range take the ordinary
-// conversion.
+// FP64 -> FP32 by truncating the significand (integer operations only: a
+// conversion instruction would hold the FP64 unit).  Relative error below
+// 2^-23, which the inflation covers.  Magnitudes below the normal FP32 range
+// give zero, above it infinity.
 __device__ __forceinline__ float f64_to_f32_trunc(double x) {
     const unsigned hi = unsigned(__double2hiint(x)), lo = unsigned(__double2loint(x));
-    const int e = int((hi >> 20) & 0x7ffu) - 1023;
-    if (e < -126 || e > 127) return float(x);
-    const unsigned bits = (hi & 0x80000000u) | (unsigned(e + 127) << 23) | ((hi & 0xfffffu) << 3) | (lo >> 29);
-    return __uint_as_float(bits);
+    const unsigned m = hi & 0x7fffffffu;
+    // the magnitude's top 31 bits, the exponent's bias changed from 1023 to 127
+    // (modulo 2^32: -(896 << 23))
+    unsigned f = __funnelshift_l(lo, m, 3) + 0x40000000u;
+    f = m < 0x38100000u ? 0u : (m >= 0x47f00000u ? 0x7f800000u : f);
+    return __uint_as_float(f | (hi & 0x80000000u));
 }
 
 // An FP32 value >= x for x >= 0 (x itself when exactly representable or one
@@ -68,7 +88,7 @@ __device__ __forceinline__ float box_enter32(const float* h, const float* x, con
         if (u[k] == 0.f) {
             if (fabsf(x[k]) > h[k] + tol) return f_inf();
         } else {
-            const float inv = __fdividef(1.f, u[k]);
+            const float inv = frcp(u[k]);
             const float a = (-h[k] - x[k]) * inv, b = (h[k] - x[k]) * inv;
             tn = fmaxf(tn, fminf(a, b));
             tf = fminf(tf, fmaxf(a, b));
@@ -292,8 +312,8 @@ __device__ __forceinline__ float safety_out_lb32(const ShapeRec32& r, const floa
             s = fsqrt(fmaf(dr, dr, dz * dz));
         } else {
             s = az - e[0];
-            s = fmaxf(s, (rho - fmaf(e[2], x[2], e[1])) * rsqrtf(fmaf(e[2], e[2], 1.f)));
-            if (e[5] != 0.f) s = fmaxf(s, (fmaf(e[4], x[2], e[3]) - rho) * rsqrtf(fmaf(e[4], e[4], 1.f)));
+            s = fmaxf(s, (rho - fmaf(e[2], x[2], e[1])) * frsqrt(fmaf(e[2], e[2], 1.f)));
+            if (e[5] != 0.f) s = fmaxf(s, (fmaf(e[4], x[2], e[3]) - rho) * frsqrt(fmaf(e[4], e[4], 1.f)));
             s = fmaxf(s, 0.f);
         }
     }
@@ -319,8 +339,8 @@ __device__ __forceinline__ float safety_in_lb32(const ShapeRec32& r, const float
             if (e[3] != 0.f) s = fminf(s, rho - fsqrt(e[0]));
         } else {
             s = e[0] - az;
-            s = fminf(s, (fmaf(e[2], x[2], e[1]) - rho) * rsqrtf(fmaf(e[2], e[2], 1.f)));
-            if (e[5] != 0.f) s = fminf(s, (rho - fmaf(e[4], x[2], e[3])) * rsqrtf(fmaf(e[4], e[4], 1.f)));
+            s = fminf(s, (fmaf(e[2], x[2], e[1]) - rho) * frsqrt(fmaf(e[2], e[2], 1.f)));
+            if (e[5] != 0.f) s = fminf(s, (rho - fmaf(e[4], x[2], e[3])) * frsqrt(fmaf(e[4], e[4], 1.f)));
         }
     }
     return fmaxf(s, 0.f) * (1.f - kSafMargin);

@@ -205,42 +205,43 @@ static __device__ __noinline__ void world_nav64(const VolView& v, const double* 
 static __device__ __forceinline__ void world_pass1(const VolView& v, const double* x, const double* u, int skip,
                                                    bool entered, RefineState& st, double& best, int& h) {
     st.status = 1;
-    st.c.n = 0;
-    st.c.dropped = f_inf();
-#pragma unroll
-    for (int k = 0; k < kCand; ++k) {
-        st.c.L[k] = f_inf();
-        st.c.j[k] = 0;
-    }
+    cands_clear(st.c);
     st.Lm = 0.f;
     if (!valid_track(x[0], x[1], x[2], u[0], u[1], u[2])) {
         best = d_nan();
         h = -2;
         return;
     }
-    const float p32[3] = {f64_to_f32_trunc(x[0]), f64_to_f32_trunc(x[1]), f64_to_f32_trunc(x[2])};
-    const float d32[3] = {f64_to_f32_trunc(u[0]), f64_to_f32_trunc(u[1]), f64_to_f32_trunc(u[2])};
-    const float dd = fmaf(d32[0], d32[0], fmaf(d32[1], d32[1], d32[2] * d32[2]));
+    Ray32 r;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        r.p[k] = f64_to_f32_trunc(x[k]);
+        r.d[k] = f64_to_f32_trunc(u[k]);
+    }
+    const float dd = fmaf(r.d[0], r.d[0], fmaf(r.d[1], r.d[1], r.d[2] * r.d[2]));
     if (!(dd > 1e-30f && dd < 1e30f)) {
         world_nav64(v, x, u, skip, entered, best, h);
         return;
     }
     const float inv_dd = __frcp_rn(dd);
-    const float inv_dn = rsqrtf(dd) * (1.f + 4.f * kEps32f);
+    r.inv_dn = rsqrtf(dd) * (1.f + 4.f * kEps32f);
+#pragma unroll
+    for (int k = 0; k < 3; ++k) r.e[k] = -r.d[k] * inv_dd;
     bool in_shrunk;
-    const float e_lo = exit32(v.m32, p32, d32, in_shrunk);
+    const float e_lo = exit32(v.m32, r.p, r.d, in_shrunk);
     const bool inside = in_shrunk || entered || contains64_cold<true>(v.m64, x[0], x[1], x[2]);
     if (!inside) {
         best = 0.0;
         h = -2;
         return;
     }
-    st.Lm = in_shrunk ? fmaxf(lower_bound(e_lo, v.m32.delta, inv_dn), 0.f) : 0.f;
+    st.Lm = in_shrunk ? fmaxf(lower_bound(e_lo, v.m32.delta, r.inv_dn), 0.f) : 0.f;
     bool dummy;
-    const float e_hi = exit32(v.m32u, p32, d32, dummy);
-    const float Um = e_hi + 16.f * kEps32f * e_hi + v.m32u.delta * inv_dn;
+    const float e_hi = exit32(v.m32u, r.p, r.d, dummy);
+    const float Um = e_hi + 16.f * kEps32f * e_hi + v.m32u.delta * r.inv_dn;
     for (int j = 0; j < v.nd; ++j)
-        if (j != skip) bound_daughter(v.d32[j], j, p32, d32, inv_dd, inv_dn, Um, st.c);
+        if (j != skip) bound_daughter(v.d32[j], j, r, Um, st.c);
+    cands_count(st.c);
     st.status = 0;
 }
 

@@ -1,0 +1,112 @@
+"""The filter's tables and the surfaces it is certain of: volumes whose numbers
+of unrotated quadrics, rotated quadrics and boxes sit at the edges of the
+32-entry chunks and of the pairs, staged in shared memory or read from global
+memory, for one basket and for a batch.  The answers are the plain FP64
+kernel's bits (GEO_FP64 evaluates every solid whole, without the filter)."""
+import numpy as np
+import pytest
+
+from paper_1312_0816_gb300 import scenes
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def g():
+    import paper_1312_0816_gb300 as pkg
+
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    pkg.load()
+    return pkg
+
+
+def filter_scene(n1, n2, n3, mother, seed):
+    """n1 unrotated tubes and cones (nested shells about two axes: shells of no
+    thickness, holes far narrower than the filter's inflation, cones ending
+    in an apex), n2 rotated ones, n3 boxes; they may overlap."""
+    rng = np.random.default_rng(seed)
+    eye = np.eye(3).reshape(9)
+    rows = []
+    for k in range(n1):
+        axis = ((0.0, 0.0), (0.0, 0.0), (60.0, -40.0))[k % 3]
+        r = 10.0 + 300.0 * k / max(n1, 1)
+        t = (axis[0], axis[1], rng.uniform(-200.0, 200.0))
+        if k % 4 == 1:
+            r1, r2 = r, r + rng.uniform(-8.0, 30.0)
+            rows.append((scenes.CONE, (rng.uniform(5.0, 150.0), r1 * 0.7, r1, r2 * 0.6, r2), eye, t))
+        else:
+            rmin = (r, r * 0.9, 1e-6, 0.0)[k % 7 % 4]
+            rows.append((scenes.TUBE, (rmin, r, rng.uniform(5.0, 300.0)), eye, t))
+    for k in range(n2):
+        t = rng.uniform(-350.0, 350.0, 3)
+        if k % 2:
+            rows.append((scenes.CONE, (rng.uniform(5.0, 40.0), 0.0, 0.0 if k % 6 == 1 else 10.0, 2.0, 25.0),
+                         scenes.haar_rotation(rng), t))
+        else:
+            rows.append((scenes.TUBE, (0.0 if k % 4 else 6.0, rng.uniform(8.0, 30.0), rng.uniform(5.0, 40.0)),
+                         scenes.haar_rotation(rng), t))
+    for k in range(n3):
+        rows.append((scenes.BOX, rng.uniform(3.0, 40.0, 3), eye if k % 3 == 0 else scenes.haar_rotation(rng),
+                     rng.uniform(-350.0, 350.0, 3)))
+    order = rng.permutation(len(rows))
+    mk, mp = (scenes.BOX, (400.0, 400.0, 400.0)) if mother == "box" else (scenes.TUBE, (0.0, 420.0, 400.0))
+    return scenes._scene(f"filter{n1}_{n2}_{n3}", mk, mp, [rows[i] for i in order])
+
+
+def tracks(sc, n, seed):
+    """Points in the mother (inside daughters and outside the mother too), isotropic
+    directions; some along an axis, some in a coordinate plane, some of
+    other lengths."""
+    rng = np.random.default_rng(seed)
+    p = rng.uniform(-405.0, 405.0, (3, n))
+    d = np.stack(scenes.isotropic(rng, n))
+    m = n // 16
+    for k in range(3):
+        d[k, k * m:(k + 1) * m] = 0.0                       # in a coordinate plane
+        d[:, (3 + k) * m:(4 + k) * m] = 0.0
+        d[k, (3 + k) * m:(4 + k) * m] = rng.choice([-1.0, 1.0], m)   # along an axis
+    d[:, 7 * m:8 * m] *= 1e-3
+    d[:2, 8 * m:9 * m] *= 1e-7                              # nearly along z
+    d[2, 9 * m:10 * m] *= 1e-7                              # nearly across it
+    return [torch.from_numpy(np.ascontiguousarray(a)).cuda() for a in (*p, *d)]
+
+
+COUNTS = [(0, 0, 1), (1, 0, 0), (1, 1, 1), (2, 1, 0), (31, 2, 5), (32, 0, 0), (33, 0, 1), (34, 31, 1), (1, 32, 32),
+          (2, 65, 33), (40, 40, 19), (0, 150, 130)]
+
+
+@pytest.mark.parametrize("mother", ["box", "tube"])
+@pytest.mark.parametrize("counts", COUNTS)
+def test_filter_equals_fp64_bitwise(g, counts, mother):
+    sc = filter_scene(*counts, mother, seed=sum(counts) + 7)
+    vol = g.geo_build_volume(sc)
+    for n in (257, 70001):   # n = 257: the small-basket kernels; 70001: the direct or the pipelined one
+        t = tracks(sc, n, n)
+        s0, h0 = g.geo_dist_to_boundary(vol, *t, mode=g.GEO_FP64)
+        s1, h1 = g.geo_dist_to_boundary(vol, *t, mode=g.GEO_FP32_REFINE)
+        assert torch.equal(h0, h1)
+        assert torch.equal(s0.view(torch.int64), s1.view(torch.int64))
+    assert len(torch.unique(h1)) > 2
+    assert g.geo_check_device_status(vol) == 0
+
+
+@pytest.mark.parametrize("which", [(1, 4, 10), (0, 11, 9, 10)])
+def test_batched_filter_equals_fp64_bitwise(g, which):
+    """Volumes whose tables fit side by side in the batch's table area, and
+    volumes that only fit one after the other or not at all."""
+    vols = [g.geo_build_volume(filter_scene(*COUNTS[w], "box", seed=100 + w)) for w in which]
+    n = 60013
+    t = tracks(None, n, 5)
+    cuts = [0, 17, 400, 20000, 20384, 45000, n]
+    rows = [(k % len(vols), a, b - a) for k, (a, b) in enumerate(zip(cuts, cuts[1:]))]
+    for tile in (384, 256):
+        batch = g.geo_build_batch(vols, rows, tile_tracks=tile)
+        s, h = g.geo_dist_to_boundary_batched(batch, *t)
+        for v, a, c in rows:
+            s0, h0 = g.geo_dist_to_boundary(vols[v], *[x[a:a + c].contiguous() for x in t], mode=g.GEO_FP64)
+            assert torch.equal(h[a:a + c], h0)
+            assert torch.equal(s[a:a + c].view(torch.int64), s0.view(torch.int64))
+    for v in vols:
+        assert g.geo_check_device_status(v) == 0
