@@ -57,6 +57,12 @@ namespace geonav {
 // and insertion work are what the FP32 pass can least afford.
 constexpr int kCand = 2;
 
+// A candidate is its daughter's index and, from bit kTagShift on, the surface it
+// is surely entered through (kTagNone: not certain).
+constexpr int kTagShift = 24;
+constexpr int kIdMask = (1 << kTagShift) - 1;
+enum : int { kTagNone = 0, kTagPlane = 1, kTagOuter = 2, kTagInner = 3, kTagAxis = 4 };   // kTagAxis + k: a box's axis k
+
 struct Cands {
     float L[kCand];
     int j[kCand];
@@ -72,6 +78,11 @@ __device__ __forceinline__ void cands_clear(Cands& c) {
     }
     c.n = 0;
     c.dropped = f_inf();
+}
+
+// whether the list holds daughter j
+__device__ __forceinline__ bool cand_holds(const Cands& c, int j) {
+    return (c.L[0] < f_inf() && (c.j[0] & kIdMask) == j) || (c.L[1] < f_inf() && (c.j[1] & kIdMask) == j);
 }
 
 // Insertion of a finite bound.  An empty slot holds +inf, so no count is needed: the
@@ -124,19 +135,13 @@ __device__ __forceinline__ void rotate_in(const float4 h1, const float4 h2, cons
 
 __device__ __forceinline__ const float4* hvy_words(const FiltHvy* h) { return reinterpret_cast<const float4*>(h); }
 
-// A candidate is its daughter's index and, from bit kTagShift on, the surface it
-// is surely entered through (kTagNone: not certain).
-constexpr int kTagShift = 24;
-constexpr int kIdMask = (1 << kTagShift) - 1;
-enum : int { kTagNone = 0, kTagPlane = 1, kTagOuter = 2, kTagInner = 3, kTagAxis = 4 };   // kTagAxis + k: a box's axis k
-
 // Bound of the entry into quadric solid h (tube or cone; cone_enter32's),
 // inserted into the list when it is within Um.  Returns the latest parameter of
 // a certain entry, else +inf.
 __device__ __forceinline__ float bound_quad(const FiltHvy* h, const Ray32& r, float Um, Cands& c) {
     const float4* H = hvy_words(h);
     const float4 h0 = H[0], h3 = H[3], h4 = H[4], h5 = H[5], h6 = H[6];
-    const float tol = h0.w;
+    const float tol = h6.z;
     const int flags = __float_as_int(h3.y);
     float s0, x[3], u[3];
     to_shifted(h0, r, s0, x);
@@ -171,10 +176,10 @@ __device__ __forceinline__ float bound_quad(const FiltHvy* h, const Ray32& r, fl
         const float hi2 = up ? h5.z : h5.y, lo2 = up ? h6.x : h5.w;
         best = fabsf(sz) > dz && sz * u[2] < 0.f && r2 <= hi2 && r2 >= lo2 ? fmaxf(tz, tmin) : f_inf();
         e = tol4 * fabsf(inv);
-        const float rh = fsqrt(r2), slack = fmaf(e, fsqrt(A0), tol4 + tol4);
+        const float rh = fsqrt(r2), slack = fmaf(e, fsqrt(A0), tol4);
         sure = rh + slack <= fmaf(bo, ze, ao) && (!hole || rh - slack >= fmaf(bi, ze, ai));
     }
-    const float zs = dz - (tol4 + tol4);
+    const float zs = dz - tol4;
     auto quadric = [&](float a, float b, bool rising, int its) {
         const float r0 = fmaf(b, x[2], a), rs = b * u[2];
         const float A = fmaf(-rs, rs, A0), B = fmaf(-r0, rs, B0), C = fmaf(-r0, r0, rho2);
@@ -215,7 +220,7 @@ __device__ __forceinline__ float bound_quad(const FiltHvy* h, const Ray32& r, fl
 __device__ __forceinline__ float bound_box(const FiltHvy* h, const Ray32& r, float Um, Cands& c) {
     const float4* H = hvy_words(h);
     const float4 h0 = H[0], h1 = H[1], h2 = H[2], h3 = H[3], h4 = H[4];
-    const float tol = h0.w;
+    const float tol = h4.w;
     float s0, q[3], x[3], u[3];
     to_shifted(h0, r, s0, q);
     rotate_in(h1, h2, h3.x, q, x);
@@ -341,6 +346,101 @@ __device__ __forceinline__ float annulus_bound(const float tz, const float4 b, c
     const float t_r = fmaxf(x.rho - b.y, b.z - x.rho) * inv_r_lo;
     const float L = fmaxf(fmaxf(t_in, t_r), 0.f);
     return t_out < L || x.rr > b.y || L > Um ? f_inf() : L;
+}
+
+// The uniform grid of a volume as the walk reads it: the short form staged in
+// shared memory (cells: offset | count << 16, 16-bit entries) or the CSR lists
+// in global memory.
+struct GridTab {
+    const uint32_t* cells;
+    const uint16_t* ids16;
+    const int32_t* off;
+    const int32_t* fids;
+    const FiltHvy* hvy;
+};
+
+// The daughters listed in the cells that the track crosses before Um (3D-DDA
+// along the FP32 ray; at most gx + gy + gz + 3 cells).  What bounds it: the lanes'
+// own walks diverge, so the loop is flat -- every turn a lane goes on to its
+// next cell if its list is done, then looks at one entry -- until the lane holds a
+// daughter whose sphere it meets; then all lanes bound their daughters together.  A certain entry shortens Um and with it the walk (the
+// 512-daughter volume: about half of the tracks enter a daughter, most
+// far before the mother's exit).  A daughter met again is skipped (4-entry mailbox,
+// then the candidate list).
+template <bool SMALL>
+__device__ __forceinline__ void filter_grid(const VolView& v, const GridTab& g, const Ray32& r, float Um, Cands& c) {
+    // per axis: cells left before the walk leaves the grid, stride of the
+    // linear index, next boundary parameter, increment
+    int n0, n1, n2, s0, s1, s2;
+    float m0, m1, m2, e0, e1, e2;
+    int cell = 0;
+    auto setup = [&](int k, int pitch, int& left, int& st, float& tm, float& te) {
+        const float lo = v.lo32[k], w = v.cell32[k];
+        const int gk = v.grid[k];
+        int ii = int(floorf((r.p[k] - lo) * v.inv_cell32[k]));
+        ii = ii < 0 ? 0 : (ii >= gk ? gk - 1 : ii);
+        cell += ii * pitch;
+        const float d = r.d[k], inv = frcp(d);
+        const bool up = d > 0.f;
+        st = up ? pitch : -pitch;
+        left = up ? gk - 1 - ii : ii;
+        tm = d != 0.f ? (fmaf(float(up ? ii + 1 : ii), w, lo) - r.p[k]) * inv : f_inf();
+        te = d != 0.f ? w * fabsf(inv) : f_inf();
+    };
+    setup(0, v.grid[1] * v.grid[2], n0, s0, m0, e0);
+    setup(1, v.grid[2], n1, s1, m1, e1);
+    setup(2, 1, n2, s2, m2, e2);
+    int cur, end;
+    auto open = [&] {
+        if (SMALL) {
+            const uint32_t w = g.cells[cell];
+            cur = int(w & 0xffffu);
+            end = cur + int(w >> 16);
+        } else {
+            cur = g.off[cell];
+            end = g.off[cell + 1];
+        }
+    };
+    open();
+    int mb0 = -1, mb1 = -1, mb2 = -1, mb3 = -1;
+    bool more = true;
+    while (more) {
+        int found = -1;
+        do {
+            if (cur >= end) {   // the next cell, if the track reaches it before Um
+                const float mn = fminf(m0, fminf(m1, m2));
+                const bool a0 = m0 <= mn, a1 = !a0 && m1 <= mn, a2 = !a0 && !a1;
+                more = mn <= Um && (a0 ? n0 : (a1 ? n1 : n2)) > 0;
+                cell += a0 ? s0 : (a1 ? s1 : s2);
+                n0 -= a0;
+                n1 -= a1;
+                n2 -= a2;
+                m0 = a0 ? m0 + e0 : m0;
+                m1 = a1 ? m1 + e1 : m1;
+                m2 = a2 ? m2 + e2 : m2;
+                if (more) open();
+            }
+            if (cur < end) {   // the next entry of its list
+                const int j = SMALL ? int(g.ids16[cur]) : g.fids[cur];
+                ++cur;
+                if (j != mb0 && j != mb1 && j != mb2 && j != mb3) {
+                    mb3 = mb2; mb2 = mb1; mb1 = mb0; mb0 = j;
+                    const float4 h0 = hvy_words(g.hvy + j)[0];
+                    float t0, q[3];
+                    to_shifted(h0, r, t0, q);
+                    const float perp2 = fmaf(q[0], q[0], fmaf(q[1], q[1], q[2] * q[2]));
+                    const float half = h0.w * r.inv_dn;
+                    if (perp2 <= h0.w * h0.w * (1.f + 4.f * kEps32f) && t0 >= -half && t0 - half <= Um) found = j;
+                }
+            }
+        } while (found < 0 && more);
+        if (found >= 0) {
+            const FiltHvy* h = g.hvy + found;
+            if (!cand_holds(c, h->id))
+                Um = fminf(Um, (h->flags & kFiltBox) ? bound_box(h, r, Um, c) : bound_quad(h, r, Um, c));
+        }
+    }
+    cands_count(c);
 }
 
 // Every daughter of the volume, 32 at a time: the cheap tests together, then

@@ -411,11 +411,14 @@ void make_filter(const geo_placed_shape* in, const std::vector<ShapeRec32>& d, s
         const ShapeRec32& r = d[order[k]];
         std::memcpy(h.t, r.t, sizeof h.t);
         std::memcpy(h.R, r.R, sizeof h.R);
+        h.brad = r.brad;
         h.delta = r.delta;
         h.id = order[k];
         h.flags = (r.flags & kRec32Identity) ? kFiltIdentity : 0;
         if (r.kind == KBOX) {
             std::memcpy(h.e, r.e, 3 * sizeof(float));
+            h.e[3] = r.delta;
+            h.flags |= kFiltBox;
             continue;
         }
         float hi[2], lo[2];   // squared acceptance limits of the end annuli at -dz, +dz
@@ -517,7 +520,7 @@ geo_status cuda_status(cudaError_t e);
 // 1e-3 of a cell, overlaps it.  The growth keeps the lists conservative for
 // an FP32 grid walk whose rounding can cut a corner between two cells.
 geo_status build_voxels(const geo_placed_shape& m, const geo_placed_shape* d, int nd, double S,
-                        const geo_build_opts* opts, cudaStream_t s, geo_volume v) {
+                        const std::vector<FiltHvy>& filt, const geo_build_opts* opts, cudaStream_t s, geo_volume v) {
     double half[3];
     const geo_placed_shape mb = m.kind == GEO_PCON ? bounding_tube(m, true) : m;
     const double* p = mb.p;
@@ -535,6 +538,9 @@ geo_status build_voxels(const geo_placed_shape& m, const geo_placed_shape* d, in
         vw.lo[k] = -half[k];
         vw.cell[k] = 2.0 * half[k] / g[k];
         vw.inv_cell[k] = 1.0 / vw.cell[k];
+        vw.lo32[k] = float(vw.lo[k]);
+        vw.cell32[k] = float(vw.cell[k]);
+        vw.inv_cell32[k] = float(vw.inv_cell[k]);
     }
     std::vector<std::vector<int32_t>> lists(static_cast<size_t>(ncells));
     for (int j = 0; j < nd; ++j) {
@@ -563,6 +569,29 @@ geo_status build_voxels(const geo_placed_shape& m, const geo_placed_shape* d, in
         off[c + 1] = off[c] + int32_t(lists[c].size());
         ids.insert(ids.end(), lists[c].begin(), lists[c].end());
     }
+    const size_t nids = ids.size();
+    // the lists as entries of the filter's tables
+    std::vector<int32_t> entry(static_cast<size_t>(std::max(nd, 1)), 0);
+    for (size_t k = 0; k < filt.size(); ++k)
+        if (filt[k].brad > 0.f) entry[size_t(filt[k].id)] = int32_t(k);   // (filling entries have no radius)
+    for (size_t q = 0; q < nids; ++q) ids.push_back(entry[size_t(ids[q])]);
+    while (ids.size() % 4) ids.push_back(0);
+    // and in short form, offsets and counts in 16 bits each
+    const size_t small_at = ids.size();
+    bool fits = nids < 65536 && filt.size() < 65536;
+    for (int64_t c = 0; c < ncells; ++c) fits = fits && off[c + 1] - off[c] < 65536;
+    if (fits) {
+        for (int64_t c = 0; c < ncells; ++c)
+            ids.push_back(int32_t(uint32_t(off[c]) | (uint32_t(off[c + 1] - off[c]) << 16)));
+        while (ids.size() % 4) ids.push_back(0);
+        vw.vox_small_cells = uint32_t((ids.size() - small_at) * sizeof(int32_t));
+        std::vector<uint16_t> lo((nids + 7) / 8 * 8, 0);
+        for (size_t q = 0; q < nids; ++q) lo[q] = uint16_t(entry[size_t(ids[q])]);
+        const size_t at = ids.size();
+        ids.resize(at + lo.size() / 2);
+        std::memcpy(ids.data() + at, lo.data(), lo.size() * sizeof(uint16_t));
+        vw.vox_small_bytes = uint32_t((ids.size() - small_at) * sizeof(int32_t));
+    }
     if (ids.empty()) ids.push_back(0);
     cudaError_t e;
     if ((e = lib_malloc(&v->vox_off, sizeof(int32_t) * off.size())) != cudaSuccess ||
@@ -573,6 +602,8 @@ geo_status build_voxels(const geo_placed_shape& m, const geo_placed_shape* d, in
             cudaSuccess ||
         (e = cudaStreamSynchronize(s)) != cudaSuccess)
         return cuda_status(e);
+    vw.vox_fids = v->vox_ids + nids;
+    vw.vox_small = fits ? reinterpret_cast<const uint32_t*>(v->vox_ids + small_at) : nullptr;
     vw.vox_off = v->vox_off;
     vw.vox_ids = v->vox_ids;
     vw.voxelized = 1;
@@ -781,7 +812,7 @@ geo_status geo_build_volume(const geo_placed_shape* mother, const geo_placed_sha
     vw.status = v->status;
     v->h64 = std::move(h64);
     if (opts && opts->voxelize) {
-        st = build_voxels(*mother, daughters, n_daughters, S, opts, s, v);
+        st = build_voxels(*mother, daughters, n_daughters, S, hhvy, opts, s, v);
         if (st != GEO_OK) {
             geo_destroy_volume(v);
             return st;

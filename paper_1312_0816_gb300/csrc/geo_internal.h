@@ -95,28 +95,30 @@ static_assert(sizeof(ShapeRec32) == 128, "ShapeRec32 layout");
 //     entry's a = (brad of both)
 //  FiltHvy, gathered per lane (112 B: seven 16-byte words, an odd number, so
 //  that gathers of different entries meet few bank conflicts):
-//   t, delta; R (9); flags, daughter index (int bits); h, e by kind:
+//   t, bounding radius; R (9); flags, daughter index (int bits); h, e by kind:
 //   quadric: h = zl (dz' + delta); e = dz', a_out', b_out, a_in', b_in, the
 //     acceptance limits of the end annuli (hi at -dz, hi at +dz, lo at -dz, lo
-//     at +dz; see ShapeRec32); g = 4 delta sqrt(1 + the larger slope squared)
-//   box: e[0..2] = h + delta
+//     at +dz; see ShapeRec32); g = 4 delta sqrt(1 + the larger slope squared);
+//     delta
+//   box: e[0..2] = h + delta, e[3] = delta
 // kFiltLoose: the copy bounds another solid (a tube segment, a polycone, a hole
 // narrower than delta, a cone with an apex on an end plane), so that no
 // surface of it is surely the solid's.
-constexpr int32_t kFiltIdentity = 1, kFiltHole = 2, kFiltLoose = 4;
+constexpr int32_t kFiltIdentity = 1, kFiltHole = 2, kFiltLoose = 4, kFiltBox = 8;
 struct __align__(16) FiltSph {
     float4 a, b;
 };
 struct __align__(16) FiltHvy {
     float t[3];
-    float delta;
+    float brad;
     float R[9];
     int32_t flags;
     int32_t id;
     float h;
     float e[9];
     float g;
-    float pad[2];
+    float delta;
+    float pad;
 };
 static_assert(sizeof(FiltSph) == 32 && sizeof(FiltHvy) == 112, "filter table layout");
 
@@ -144,8 +146,15 @@ struct __align__(16) VolView {
     double lo[3];
     double cell[3];
     double inv_cell[3];
+    float lo32[3], cell32[3], inv_cell32[3];   // the same for the FP32 walk (a conversion holds the FP64 unit)
+    int32_t pad2_;
     const int32_t* vox_off;    // [ncells+1] CSR offsets
     const int32_t* vox_ids;    // daughter ids
+    const int32_t* vox_fids;   // the same daughters as entries of the filter's tables
+    const uint32_t* vox_small; // the grid in short form for staging: per cell offset | count << 16, then
+                               // the 16-bit filter entries (null: it does not fit 16 bits)
+    uint32_t vox_small_cells;  // bytes of the cells' part (a multiple of 16)
+    uint32_t vox_small_bytes;  // bytes of both parts (a multiple of 16)
     unsigned int* status;      // device error word (0 = ok)
 };
 

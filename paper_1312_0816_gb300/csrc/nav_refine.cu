@@ -192,8 +192,8 @@ __global__ void __launch_bounds__(P + C, 2) k_dist_batched(BatchView bv, Basket 
                 int h = -2, nev = 0;
                 rs.status = 1;
                 if (live)
-                    refine_pass1<GLOB ? kTravEither : kTravAll, SEGS>(v, f, v.d64, px, py, pz, qx, qy, qz,
-                                                                [&](int c) { return st_.pd[c][t]; }, rs, best, h, nev);
+                    refine_pass1<GLOB ? kTravEither : kTravAll, SEGS>(v, f, GridTab{}, v.d64, px, py, pz, qx, qy, qz,
+                                                                      [&](int c) { return st_.pd[c][t]; }, rs, best, h, nev);
                 int task = 0, bin = -1;
                 if (rs.status == 0) {
                     task = first_task(rs);
@@ -343,7 +343,7 @@ cudaError_t launch_dist_batched(const BatchView& bv, const Basket& b, double* st
 cudaError_t launch_dist_refine_stats(const VolView& v, const Basket& b, double* step, int32_t* hit,
                                      double* bpoint, int32_t* nref, cudaStream_t s, int num_sms) {
     if (split_basket(v, b.n, num_sms)) return launch_dist_refine_split(v, b, step, hit, bpoint, nref, s);
-    if (!v.segs && !v.voxelized) return launch_dist_direct(v, b, step, hit, bpoint, nref, s, num_sms);
+    if (!v.segs) return launch_dist_direct(v, b, step, hit, bpoint, nref, s, num_sms);
     if (b.n <= int64_t(4) * num_sms * kLatProd)
         return launch_dist_refine_latency(v, b, step, hit, bpoint, nref, s, num_sms);
     return launch_refine_cfg<kProd, kCons>(v, b, step, hit, bpoint, nref, s, num_sms);

@@ -40,78 +40,6 @@ __device__ __forceinline__ void bound_daughter(const ShapeRec32& r, int j, const
     cand_put(c, L, j);
 }
 
-// Walk of the uniform grid (3D-DDA) along the FP32 ray from its start to the
-// parameter tend, calling visit(j) for every daughter listed in every cell
-// entered.  At most gx + gy + gz + 3 cells.
-template <class F>
-__device__ __forceinline__ void vox_walk32(const VolView& v, const float* p, const float* d, float tend,
-                                           F&& visit) {
-    // per axis: cell index, step direction, next boundary parameter, increment
-    int i0, i1, i2, s0, s1, s2;
-    float m0, m1, m2, e0, e1, e2;
-    auto setup = [&](int k, int& ii, int& st, float& tm, float& te) {
-        const float lo = float(v.lo[k]), cell = float(v.cell[k]);
-        const int g = v.grid[k];
-        ii = int(floorf((p[k] - lo) * float(v.inv_cell[k])));
-        ii = ii < 0 ? 0 : (ii >= g ? g - 1 : ii);
-        if (d[k] > 0.f) {
-            st = 1;
-            tm = (fmaf(float(ii + 1), cell, lo) - p[k]) / d[k];
-            te = cell / d[k];
-        } else if (d[k] < 0.f) {
-            st = -1;
-            tm = (fmaf(float(ii), cell, lo) - p[k]) / d[k];
-            te = -cell / d[k];
-        } else {
-            st = 0;
-            tm = f_inf();
-            te = f_inf();
-        }
-    };
-    setup(0, i0, s0, m0, e0);
-    setup(1, i1, s1, m1, e1);
-    setup(2, i2, s2, m2, e2);
-    const int g0 = v.grid[0], g1 = v.grid[1], g2 = v.grid[2];
-    const int maxit = g0 + g1 + g2 + 3;
-    for (int it = 0; it < maxit; ++it) {
-        const int c = (i0 * g1 + i1) * g2 + i2;
-        const int q1 = v.vox_off[c + 1];
-        for (int q = v.vox_off[c]; q < q1; ++q) visit(v.vox_ids[q]);
-        if (m0 <= m1 && m0 <= m2) {
-            if (!(m0 <= tend)) break;
-            i0 += s0;
-            if (i0 < 0 || i0 >= g0) break;
-            m0 += e0;
-        } else if (m1 <= m2) {
-            if (!(m1 <= tend)) break;
-            i1 += s1;
-            if (i1 < 0 || i1 >= g1) break;
-            m1 += e1;
-        } else {
-            if (!(m2 <= tend)) break;
-            i2 += s2;
-            if (i2 < 0 || i2 >= g2) break;
-            m2 += e2;
-        }
-    }
-}
-
-// The daughters listed in the cells the track crosses before the mother's
-// exit (upper bound Um); a daughter met again is skipped (4-entry mailbox,
-// then the candidate list).
-__device__ __forceinline__ void bound_grid(const VolView& v, const Ray32& r, float Um, Cands& c) {
-    int mb0 = -1, mb1 = -1, mb2 = -1, mb3 = -1;
-    vox_walk32(v, r.p, r.d, Um, [&](int j) {
-        if (j == mb0 || j == mb1 || j == mb2 || j == mb3) return;
-        mb3 = mb2; mb2 = mb1; mb1 = mb0; mb0 = j;
-#pragma unroll
-        for (int k = 0; k < kCand; ++k)
-            if (c.L[k] < f_inf() && c.j[k] == j) return;
-        bound_daughter(v.d32[j], j, r, Um, c);
-    });
-    cands_count(c);
-}
-
 // The filter's cold FP64 paths (a direction magnitude outside the FP32
 // range, a start between the mother's shrunk copy and the mother, a bound
 // evicted from the list that could still win), out of line: inlined, their
@@ -225,19 +153,23 @@ __device__ __forceinline__ MotherExit mother_exit32(const VolView& v, const Ray3
 }
 
 // Which daughters the FP32 pass bounds: every daughter (filter_daughters),
-// the uniform grid's walk, either one by the volume, or the daughters j_first,
-// j_first + j_step, ... of the volume's own order (a share of them).
-enum : int { kTravAll = 0, kTravGrid = 1, kTravEither = 2, kTravShare = 3 };
+// the uniform grid's walk (over the CSR lists, or over their staged short
+// form), either one by the volume, or the daughters j_first, j_first + j_step,
+// ... of the volume's own order (a share of them).
+enum : int { kTravAll = 0, kTravGrid = 1, kTravEither = 2, kTravShare = 3, kTravGridSmall = 4 };
+
+// the grid's lists in global memory
+__device__ __forceinline__ GridTab grid_lists(const VolView& v) { return {nullptr, nullptr, v.vox_off, v.vox_fids, v.fhvy}; }
 
 // FP32 pass: bounds of the mother and of the daughters.  When status == 1 on
 // return, best/h already hold the final answer.  The FP64 track is taken from
 // `src` (src(k): x, y, z, dx, dy, dz) where the rare FP64 paths need it again, so
 // that a caller that holds it in shared memory need not keep it in registers.
 template <int TRAV, bool SEGS = true, class Src>
-__device__ __forceinline__ void refine_pass1(const VolView& v, const FiltTab& f, const ShapeRec64* __restrict__ tab64,
-                                             double px, double py, double pz, double qx, double qy, double qz, Src src,
-                                             RefineState& st, double& best, int& h, int& nev, int j_first = 0,
-                                             int j_step = 1) {
+__device__ __forceinline__ void refine_pass1(const VolView& v, const FiltTab& f, const GridTab& grid,
+                                             const ShapeRec64* __restrict__ tab64, double px, double py, double pz,
+                                             double qx, double qy, double qz, Src src, RefineState& st, double& best,
+                                             int& h, int& nev, int j_first = 0, int j_step = 1) {
     nev = 0;
     st.status = 1;
     cands_clear(st.c);
@@ -277,8 +209,10 @@ __device__ __forceinline__ void refine_pass1(const VolView& v, const FiltTab& f,
     if (TRAV == kTravShare) {
         for (int j = j_first; j < v.nd; j += j_step) bound_daughter(v.d32[j], j, r, Um, st.c);
         cands_count(st.c);
+    } else if (TRAV == kTravGridSmall) {
+        filter_grid<true>(v, grid, r, Um, st.c);
     } else if (TRAV == kTravGrid || (TRAV == kTravEither && v.voxelized)) {
-        bound_grid(v, r, Um, st.c);
+        filter_grid<false>(v, grid_lists(v), r, Um, st.c);
     } else {
         filter_daughters(f, r, Um, st.c);
     }

@@ -65,7 +65,7 @@ __global__ void __launch_bounds__(kSplitWarps * 32, kSplitBlocksPerSm)
         int h = -2, nev = 0;
         if (live) {
             const double tr[6] = {px, py, pz, qx, qy, qz};
-            refine_pass1<kTravShare, SEGS>(v, FiltTab{}, v.d64, px, py, pz, qx, qy, qz, [&](int k) { return tr[k]; }, rs,
+            refine_pass1<kTravShare, SEGS>(v, FiltTab{}, GridTab{}, v.d64, px, py, pz, qx, qy, qz, [&](int k) { return tr[k]; }, rs,
                                            best, h, nev, w, kSplitWarps);
         }
 #pragma unroll

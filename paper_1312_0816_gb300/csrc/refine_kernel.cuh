@@ -287,7 +287,7 @@ __global__ void __launch_bounds__(P + C, 2) k_dist_refine(const __grid_constant_
             int h = -2, nev = 0;
             rs.status = 1;
             if (live)
-                refine_pass1<TRAV, SEGS>(v, f, tab64, px, py, pz, qx, qy, qz, [&](int c) { return st_.pd[c][t]; }, rs, best,
+                refine_pass1<TRAV, SEGS>(v, f, GridTab{}, tab64, px, py, pz, qx, qy, qz, [&](int c) { return st_.pd[c][t]; }, rs, best,
                                          h, nev);
             int task = 0, bin = -1;
             if (rs.status == 0) {
@@ -366,17 +366,14 @@ static cudaError_t launch_refine_cfg(const VolView& v, const Basket& b, double* 
     static_assert(sizeof(Stage<P>) % 16 == 0 && sizeof(Answers<P>) % 16 == 0, "the tables stay 16-byte aligned");
     const int stages = 2 * int(sizeof(Stage<P>) + sizeof(Answers<P>));
     const int filt = v.nf * int(sizeof(FiltSph) + sizeof(FiltHvy));
+    // volumes without segments and polycones take the direct kernels
     if (v.voxelized) {
         // the grid walk needs registers: 12 + 2 warps at 72 registers beat
         // 12 + 4 at 64 (7.0 against 7.4 ms for 2^24 tracks in 512 daughters)
         constexpr int CV = P == kProd ? kVoxCons : C;
-        if (v.segs)
-            return launch_refine<P, CV>(k_dist_refine<P, CV, 0, kTravGrid, true>, stages, v, b, step, hit, bpoint, nref,
-                                        s, num_sms);
-        return launch_refine<P, CV>(k_dist_refine<P, CV, 0, kTravGrid, false>, stages, v, b, step, hit, bpoint, nref, s,
+        return launch_refine<P, CV>(k_dist_refine<P, CV, 0, kTravGrid, true>, stages, v, b, step, hit, bpoint, nref, s,
                                     num_sms);
     }
-    // volumes without segments and polycones take the direct kernel
     if (v.smem_refine == 2)
         return launch_refine<P, C>(k_dist_refine<P, C, 2, kTravAll, true>, stages + filt + v.nd * int(sizeof(ShapeRec64)), v,
                                    b, step, hit, bpoint, nref, s, num_sms);

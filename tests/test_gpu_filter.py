@@ -110,3 +110,20 @@ def test_batched_filter_equals_fp64_bitwise(g, which):
             assert torch.equal(s[a:a + c].view(torch.int64), s0.view(torch.int64))
     for v in vols:
         assert g.geo_check_device_status(v) == 0
+
+
+@pytest.mark.parametrize("grid", [(0, 0, 0), (1, 1, 1), (7, 3, 40)])
+@pytest.mark.parametrize("counts", [(1, 1, 1), (34, 31, 1), (0, 150, 130)])
+def test_grid_equals_fp64_bitwise(g, counts, grid):
+    """The grid's walk over the lists in global memory (one wave of tracks or
+    less) and over the short form staged in shared memory (beyond)."""
+    sc = filter_scene(*counts, "box", seed=sum(counts) + 7)
+    vol = g.geo_build_volume(sc, voxelize=True, grid=grid)
+    wave = 1024 * torch.cuda.get_device_properties(0).multi_processor_count
+    for n in (30011, wave - 1, wave, wave + 333):
+        t = tracks(sc, n, n)
+        s0, h0 = g.geo_dist_to_boundary(vol, *t, mode=g.GEO_FP64)
+        s1, h1 = g.geo_dist_to_boundary(vol, *t, mode=g.GEO_FP32_REFINE)
+        assert torch.equal(h0, h1)
+        assert torch.equal(s0.view(torch.int64), s1.view(torch.int64))
+    assert g.geo_check_device_status(vol) == 0
