@@ -34,17 +34,22 @@
 // with a square root and a division.  So the bound also says which surface the
 // exact line enters through, when that is certain, and FP64 evaluates that
 // surface alone, with the same operations as the whole routine and so the
-// same bits (surface64 in nav_refine.cuh).  Certain means: with every FP32 error
-// within delta of the true solid (the inflation's premise) the crossing lies in
-// [t, t + e]; over that interval it keeps several delta from every limit of
-// its acceptance (no edge nearby); no other surface of the solid has a
-// crossing before t + e; and the start is outside the inflated copy.  e is
-// the crossing's shift under a change of 4 delta of the solid: 4 delta / |u_z|
-// for an end plane, 4 delta R / sqrt(D) for a quadric, used only where D
-// exceeds its own change eightfold.  An accepted crossing that keeps clear of
-// the edges is the entry: before it the line is outside the surface's
-// constraint, which every earlier entry would have to satisfy.  The
-// upper bound t + e of a certain entry is also what the cut above uses.
+// same bits (surface64 in nav_refine.cuh).  The premise is that of the
+// inflation, with the room it leaves: the FP32 line lies within delta / 2 of
+// the exact one, rounding of the quadrics included (48 eps32 S of the
+// extent S are in delta; the roundings of position, direction, shift and
+// rotation add up to less than 16).  The copy is delta larger than the solid,
+// so the exact crossing is that of a solid delta / 2 to 3 delta / 2 smaller
+// than the copy.  Certain then means: under such a change the crossing lies in
+// [t, t + e]; over that interval it keeps clear of every limit of its
+// acceptance (no edge nearby); no other surface of the solid has a crossing before
+// t + e; and the start is outside the inflated copy.  e is 2 delta / |u_z| for
+// an end plane and 2 delta R / sqrt(D) for a quadric (R / sqrt(D) is the
+// crossing's derivative by R), used only where D exceeds four times its own
+// change.  An accepted crossing that keeps clear of the edges is the
+// entry: before it the line is outside the surface's constraint, which every
+// earlier entry would have to satisfy.  The upper bound t + e of a certain
+// entry is also what the cut above uses.
 #pragma once
 #include "geo_internal.h"
 #include "shapes32.cuh"
@@ -162,7 +167,7 @@ __device__ __forceinline__ float bound_quad(const FiltHvy* h, const Ray32& r, fl
     const float A0 = fmaf(u[0], u[0], u[1] * u[1]);
     const float B0 = fmaf(x[0], u[0], x[1] * u[1]);
     const float rho2 = fmaf(x[0], x[0], x[1] * x[1]);
-    const float tol4 = 4.f * tol, az = fabsf(u[2]);
+    const float tol2 = 2.f * tol, az = fabsf(u[2]);
     float best, e, second = f_inf();
     int tag = kTagPlane;
     bool sure;
@@ -175,11 +180,11 @@ __device__ __forceinline__ float bound_quad(const FiltHvy* h, const Ray32& r, fl
         const bool up = sz > 0.f;
         const float hi2 = up ? h5.z : h5.y, lo2 = up ? h6.x : h5.w;
         best = fabsf(sz) > dz && sz * u[2] < 0.f && r2 <= hi2 && r2 >= lo2 ? fmaxf(tz, tmin) : f_inf();
-        e = tol4 * fabsf(inv);
-        const float rh = fsqrt(r2), slack = fmaf(e, fsqrt(A0), tol4);
+        e = tol2 * fabsf(inv);
+        const float rh = fsqrt(r2), slack = fmaf(e, fsqrt(A0), tol2);
         sure = rh + slack <= fmaf(bo, ze, ao) && (!hole || rh - slack >= fmaf(bi, ze, ai));
     }
-    const float zs = dz - tol4;
+    const float zs = dz - tol2;
     auto quadric = [&](float a, float b, bool rising, int its) {
         const float r0 = fmaf(b, x[2], a), rs = b * u[2];
         const float A = fmaf(-rs, rs, A0), B = fmaf(-r0, rs, B0), C = fmaf(-r0, r0, rho2);
@@ -193,8 +198,8 @@ __device__ __forceinline__ float bound_quad(const FiltHvy* h, const Ray32& r, fl
         const float s = real && (bneg || A != 0.f) ? s0r : f_inf();
         const float z = fmaf(s, u[2], x[2]);
         if (s >= tmin && fabsf(z) <= zl) {
-            const float es = fdiv(h6.y * fabsf(fmaf(s, rs, r0)), sq);   // h6.y: 4 delta sqrt(1 + slope^2)
-            const bool ok = sq * sq > 4.f * h6.y * fmaf(A0, h6.y, fabsf(fmaf(A, r0, -B * rs))) &&
+            const float es = fdiv(h6.y * fabsf(fmaf(s, rs, r0)), sq);   // h6.y: 2 delta sqrt(1 + slope^2)
+            const bool ok = sq * sq > 6.f * h6.y * fmaf(A0, h6.y, fabsf(fmaf(A, r0, -B * rs))) &&
                             fmaf(az, es, fabsf(z)) <= zs;
             const bool first = s < best;
             second = first ? best : fminf(second, s);
@@ -212,11 +217,11 @@ __device__ __forceinline__ float bound_quad(const FiltHvy* h, const Ray32& r, fl
     const float last = best + e;
     sure = sure && !in0 && !(flags & kFiltLoose) && last + 32.f * kEps32f * fabsf(last) < second;
     cand_put(c, L, __float_as_int(h3.z) | (sure ? tag << kTagShift : 0));
-    return sure ? fmaf(32.f * kEps32f, fabsf(s0 + last), s0 + last) + tol4 * r.inv_dn : f_inf();
+    return sure ? fmaf(32.f * kEps32f, fabsf(s0 + last), s0 + last) + tol2 * r.inv_dn : f_inf();
 }
 
 // The same for a box: the axis of the latest slab entry, certain when it stays
-// the latest, and before every slab's exit, under a change of 4 delta.
+// the latest, and before every slab's exit, under a change of 2 delta.
 __device__ __forceinline__ float bound_box(const FiltHvy* h, const Ray32& r, float Um, Cands& c) {
     const float4* H = hvy_words(h);
     const float4 h0 = H[0], h1 = H[1], h2 = H[2], h3 = H[3], h4 = H[4];
@@ -238,7 +243,7 @@ __device__ __forceinline__ float bound_box(const FiltHvy* h, const Ray32& r, flo
         const float inv = fdiv(1.f, u[k]);
         const float a0 = (-hh[k] - x[k]) * inv, b0 = (hh[k] - x[k]) * inv;
         const float a = fminf(a0, b0), b = fmaxf(a0, b0);
-        const float e = 4.f * tol * fabsf(inv);
+        const float e = 2.f * tol * fabsf(inv);
         if (u[k] == 0.f) {
             miss = miss || fabsf(x[k]) > hh[k] + tol;
             out = -f_inf();   // not certain
@@ -257,9 +262,9 @@ __device__ __forceinline__ float bound_box(const FiltHvy* h, const Ray32& r, flo
     const float L = lower_bound(s0 + tn, tol, r.inv_dn);
     if (!(L <= Um)) return f_inf();
     const float m = 32.f * kEps32f * fmaxf(fabsf(tn), fabsf(last));
-    const bool sure = tag != kTagNone && tn - m > others && last + m < out && tn > tmin + m + 4.f * tol * r.inv_dn;
+    const bool sure = tag != kTagNone && tn - m > others && last + m < out && tn > tmin + m + 2.f * tol * r.inv_dn;
     cand_put(c, L, __float_as_int(h3.z) | (sure ? tag << kTagShift : 0));
-    return sure ? fmaf(32.f * kEps32f, fabsf(s0 + last), s0 + last) + 4.f * tol * r.inv_dn : f_inf();
+    return sure ? fmaf(32.f * kEps32f, fabsf(s0 + last), s0 + last) + 2.f * tol * r.inv_dn : f_inf();
 }
 
 // Two FP32 values in one register pair: one instruction for both (the

@@ -438,7 +438,7 @@ void make_filter(const geo_placed_shape* in, const std::vector<ShapeRec32>& d, s
         }
         h.e[5] = hi[0]; h.e[6] = hi[1]; h.e[7] = lo[0]; h.e[8] = lo[1];
         const double slope = std::max(std::fabs(double(h.e[2])), std::fabs(double(h.e[4])));
-        h.g = float_up(4.0 * double(r.delta) * std::sqrt(1.0 + slope * slope));
+        h.g = float_up(2.0 * double(r.delta) * std::sqrt(1.0 + slope * slope));
         const geo_placed_shape& sh = in[order[k]];
         const bool has_hole = sh.kind == GEO_TUBE ? sh.p[0] > 0 : (sh.kind == GEO_CONE && (sh.p[1] > 0 || sh.p[3] > 0));
         if (needs_segs_code(sh) || (has_hole && !(h.flags & kFiltHole))) h.flags |= kFiltLoose;

@@ -98,7 +98,7 @@ static_assert(sizeof(ShapeRec32) == 128, "ShapeRec32 layout");
 //   t, bounding radius; R (9); flags, daughter index (int bits); h, e by kind:
 //   quadric: h = zl (dz' + delta); e = dz', a_out', b_out, a_in', b_in, the
 //     acceptance limits of the end annuli (hi at -dz, hi at +dz, lo at -dz, lo
-//     at +dz; see ShapeRec32); g = 4 delta sqrt(1 + the larger slope squared);
+//     at +dz; see ShapeRec32); g = 2 delta sqrt(1 + the larger slope squared);
 //     delta
 //   box: e[0..2] = h + delta, e[3] = delta
 // kFiltLoose: the copy bounds another solid (a tube segment, a polycone, a hole

@@ -395,4 +395,23 @@ static __device__ __noinline__ void refine_rest(const VolView& v, const ShapeRec
     }
 }
 
+// a track whose first task is not certain: the whole solid (rare, out of line)
+static __device__ __noinline__ double eval64_cold(const VolView& v, const ShapeRec64* __restrict__ tab64, int j, double px,
+                                                  double py, double pz, double qx, double qy, double qz) {
+    return eval64<false>(v, tab64, j, px, py, pz, qx, qy, qz);
+}
+
+// The FP64 part of a track after its FP32 pass.
+__device__ __forceinline__ void finish_direct(const VolView& v, const ShapeRec64* __restrict__ tab64, const ShapeRec64& m64,
+                                              const RefineState& rs, double px, double py, double pz, double qx,
+                                              double qy, double qz, double& best, int& h, int& nev) {
+    if (rs.status != 0) return;
+    const int task = first_task(rs);
+    double s1;
+    if (rs.tag != kTagNone) s1 = surface64(task < 0 ? m64 : tab64[task], rs.tag, task < 0, px, py, pz, qx, qy, qz);
+    else s1 = eval64_cold(v, tab64, task, px, py, pz, qx, qy, qz);
+    nev = 1;
+    if (!refine_fast(rs, s1, best, h)) refine_rest<false>(v, tab64, rs, s1, px, py, pz, qx, qy, qz, best, h, nev);
+}
+
 }  // namespace geonav

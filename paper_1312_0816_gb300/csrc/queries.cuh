@@ -131,7 +131,7 @@ __device__ __forceinline__ float above(double s, float tau) {
 // inflated radius covers the FP32 position errors; the square root is
 // lowered by the relative margin).
 __device__ __forceinline__ float sphere_lb32(const ShapeRec32& r, float c2) {
-    return fsqrt(c2) * (1.f - kSafMargin) - r.brad;
+    return saf_sqrt(c2) * (1.f - kSafMargin) - r.brad;
 }
 
 // Bounding-sphere cull of daughter r against a bound L: true when the whole

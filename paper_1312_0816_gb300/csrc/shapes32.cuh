@@ -286,6 +286,10 @@ __device__ __forceinline__ bool contains32(const ShapeRec32& r, const float* x) 
 // part, proportional to the solid's size, is inside delta).
 constexpr float kSafMargin = 3.8146973e-06f;   // 2^-18
 
+// The safety bounds are results too (GEO_SAFETY_ESTIMATE), so they keep these
+// forms of the roots.
+__device__ __forceinline__ float saf_sqrt(float a) { return a > 0.f ? a * rsqrtf(a) : 0.f; }
+
 // Lower bound of the outside-safety of an INFLATED copy (distance from x to
 // the solid).  Box and tube: the exact Euclidean distance to the copy (the
 // tube in the meridian half-plane, to the rectangle [rmin, rmax] x [-dz, dz]).
@@ -300,20 +304,20 @@ __device__ __forceinline__ float safety_out_lb32(const ShapeRec32& r, const floa
     if (r.kind == KBOX) {
         const float a = fmaxf(fabsf(x[0]) - e[0], 0.f), b = fmaxf(fabsf(x[1]) - e[1], 0.f),
                     c = fmaxf(fabsf(x[2]) - e[2], 0.f);
-        s = fsqrt(fmaf(a, a, fmaf(b, b, c * c)));
+        s = saf_sqrt(fmaf(a, a, fmaf(b, b, c * c)));
     } else {
-        const float rho = fsqrt(fmaf(x[0], x[0], x[1] * x[1]));
+        const float rho = saf_sqrt(fmaf(x[0], x[0], x[1] * x[1]));
         const float az = fabsf(x[2]);
         if (r.kind == KTUBE) {
-            float dr = rho - fsqrt(e[1]);
-            if (e[3] != 0.f) dr = fmaxf(dr, fsqrt(e[0]) - rho);
+            float dr = rho - saf_sqrt(e[1]);
+            if (e[3] != 0.f) dr = fmaxf(dr, saf_sqrt(e[0]) - rho);
             dr = fmaxf(dr, 0.f);
             const float dz = fmaxf(az - e[2], 0.f);
-            s = fsqrt(fmaf(dr, dr, dz * dz));
+            s = saf_sqrt(fmaf(dr, dr, dz * dz));
         } else {
             s = az - e[0];
-            s = fmaxf(s, (rho - fmaf(e[2], x[2], e[1])) * frsqrt(fmaf(e[2], e[2], 1.f)));
-            if (e[5] != 0.f) s = fmaxf(s, (fmaf(e[4], x[2], e[3]) - rho) * frsqrt(fmaf(e[4], e[4], 1.f)));
+            s = fmaxf(s, (rho - fmaf(e[2], x[2], e[1])) * rsqrtf(fmaf(e[2], e[2], 1.f)));
+            if (e[5] != 0.f) s = fmaxf(s, (fmaf(e[4], x[2], e[3]) - rho) * rsqrtf(fmaf(e[4], e[4], 1.f)));
             s = fmaxf(s, 0.f);
         }
     }
@@ -332,15 +336,15 @@ __device__ __forceinline__ float safety_in_lb32(const ShapeRec32& r, const float
     if (r.kind == KBOX) {
         s = fminf(e[0] - fabsf(x[0]), fminf(e[1] - fabsf(x[1]), e[2] - fabsf(x[2])));
     } else {
-        const float rho = fsqrt(fmaf(x[0], x[0], x[1] * x[1]));
+        const float rho = saf_sqrt(fmaf(x[0], x[0], x[1] * x[1]));
         const float az = fabsf(x[2]);
         if (r.kind == KTUBE) {
-            s = fminf(fsqrt(e[1]) - rho, e[2] - az);
-            if (e[3] != 0.f) s = fminf(s, rho - fsqrt(e[0]));
+            s = fminf(saf_sqrt(e[1]) - rho, e[2] - az);
+            if (e[3] != 0.f) s = fminf(s, rho - saf_sqrt(e[0]));
         } else {
             s = e[0] - az;
-            s = fminf(s, (fmaf(e[2], x[2], e[1]) - rho) * frsqrt(fmaf(e[2], e[2], 1.f)));
-            if (e[5] != 0.f) s = fminf(s, (rho - fmaf(e[4], x[2], e[3])) * frsqrt(fmaf(e[4], e[4], 1.f)));
+            s = fminf(s, (fmaf(e[2], x[2], e[1]) - rho) * rsqrtf(fmaf(e[2], e[2], 1.f)));
+            if (e[5] != 0.f) s = fminf(s, (rho - fmaf(e[4], x[2], e[3])) * rsqrtf(fmaf(e[4], e[4], 1.f)));
         }
     }
     return fmaxf(s, 0.f) * (1.f - kSafMargin);
