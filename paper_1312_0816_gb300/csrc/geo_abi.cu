@@ -441,6 +441,12 @@ void make_filter(const geo_placed_shape* in, const std::vector<ShapeRec32>& d, s
         h.g = float_up(2.0 * double(r.delta) * std::sqrt(1.0 + slope * slope));
         const geo_placed_shape& sh = in[order[k]];
         const bool has_hole = sh.kind == GEO_TUBE ? sh.p[0] > 0 : (sh.kind == GEO_CONE && (sh.p[1] > 0 || sh.p[3] > 0));
+        if (sh.kind == GEO_CONE) {
+            const double r[5] = {sh.p[1], sh.p[2], sh.p[4], sh.p[3], sh.p[1]};
+            bool exact = true;
+            for (int q = 0; q < 4; ++q) exact = exact && r[q] + (r[q + 1] - r[q]) == r[q + 1];
+            if (exact) h.flags |= kFiltVertex;
+        }
         if (needs_segs_code(sh) || (has_hole && !(h.flags & kFiltHole))) h.flags |= kFiltLoose;
         if (k < nq1) {
             const bool axis = k % 32 == 0 || r.t[0] != sph[k - 1].a.x || r.t[1] != sph[k - 1].a.y;

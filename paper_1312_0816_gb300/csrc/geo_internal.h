@@ -104,7 +104,9 @@ static_assert(sizeof(ShapeRec32) == 128, "ShapeRec32 layout");
 // kFiltLoose: the copy bounds another solid (a tube segment, a polycone, a hole
 // narrower than delta, a cone with an apex on an end plane), so that no
 // surface of it is surely the solid's.
-constexpr int32_t kFiltIdentity = 1, kFiltHole = 2, kFiltLoose = 4, kFiltBox = 8;
+// kFiltVertex: a cone whose edges end on its vertices exactly (a + (b - a) = b
+// in FP64 for every edge's radii).
+constexpr int32_t kFiltIdentity = 1, kFiltHole = 2, kFiltLoose = 4, kFiltBox = 8, kFiltVertex = 16;
 struct __align__(16) FiltSph {
     float4 a, b;
 };

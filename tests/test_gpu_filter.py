@@ -22,10 +22,11 @@ def g():
     return pkg
 
 
-def filter_scene(n1, n2, n3, mother, seed):
+def filter_scene(n1, n2, n3, mother, seed, apex=False):
     """n1 unrotated tubes and cones (nested shells about two axes: shells of no
-    thickness, holes far narrower than the filter's inflation, cones ending
-    in an apex), n2 rotated ones, n3 boxes; they may overlap."""
+    thickness, holes far narrower than the filter's inflation), n2 rotated
+    ones (apex: cones ending in an apex too, whose volumes take other
+    kernels), n3 boxes; they may overlap."""
     rng = np.random.default_rng(seed)
     eye = np.eye(3).reshape(9)
     rows = []
@@ -42,7 +43,7 @@ def filter_scene(n1, n2, n3, mother, seed):
     for k in range(n2):
         t = rng.uniform(-350.0, 350.0, 3)
         if k % 2:
-            rows.append((scenes.CONE, (rng.uniform(5.0, 40.0), 0.0, 0.0 if k % 6 == 1 else 10.0, 2.0, 25.0),
+            rows.append((scenes.CONE, (rng.uniform(5.0, 40.0), 0.0 if apex else 1.0, 0.0 if apex and k % 6 == 1 else 10.0, 2.0, 25.0),
                          scenes.haar_rotation(rng), t))
         else:
             rows.append((scenes.TUBE, (0.0 if k % 4 else 6.0, rng.uniform(8.0, 30.0), rng.uniform(5.0, 40.0)),
@@ -77,10 +78,10 @@ COUNTS = [(0, 0, 1), (1, 0, 0), (1, 1, 1), (2, 1, 0), (31, 2, 5), (32, 0, 0), (3
           (2, 65, 33), (40, 40, 19), (0, 150, 130)]
 
 
-@pytest.mark.parametrize("mother", ["box", "tube"])
+@pytest.mark.parametrize("mother,apex", [("box", False), ("tube", False), ("box", True)])
 @pytest.mark.parametrize("counts", COUNTS)
-def test_filter_equals_fp64_bitwise(g, counts, mother):
-    sc = filter_scene(*counts, mother, seed=sum(counts) + 7)
+def test_filter_equals_fp64_bitwise(g, counts, mother, apex):
+    sc = filter_scene(*counts, mother, seed=sum(counts) + 7, apex=apex)
     vol = g.geo_build_volume(sc)
     for n in (257, 70001):   # n = 257: the small-basket kernels; 70001: the direct or the pipelined one
         t = tracks(sc, n, n)
@@ -126,4 +127,29 @@ def test_grid_equals_fp64_bitwise(g, counts, grid):
         s1, h1 = g.geo_dist_to_boundary(vol, *t, mode=g.GEO_FP32_REFINE)
         assert torch.equal(h0, h1)
         assert torch.equal(s0.view(torch.int64), s1.view(torch.int64))
+    assert g.geo_check_device_status(vol) == 0
+
+
+@pytest.mark.parametrize("mother", ["box", "tube"])
+@pytest.mark.parametrize("counts", COUNTS)
+def test_point_queries_equal_fp64_bitwise(g, counts, mother):
+    """Contains and Safety of points anywhere, on the solids' surfaces and a
+    little beside them (where FP32 cannot decide and whole solids are
+    evaluated), on their axes and in their coordinate planes."""
+    sc = filter_scene(*counts, mother, seed=sum(counts) + 7)
+    vol = g.geo_build_volume(sc)
+    rng = np.random.default_rng(3)
+    for n in (33, 5003, 170001):   # 33 and 5003: 32 points a warp; 170001: 64
+        t = tracks(sc, n, n + 1)
+        s, _ = g.geo_dist_to_boundary(vol, *t, mode=g.GEO_FP64)
+        s = torch.where(torch.isfinite(s), s, 0.0) * (1.0 + 1e-9 * torch.from_numpy(rng.integers(-1, 2, n)).cuda())
+        on = [t[k] + s * t[3 + k] for k in range(3)]
+        j = rng.integers(0, sc.n_daughters, n)
+        axis = sc.trans[j] + np.einsum("nij,nj->ni", sc.rot[j].reshape(n, 3, 3),
+                                       rng.uniform(-1.5, 1.5, (n, 3)) * 40.0 * rng.integers(0, 2, (n, 3)))
+        axis = [torch.from_numpy(np.ascontiguousarray(axis[:, k])).cuda() for k in range(3)]
+        for p in (t[:3], on, axis):
+            assert torch.equal(g.geo_contains(vol, *p, mode=g.GEO_FP64), g.geo_contains(vol, *p))
+            s0, s1 = g.geo_safety(vol, *p, mode=g.GEO_FP64), g.geo_safety(vol, *p)
+            assert torch.equal(s0.view(torch.int64), s1.view(torch.int64))
     assert g.geo_check_device_status(vol) == 0
