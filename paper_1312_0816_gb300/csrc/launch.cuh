@@ -19,9 +19,12 @@ static inline int blocks_for(K kernel, int64_t n, int smem, int num_sms, int thr
     return int(need < cap ? need : cap);
 }
 
+// Lets a kernel take `smem` bytes of dynamic shared memory.  The limit that
+// holds without this (48 KB) counts the kernel's static shared memory too, of
+// which the callers' kernels have up to 16 KB.
 template <typename K>
 static inline cudaError_t prep(K kernel, int smem) {
-    if (smem > 48 * 1024) return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    if (smem > 32 * 1024) return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     return cudaSuccess;
 }
 
