@@ -181,8 +181,10 @@ __device__ __forceinline__ float bound_quad(const FiltHvy* h, const Ray32& r, fl
         const float hi2 = up ? h5.z : h5.y, lo2 = up ? h6.x : h5.w;
         best = fabsf(sz) > dz && sz * u[2] < 0.f && r2 <= hi2 && r2 >= lo2 ? fmaxf(tz, tmin) : f_inf();
         e = tol2 * fabsf(inv);
-        const float rh = fsqrt(r2), slack = fmaf(e, fsqrt(A0), tol2);
-        sure = rh + slack <= fmaf(bo, ze, ao) && (!hole || rh - slack >= fmaf(bi, ze, ai));
+        // against the solid's own annulus: its radius lines at its own end (the
+        // copy's are delta sqrt(1 + slope^2) further out, and its end delta)
+        const float rh = fsqrt(r2), slack = fmaf(e, fsqrt(A0), fmaf(0.5f, h6.y, tol)), zt = copysignf(dz - tol, sz);
+        sure = rh + slack <= fmaf(bo, zt, ao) && (!hole || rh - slack >= fmaf(bi, zt, ai));
     }
     const float zs = dz - tol2;
     auto quadric = [&](float a, float b, bool rising, int its) {
@@ -448,11 +450,95 @@ __device__ __forceinline__ void filter_grid(const VolView& v, const GridTab& g, 
     cands_count(c);
 }
 
+// Re-entry of a track into solid h that it has just left (it starts on the
+// solid's surface): kReentryNone when the exact line surely does not enter it again,
+// the surface (kTagOuter / kTagInner) of the sure next entry with a lower
+// bound of its parameter in L, kTagNone when it is not certain.  The margins
+// are those of a certain entry (above).
+constexpr int kReentryNone = -1;
+__device__ __forceinline__ int reentry32(const FiltHvy* h, const Ray32& r, float& L) {
+    const float4* H = hvy_words(h);
+    const float4 h0 = H[0], h3 = H[3], h4 = H[4];
+    const int flags = __float_as_int(h3.y);
+    L = 0.f;
+    if (flags & kFiltLoose) return kTagNone;
+    const float w[3] = {r.p[0] - h0.x, r.p[1] - h0.y, r.p[2] - h0.z};
+    float x[3], u[3];
+    if (flags & kFiltIdentity) {
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            x[k] = w[k];
+            u[k] = r.d[k];
+        }
+    } else {
+        const float4 h1 = H[1], h2 = H[2];
+        rotate_in(h1, h2, h3.x, w, x);
+        rotate_in(h1, h2, h3.x, r.d, u);
+    }
+    const float umin = 16.f * kEps32f * frcp(r.inv_dn);   // a component's sign is certain above it
+    if (flags & kFiltBox) {
+        // one face near, the track moving out of its slab, the others far: the
+        // box's exit from that slab lies behind the start
+        const float d = h4.w, hh[3] = {h4.x, h4.y, h4.z};
+        int near = 0;
+        bool ok = true;
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            const float a = fabsf(x[k]) - (hh[k] - d);
+            if (a > -2.f * d) {
+                ++near;
+                ok = ok && a < 2.f * d && fabsf(x[k]) > 2.f * d && x[k] * u[k] > 0.f && fabsf(u[k]) > umin;
+            }
+        }
+        return ok && near == 1 ? kReentryNone : kTagNone;
+    }
+    const float4 h5 = H[5], h6 = H[6];
+    const float d = h6.z, g = h6.y, dz = h4.x - d;
+    const float az = fabsf(x[2]) - dz;
+    if (az > 2.f * d || (az > -2.f * d && !(fabsf(x[2]) > 2.f * d && x[2] * u[2] > 0.f && fabsf(u[2]) > umin)))
+        return kTagNone;
+    const float A0 = fmaf(u[0], u[0], u[1] * u[1]);
+    const float B0 = fmaf(x[0], u[0], x[1] * u[1]);
+    const float rho2 = fmaf(x[0], x[0], x[1] * x[1]);
+    float hi = f_inf();   // the entry found lies in [L, hi]
+    int tag = kReentryNone;
+    bool ok = true;
+    // (the copy's radius lines: the solid's own are delta away, inside g's margin)
+    auto quadric = [&](float a, float b, bool rising, int its) {
+        const float r0 = fmaf(b, x[2], a), rs = b * u[2];
+        const float A = fmaf(-rs, rs, A0), B = fmaf(-r0, rs, B0), C = fmaf(-r0, r0, rho2);
+        const float D = fmaf(B, B, -A * C);
+        const float change = 6.f * g * fmaf(A0, g, fabsf(fmaf(A, r0, -B * rs)));
+        if (D < -change - 16.f * kEps32f * fmaf(B, B, fabsf(A * C))) return;   // no crossing at all
+        if (!(D > change) || !(fabsf(A) > 1e-6f * A0)) {
+            ok = false;
+            return;
+        }
+        const float sq = fsqrt(D), sg = rising ? -1.f : 1.f, Bs = sg * B;
+        const bool bneg = Bs < 0.f;
+        const float s = fdiv(bneg ? sg * C : -Bs - sq, bneg ? sq - Bs : sg * A);
+        const float e = fmaf(32.f * kEps32f, fabsf(s), fdiv(g * fabsf(fmaf(s, rs, r0)), sq)) + 2.f * d * r.inv_dn;
+        if (s < -e || s - e > hi) return;   // behind, or after the other entry
+        const float z = fabsf(fmaf(s, u[2], x[2])), zs = fmaf(fabsf(u[2]), e, 2.f * d);
+        if (s > e && z - zs > dz) return;   // beyond the ends
+        const bool sure = s > e && z + zs < dz;
+        ok = ok && sure && (tag == kReentryNone || s + e < L);
+        hi = s + e;
+        L = s - e;
+        tag = its;
+    };
+    quadric(h4.y, h4.z, false, kTagOuter);
+    if (ok && (flags & kFiltHole)) quadric(h4.w, h5.x, true, kTagInner);
+    return ok ? tag : kTagNone;
+}
+
 // Every daughter of the volume, 32 at a time: the cheap tests together, then
 // each lane's own solids (one call site per kind of bound: the pass's code has
 // to stay small, warps run its parts at different times and share the
 // instruction caches).
-__device__ __forceinline__ void filter_daughters(const FiltTab& f, const Ray32& r, float Um, Cands& c) {
+// SKIP: the entry `skip` (-1 none) is left out.
+template <bool SKIP = false>
+__device__ __forceinline__ void filter_daughters(const FiltTab& f, const Ray32& r, float Um, Cands& c, int skip = -1) {
     // a direction within 1e-6 of the axis: no radial bound (its FP32
     // perpendicular part may have lost its precision)
     const float perp2 = fmaf(r.d[0], r.d[0], r.d[1] * r.d[1]);
@@ -472,7 +558,8 @@ __device__ __forceinline__ void filter_daughters(const FiltTab& f, const Ray32& 
         for (; k < n1; ++k) {
             const float4 a = S[k].a, b = S[k].b;
             if (a.w != 0.f) to_axis(a, r, inv_r, ax);   // warp-uniform: another axis than the solid before
-            const float L = annulus_bound(a.z, b, ax, r, inv_z_lo, inv_z_hi, inv_r_lo, Um);
+            float L = annulus_bound(a.z, b, ax, r, inv_z_lo, inv_z_hi, inv_r_lo, Um);
+            if (SKIP) L = base + k == skip ? f_inf() : L;
             m |= L < f_inf() ? 1u << k : 0u;
             const bool p1 = L < l1, p2 = L < l2;
             l3 = fminf(l3, fmaxf(l2, L));
@@ -487,6 +574,7 @@ __device__ __forceinline__ void filter_daughters(const FiltTab& f, const Ray32& 
 #pragma unroll 2
             for (; k < cnt; k += 2) m |= spheres_ahead(S + k, r2, Um) << k;
         }
+        if (SKIP && skip >= base && skip < base + 32) m &= ~(1u << (skip - base));
         // quadrics: the two with the least annulus bounds first, then the
         // others in order; an annulus bit is looked at again, against the bound
         // Um of what has been found since

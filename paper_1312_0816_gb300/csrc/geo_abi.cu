@@ -455,6 +455,8 @@ void make_filter(const geo_placed_shape* in, const std::vector<ShapeRec32>& d, s
                               float_down(std::sqrt(double(std::min(lo[0], lo[1])))), h.h);
         }
     }
+    for (int k = 0; k < nf; ++k)
+        if (order[k] >= 0) hvy[size_t(order[k])].entry = k;
     for (int k = nq1; k < nf; k += 2) {
         float t[2][3] = {}, b2[2] = {-1.f, -1.f}, br[2] = {};
         for (int q = 0; q < 2; ++q) {

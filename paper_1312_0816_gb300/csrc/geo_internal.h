@@ -101,6 +101,7 @@ static_assert(sizeof(ShapeRec32) == 128, "ShapeRec32 layout");
 //     at +dz; see ShapeRec32); g = 2 delta sqrt(1 + the larger slope squared);
 //     delta
 //   box: e[0..2] = h + delta, e[3] = delta
+//   entry: of daughter k (k the record's own position), the inverse of id
 // kFiltLoose: the copy bounds another solid (a tube segment, a polycone, a hole
 // narrower than delta, a cone with an apex on an end plane), so that no
 // surface of it is surely the solid's.
@@ -120,7 +121,7 @@ struct __align__(16) FiltHvy {
     float e[9];
     float g;
     float delta;
-    float pad;
+    int32_t entry;
 };
 static_assert(sizeof(FiltSph) == 32 && sizeof(FiltHvy) == 112, "filter table layout");
 
@@ -143,7 +144,8 @@ struct __align__(16) VolView {
     // voxel grid (uniform over the mother's bounding box)
     int32_t voxelized;
     int32_t grid[3];
-    int32_t segs;              // 1 if the mother or a daughter is a tube segment or a polycone
+    int32_t segs;              // 1 if the mother or a daughter is a tube segment or a polycone, or a cone with an
+                               // apex on an end plane (needs_segs_code)
     int32_t pad_;
     double lo[3];
     double cell[3];

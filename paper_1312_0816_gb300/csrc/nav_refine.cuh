@@ -78,14 +78,20 @@ __device__ __forceinline__ int first_task(const RefineState& st) {
 // other surface's exit from the shrunk one.
 struct MotherExit {
     float lo, hi;
-    bool in;    // inside the shrunk copy
+    bool in;    // inside the shrunk copy: the bounds hold
     int tag;    // kTagPlane / kTagOuter / kTagInner, a box's kTagAxis + k, kTagNone: not certain
 };
 
-__device__ __forceinline__ MotherExit mother_exit32(const VolView& v, const Ray32& r) {
+// `entered`: the track starts on the mother's surface, moving in.  The bounds
+// hold then as well (`in`) when the line crosses the shrunk copy's outer
+// surface (it does not graze it) and does not leave through the inner one at
+// its start: it starts off that surface, or moves away from the axis.
+template <bool ENTERED = false>
+__device__ __forceinline__ MotherExit mother_exit32(const VolView& v, const Ray32& r, bool entered = false) {
     const float *el = v.m32.e, *eh = v.m32u.e, *x = r.p, *u = r.d;
     MotherExit m;
     float second = f_inf(), thi = f_inf();
+    bool crosses = true;   // (entered)
     m.lo = m.hi = f_inf();
     m.tag = kTagNone;
     auto take = [&](float lo, float hi, int tag) {
@@ -108,16 +114,22 @@ __device__ __forceinline__ MotherExit mother_exit32(const VolView& v, const Ray3
         const float rho2 = fmaf(x[0], x[0], x[1] * x[1]);
         const float A0 = fmaf(u[0], u[0], u[1] * u[1]);
         const float B0 = fmaf(x[0], u[0], x[1] * u[1]);
+        // both copies' quadrics: the outer one left where it rises, the inner one where it falls
+        auto outer = [&](float Al, float Bl, float Cl, float Ah, float Bh, float Ch) {
+            const float lo = root_rising32(Al, Bl, Cl), hi = root_rising32(Ah, Bh, Ch);
+            if (ENTERED) crosses = fmaf(Bl, Bl, -Al * Cl) > 16.f * kEps32f * fmaf(Bl, Bl, fabsf(Al * Cl)) && lo >= 0.f;
+            take(lo >= 0.f ? lo : f_inf(), hi >= 0.f ? hi : f_inf(), kTagOuter);
+        };
+        auto inner = [&](float Al, float Bl, float Cl, bool hole, float Ah, float Bh, float Ch) {
+            const float lo = root_falling32(Al, Bl, Cl), hi = hole ? root_falling32(Ah, Bh, Ch) : f_inf();
+            if (ENTERED) crosses = crosses && (Cl >= 0.f || Bl > 64.f * kEps32f * fsqrt(Al > 0.f ? Al * rho2 : f_inf()));
+            take(lo >= 0.f ? lo : f_inf(), hi >= 0.f ? hi : f_inf(), kTagInner);
+        };
         if (kind == KTUBE) {
             m.in = fabsf(x[2]) <= el[2] && rho2 <= el[1] && (el[3] == 0.f || rho2 >= el[0]);
             plane(2, el[2], eh[2], kTagPlane);
-            float lo = root_rising32(A0, B0, rho2 - el[1]), hi = root_rising32(A0, B0, rho2 - eh[1]);
-            take(lo >= 0.f ? lo : f_inf(), hi >= 0.f ? hi : f_inf(), kTagOuter);
-            if (el[3] != 0.f) {
-                lo = root_falling32(A0, B0, rho2 - el[0]);
-                hi = eh[3] != 0.f ? root_falling32(A0, B0, rho2 - eh[0]) : f_inf();
-                take(lo >= 0.f ? lo : f_inf(), hi >= 0.f ? hi : f_inf(), kTagInner);
-            }
+            outer(A0, B0, rho2 - el[1], A0, B0, rho2 - eh[1]);
+            if (el[3] != 0.f) inner(A0, B0, rho2 - el[0], eh[3] != 0.f, A0, B0, rho2 - eh[0]);
         } else {
             // inside test on the same rounded constants as the roots, so that a
             // point counted inside never sees a root behind it
@@ -127,24 +139,22 @@ __device__ __forceinline__ MotherExit mother_exit32(const VolView& v, const Ray3
                 B = fmaf(-r0, rs, B0);
                 C = fmaf(-r0, r0, rho2);
             };
-            float A, B, C, Ch;
+            float A, B, C, Ah, Bh, Ch;
             cone(el, 1, A, B, C);
+            cone(eh, 1, Ah, Bh, Ch);
             m.in = fabsf(x[2]) <= el[0] && C <= 0.f;
             plane(2, el[0], eh[0], kTagPlane);
-            float lo = root_rising32(A, B, C);
-            cone(eh, 1, A, B, Ch);
-            float hi = root_rising32(A, B, Ch);
-            take(lo >= 0.f ? lo : f_inf(), hi >= 0.f ? hi : f_inf(), kTagOuter);
+            outer(A, B, C, Ah, Bh, Ch);
             if (el[5] != 0.f) {
                 cone(el, 3, A, B, C);
+                cone(eh, 3, Ah, Bh, Ch);
                 m.in = m.in && C >= 0.f;
-                lo = root_falling32(A, B, C);
-                cone(eh, 3, A, B, Ch);
-                hi = eh[5] != 0.f ? root_falling32(A, B, Ch) : f_inf();
-                take(lo >= 0.f ? lo : f_inf(), hi >= 0.f ? hi : f_inf(), kTagInner);
+                inner(A, B, C, eh[5] != 0.f, Ah, Bh, Ch);
             }
+            if (ENTERED) crosses = false;   // (the double cone's other nappe: not argued)
         }
     }
+    if (ENTERED) m.in = m.in || (entered && crosses && v.m64.kind < KTUBS);
     m.lo = fmaxf(m.lo, 0.f);
     m.hi = fmaxf(m.hi, 0.f);
     const float dt = 4.f * v.m32u.delta * r.inv_dn;

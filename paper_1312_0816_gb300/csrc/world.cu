@@ -94,6 +94,47 @@ __global__ void __launch_bounds__(256) k_world_scatter(WorldView w, int64_t n, c
     }
 }
 
+// The same by blocks: each block counts its share of the tracks per group in
+// shared memory, reserves its slots with one global atomic per group, then
+// places its tracks with shared atomics.  (With one global atomic per group
+// and warp the few groups' counters set the pace: 2^20 tracks of the toy world
+// 68 us, 12 us so.)
+constexpr int kScatterThreads = 512;
+__global__ void __launch_bounds__(kScatterThreads) k_world_scatter_block(WorldView w, int64_t n,
+                                                                         const int32_t* __restrict__ node_in, int nkeys,
+                                                                         int32_t* __restrict__ off,
+                                                                         int32_t* __restrict__ perm) {
+    extern __shared__ int32_t h_smem[];   // counts, then next slots
+    const int lane = threadIdx.x & 31;
+    const int64_t share = (n + gridDim.x - 1) / gridDim.x;
+    const int64_t a = share * blockIdx.x, e = a + share < n ? a + share : n;
+    for (int k = threadIdx.x; k < nkeys; k += kScatterThreads) h_smem[k] = 0;
+    __syncthreads();
+    for (int pass = 0; pass < 2; ++pass) {
+        for (int64_t base = a; base < e; base += kScatterThreads) {
+            const int64_t i = base + threadIdx.x;
+            const bool live = i < e;
+            const int key = live ? world_key(w, nkeys - 1, node_in[i]) : -1;
+            const unsigned same = __match_any_sync(0xffffffffu, key);
+            const int leader = __ffs(same) - 1;
+            int pos = 0;
+            if (live && lane == leader) pos = atomicAdd(&h_smem[key], __popc(same));
+            if (pass == 1) {
+                pos = __shfl_sync(0xffffffffu, pos, leader);
+                if (live) perm[pos + __popc(same & ((1u << lane) - 1u))] = int32_t(i);
+            }
+        }
+        __syncthreads();
+        if (pass == 0) {
+            for (int k = threadIdx.x; k < nkeys; k += kScatterThreads) {
+                const int c = h_smem[k];
+                h_smem[k] = c ? atomicAdd(&off[k], c) : 0;
+            }
+            __syncthreads();
+        }
+    }
+}
+
 // The plain FP64 step (GEO_FP64), one thread per track over the grouped
 // order.  Three resident blocks per SM (80 registers, some spills) instead of
 // two at 124 (measured on the filtered step when it ran this way: 0.44 ->
@@ -128,7 +169,8 @@ __global__ void __launch_bounds__(256, 3) k_world_step(WorldView w, Basket b, co
     }
 }
 
-// The filtered step (GEO_FP32_REFINE) by tiles of 256 tracks of the grouped
+// The filtered step (GEO_FP32_REFINE) of a tree with tube segments, polycones or
+// cones with an apex on an end plane (the others: world_direct.cu), by tiles of 256 tracks of the grouped
 // order, with the FP64 evaluations every track needs binned by solid kind:
 // the FP32 pass per track; then each track's first FP64 task and, after it
 // left a daughter, that daughter's re-entry distance, run by whole warps over
@@ -324,7 +366,11 @@ cudaError_t launch_world_group(const WorldView& w, int64_t n, const int32_t* nod
                                                                                           cnt);
     }
     k_world_scan<<<1, 1024, 0, s>>>(nkeys, cnt);
-    k_world_scatter<<<blocks_for(k_world_scatter, n, 0, num_sms), 256, 0, s>>>(w, n, node_in, nkeys, cnt, perm);
+    if (nkeys <= kHistSmemKeys)
+        k_world_scatter_block<<<blocks_for(k_world_scatter_block, n, int(sizeof(int32_t)) * nkeys, num_sms, kScatterThreads),
+                                kScatterThreads, sizeof(int32_t) * nkeys, s>>>(w, n, node_in, nkeys, cnt, perm);
+    else
+        k_world_scatter<<<blocks_for(k_world_scatter, n, 0, num_sms), 256, 0, s>>>(w, n, node_in, nkeys, cnt, perm);
     return cudaGetLastError();
 }
 
@@ -334,6 +380,8 @@ cudaError_t launch_world_step(const WorldView& w, const Basket& b, const int32_t
     if (mode == GEO_FP64)
         k_world_step<<<blocks_for(k_world_step, b.n, 0, num_sms), 256, 0, s>>>(w, b, perm, node_in, flag_in, step,
                                                                             node_out, flag_out);
+    else if (!w.segs)
+        return launch_world_step_direct(w, b, perm, node_in, flag_in, step, node_out, flag_out, s, num_sms);
     else
         k_world_step_binned<<<blocks_for(k_world_step_binned, b.n, 0, num_sms), kWorldTile, 0, s>>>(
             w, b, perm, node_in, flag_in, step, node_out, flag_out);

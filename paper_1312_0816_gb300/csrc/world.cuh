@@ -46,6 +46,7 @@ struct WorldView {
     const int32_t* first;
     const double* xf;   // [12 * nnodes]
     int32_t nnodes;
+    int32_t segs;       // 1 if a logical volume needs the segments' code
 };
 
 cudaError_t launch_world_locate(const WorldView& w, const Basket& b, int32_t* node, cudaStream_t s, int num_sms);
@@ -57,10 +58,26 @@ cudaError_t launch_world_step(const WorldView& w, const Basket& b, const int32_t
                               const int32_t* flag_in, double* step, int32_t* node_out, int32_t* flag_out, int mode,
                               cudaStream_t s, int num_sms);
 
+// the filtered step, one thread per track, for trees whose volumes hold boxes,
+// tubes and cones alone (no `segs`)
+cudaError_t launch_world_step_direct(const WorldView& w, const Basket& b, const int32_t* perm, const int32_t* node_in,
+                                     const int32_t* flag_in, double* step, int32_t* node_out, int32_t* flag_out,
+                                     cudaStream_t s, int num_sms);
+
 // x in N's frame: R^T (p - t)
+// (a rotation that is exactly the identity leaves them as they are, up to the
+// sign of a zero, which no later operation looks at)
 __device__ __forceinline__ void world_to_node(const double* G, double px, double py, double pz, double qx,
                                               double qy, double qz, double* x, double* u) {
     const double w0 = SUB(px, G[9]), w1 = SUB(py, G[10]), w2 = SUB(pz, G[11]);
+    constexpr long long kOneBits = 0x3ff0000000000000LL;
+    const bool ident = BITS(G[0]) == kOneBits && BITS(G[4]) == kOneBits && BITS(G[8]) == kOneBits && IS_ZERO(G[1]) && IS_ZERO(G[2]) && IS_ZERO(G[3]) &&
+                       IS_ZERO(G[5]) && IS_ZERO(G[6]) && IS_ZERO(G[7]);
+    if (ident) {
+        x[0] = w0; x[1] = w1; x[2] = w2;
+        u[0] = qx; u[1] = qy; u[2] = qz;
+        return;
+    }
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
         x[k] = FMA(G[6 + k], w2, FMA(G[3 + k], w1, MUL(G[k], w0)));

@@ -21,6 +21,7 @@ struct geo_world_s {
     int32_t nnodes = 0;
     int32_t max_depth = 0;
     int32_t nlv = 0;
+    int32_t segs = 0;            // a logical volume needs the segments' code
     // grouping scratch of geo_world_step (grown on demand)
     int32_t* d_cnt = nullptr;
     int32_t* d_perm = nullptr;
@@ -59,6 +60,7 @@ WorldView world_view(const geo_world_s* w) {
     v.first = w->d_node + 3 * size_t(w->nnodes);
     v.xf = w->d_xf;
     v.nnodes = w->nnodes;
+    v.segs = w->segs;
     return v;
 }
 
@@ -137,6 +139,7 @@ geo_status geo_build_world(const geo_volume* volumes, int32_t n_volumes, const i
     if (!w) return GEO_ERR_OOM;
     w->device = dev;
     w->nlv = n_volumes;
+    for (int v = 0; v < n_volumes; ++v) w->segs = w->segs || volume_view(volumes[v])->segs;
     w->nnodes = int32_t(lv.size());
     w->max_depth = maxd;
     w->h_lv = lv;

@@ -75,7 +75,7 @@ def tracks(sc, n, seed):
 
 
 COUNTS = [(0, 0, 1), (1, 0, 0), (1, 1, 1), (2, 1, 0), (31, 2, 5), (32, 0, 0), (33, 0, 1), (34, 31, 1), (1, 32, 32),
-          (2, 65, 33), (40, 40, 19), (0, 150, 130)]
+          (2, 65, 33), (40, 40, 19), (0, 150, 130), (10, 50, 32)]
 
 
 @pytest.mark.parametrize("mother,apex", [("box", False), ("tube", False), ("box", True)])
@@ -153,3 +153,37 @@ def test_point_queries_equal_fp64_bitwise(g, counts, mother):
             s0, s1 = g.geo_safety(vol, *p, mode=g.GEO_FP64), g.geo_safety(vol, *p)
             assert torch.equal(s0.view(torch.int64), s1.view(torch.int64))
     assert g.geo_check_device_status(vol) == 0
+
+
+@pytest.mark.parametrize("n", [33, 4099, 300007])
+def test_world_states_equal_fp64_bitwise(g, n):
+    """The geometry-tree step from consistent states (Locate, then steps with
+    the flags they return) and from arbitrary ones (any node, any flag, any
+    point): re-entries and entered nodes that FP32 decides alone give the
+    FP64 mode's bits."""
+    tree = scenes.world_toy()
+    vols = [g.geo_build_volume(s) for s in tree.volumes]
+    world = g.geo_build_world(vols, tree.child, tree.root)
+    rng = np.random.default_rng(n)
+    t = [torch.from_numpy(f).cuda() for f in scenes.world_points(tree, n, n).fields()]
+    node = g.geo_world_locate(world, *t[:3])
+    flag = torch.full_like(node, -1)
+
+    def both(t, node, flag):
+        a = g.geo_world_step(world, *t, node, flag, mode=g.GEO_FP64)
+        b = g.geo_world_step(world, *t, node, flag, mode=g.GEO_FP32_REFINE)
+        assert torch.equal(a[0].view(torch.int64), b[0].view(torch.int64))
+        assert torch.equal(a[1], b[1]) and torch.equal(a[2], b[2])
+        return b
+
+    for _ in range(5):
+        any_node = torch.from_numpy(rng.integers(-2, world.n_nodes + 2, n).astype(np.int32)).cuda()
+        any_flag = torch.from_numpy(rng.integers(-3, 44, n).astype(np.int32)).cuda()
+        both(t, any_node, any_flag)
+        both(t, node, any_flag)
+        s, node2, flag = both(t, node, flag)
+        s = torch.where(torch.isfinite(s), s, 0.0)
+        t = [t[k] + s * t[3 + k] for k in range(3)] + t[3:]
+        if rng.random() < 0.5:   # scattered: another direction from the boundary
+            t = t[:3] + [torch.from_numpy(f).cuda() for f in scenes.isotropic(rng, n)]
+        node = node2
