@@ -7,13 +7,34 @@
 
 namespace geonav {
 
-template <typename K>
-static inline int blocks_for(K kernel, int64_t n, int smem, int num_sms, int threads = 256) {
-    int per_sm = 0;
+// Resident blocks per SM of a kernel (at least 1).  The occupancy query costs
+// about as much host time as a launch, and its answer depends on the kernel, the block
+// and the device alone, so each thread keeps the answers it has had.
+static inline int resident_blocks(const void* kernel, int threads, int smem) {
+    struct Entry {
+        const void* kernel;
+        int threads, smem, device, blocks;
+    };
+    constexpr int kEntries = 64;
+    static thread_local Entry cache[kEntries];
+    static thread_local int used = 0;
+    int device = -1, per_sm = 0;
+    const bool known = cudaGetDevice(&device) == cudaSuccess;
+    for (int k = 0; known && k < used; ++k) {
+        const Entry& e = cache[k];
+        if (e.kernel == kernel && e.threads == threads && e.smem == smem && e.device == device) return e.blocks;
+    }
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, threads, smem) != cudaSuccess || per_sm < 1) {
         cudaGetLastError();
-        per_sm = 1;
+        return 1;
     }
+    if (known && used < kEntries) cache[used++] = {kernel, threads, smem, device, per_sm};
+    return per_sm;
+}
+
+template <typename K>
+static inline int blocks_for(K kernel, int64_t n, int smem, int num_sms, int threads = 256) {
+    const int per_sm = resident_blocks(reinterpret_cast<const void*>(kernel), threads, smem);
     const int64_t need = (n + threads - 1) / threads;
     const int64_t cap = int64_t(per_sm) * num_sms;
     return int(need < cap ? need : cap);

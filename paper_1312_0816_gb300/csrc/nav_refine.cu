@@ -299,13 +299,7 @@ static cudaError_t launch_batched(const BatchView& bv, const Basket& b, double* 
     cudaError_t e =
         cudaFuncSetAttribute(k_dist_batched<SEGS, GLOB, P, C>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
-    int maxb = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&maxb, k_dist_batched<SEGS, GLOB, P, C>, P + C, smem) !=
-            cudaSuccess ||
-        maxb < 1) {
-        cudaGetLastError();
-        maxb = 1;
-    }
+    const int maxb = resident_blocks(reinterpret_cast<const void*>(k_dist_batched<SEGS, GLOB, P, C>), P + C, smem);
     const int per_sm = (blocks_per_sm <= 0 || blocks_per_sm > maxb) ? maxb : blocks_per_sm;
     k_dist_batched<SEGS, GLOB, P, C><<<per_sm * num_sms, P + C, smem, s>>>(bv, b, step, hit, room);
     return cudaGetLastError();

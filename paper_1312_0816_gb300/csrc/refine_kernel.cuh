@@ -339,11 +339,7 @@ __global__ void __launch_bounds__(P + C, 2) k_dist_refine(const __grid_constant_
 
 template <int P, int C, typename K>
 static int grid_refine(K kernel, int64_t n, int smem, int num_sms) {
-    int per_sm = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, P + C, smem) != cudaSuccess || per_sm < 1) {
-        cudaGetLastError();
-        per_sm = 1;
-    }
+    const int per_sm = resident_blocks(reinterpret_cast<const void*>(kernel), P + C, smem);
     const int64_t need = (n + P - 1) / P;
     const int64_t cap = int64_t(per_sm) * num_sms;
     return int(need < cap ? need : cap);

@@ -124,12 +124,30 @@ def _check(st: int, what: str):
         raise GeoError(st, what)
 
 
-def _stream(stream):
-    import torch
+_torch = None
 
+
+def _th():
+    """The torch module (imported on first use: building volumes and the CPU
+    tests need no CUDA tensors)."""
+    global _torch
+    if _torch is None:
+        import torch
+
+        _torch = torch
+    return _torch
+
+
+def _stream(stream) -> int:
+    """The cudaStream_t as an integer: `stream`, or torch's current stream of
+    the current device (read as the raw handle, which costs a tenth of a
+    microsecond where building a torch.cuda.Stream object costs three)."""
     if stream is None:
-        stream = torch.cuda.current_stream()
-    return ctypes.c_void_p(int(stream.cuda_stream) if hasattr(stream, "cuda_stream") else int(stream))
+        T = _th()
+        if T.cuda.is_initialized():
+            return T._C._cuda_getCurrentRawStream(T._C._cuda_getDevice())
+        stream = T.cuda.current_stream()
+    return int(stream.cuda_stream) if hasattr(stream, "cuda_stream") else int(stream)
 
 
 def _shape_struct(kind, params, rot=None, trans=None, pdata=None, keep=None) -> geo_placed_shape:
@@ -218,22 +236,20 @@ def geo_volume_info(vol: Volume):
     return {"n_daughters": nd.value, "voxelized": bool(vx.value), "grid": tuple(g)}
 
 
-def _dev(t, dtype, n, name):
-    import torch
-
-    if not isinstance(t, torch.Tensor) or not t.is_cuda:
+def _dev(t, dtype, n, name) -> int:
+    """The device address of a contiguous CUDA tensor of n elements."""
+    if not isinstance(t, _torch.Tensor) or not t.is_cuda:
         raise TypeError(f"{name}: expected a CUDA tensor")
-    if t.dtype != dtype or not t.is_contiguous() or t.numel() != n:
+    if t.dtype is not dtype or t.numel() != n or not t.is_contiguous():
         raise ValueError(f"{name}: expected contiguous {dtype} with {n} elements")
-    return ctypes.c_void_p(t.data_ptr())
+    return t.data_ptr()
 
 
 def geo_dist_to_boundary(vol: Volume, x, y, z, dx, dy, dz, mode: int = GEO_FP32_REFINE, step=None, hit=None,
                          bpoint=None, want_bpoint: bool = False, stream=None):
     """Fig. 1 navigator step for a basket of CUDA float64 tensors.  Returns
     (step, hit) or (step, hit, bpoint[3, n])."""
-    import torch
-
+    torch = _th()
     n = int(x.numel())
     f64 = torch.float64
     if step is None:
@@ -243,7 +259,7 @@ def geo_dist_to_boundary(vol: Volume, x, y, z, dx, dy, dz, mode: int = GEO_FP32_
     if want_bpoint and bpoint is None:
         bpoint = torch.empty((3, n), dtype=f64, device=x.device)
     args = [_dev(a, f64, n, nm) for a, nm in ((x, "x"), (y, "y"), (z, "z"), (dx, "dx"), (dy, "dy"), (dz, "dz"))]
-    bp = _dev(bpoint, f64, 3 * n, "bpoint") if bpoint is not None else ctypes.c_void_p(0)
+    bp = _dev(bpoint, f64, 3 * n, "bpoint") if bpoint is not None else None
     _check(load().geo_dist_to_boundary(vol.handle, *args, n, _dev(step, f64, n, "step"),
                                        _dev(hit, torch.int32, n, "hit"), bp, int(mode), _stream(stream)),
            "geo_dist_to_boundary")
@@ -254,8 +270,7 @@ def geo_contains(vol: Volume, x, y, z, mode: int = GEO_FP32_REFINE, where=None, 
     """Navigator-level Contains: -2 outside the mother, -1 mother only, else
     the lowest-index daughter containing the point (same answer in both
     modes)."""
-    import torch
-
+    torch = _th()
     n = int(x.numel())
     if where is None:
         where = torch.empty(n, dtype=torch.int32, device=x.device)
@@ -269,8 +284,7 @@ def geo_safety(vol: Volume, x, y, z, mode: int = GEO_FP32_REFINE, safety=None, s
     """Navigator-level Safety: exact Euclidean in GEO_FP64 and GEO_FP32_REFINE
     (the same FP64 value), or the cheaper lower bound with
     GEO_SAFETY_ESTIMATE."""
-    import torch
-
+    torch = _th()
     n = int(x.numel())
     f64 = torch.float64
     if safety is None:
@@ -288,8 +302,7 @@ def geo_shape_query(kind, params, what, x, y, z, dx=None, dy=None, dz=None, rot=
     """One solid's DistFromOutside / DistFromInside / safeties / Contains for a
     basket of CUDA float64 tensors (positions in the frame the solid is placed
     in).  Returns out, or (out, face) with want_face."""
-    import torch
-
+    torch = _th()
     n = int(x.numel())
     f64 = torch.float64
     if out is None:
@@ -299,10 +312,10 @@ def geo_shape_query(kind, params, what, x, y, z, dx=None, dy=None, dz=None, rot=
     keep = []
     shape = _shape_struct(kind, params, rot, trans, keep=keep)
     dist = what in (GEO_Q_DIST_OUT, GEO_Q_DIST_IN)
-    dirs = [_dev(a, f64, n, nm) if dist else ctypes.c_void_p(0) for a, nm in ((dx, "dx"), (dy, "dy"), (dz, "dz"))]
+    dirs = [_dev(a, f64, n, nm) if dist else None for a, nm in ((dx, "dx"), (dy, "dy"), (dz, "dz"))]
     _check(load().geo_shape_query(ctypes.byref(shape), int(what), _dev(x, f64, n, "x"), _dev(y, f64, n, "y"),
                                   _dev(z, f64, n, "z"), *dirs, n, _dev(out, f64, n, "out"),
-                                  _dev(face, torch.int32, n, "face") if face is not None else ctypes.c_void_p(0),
+                                  _dev(face, torch.int32, n, "face") if face is not None else None,
                                   _stream(stream)), "geo_shape_query")
     return (out, face) if want_face else out
 
@@ -367,8 +380,7 @@ def geo_world_nodes(world: World) -> dict:
 
 
 def geo_world_locate(world: World, x, y, z, node=None, stream=None):
-    import torch
-
+    torch = _th()
     n = int(x.numel())
     f64 = torch.float64
     if node is None:
@@ -382,8 +394,7 @@ def geo_world_step(world: World, x, y, z, dx, dy, dz, node, flag=None, mode: int
                    node_out=None, flag_out=None, stream=None):
     """One step of every track in its node, then relocation.  Returns
     (step, node_out, flag_out)."""
-    import torch
-
+    torch = _th()
     n = int(x.numel())
     f64 = torch.float64
     if step is None:
@@ -394,7 +405,7 @@ def geo_world_step(world: World, x, y, z, dx, dy, dz, node, flag=None, mode: int
         flag_out = torch.empty(n, dtype=torch.int32, device=x.device)
     args = [_dev(a, f64, n, nm) for a, nm in ((x, "x"), (y, "y"), (z, "z"), (dx, "dx"), (dy, "dy"), (dz, "dz"))]
     _check(load().geo_world_step(world.handle, *args, n, _dev(node, torch.int32, n, "node"),
-                                 _dev(flag, torch.int32, n, "flag") if flag is not None else ctypes.c_void_p(0),
+                                 _dev(flag, torch.int32, n, "flag") if flag is not None else None,
                                  _dev(step, f64, n, "step"), _dev(node_out, torch.int32, n, "node_out"),
                                  _dev(flag_out, torch.int32, n, "flag_out"), int(mode), _stream(stream)),
            "geo_world_step")
@@ -435,8 +446,7 @@ def geo_dist_to_boundary_host(vol: Volume, x, y, z, dx, dy, dz, mode: int = GEO_
 def geo_dist_to_boundary_stats(vol: Volume, x, y, z, dx, dy, dz, stream=None):
     """FP32+refine step that also returns the per-track count of FP64 solid
     evaluations.  Returns (step, hit, nref)."""
-    import torch
-
+    torch = _th()
     n = int(x.numel())
     f64 = torch.float64
     step = torch.empty(n, dtype=f64, device=x.device)
@@ -531,8 +541,7 @@ def geo_destroy_batch(batch: Batch):
 
 def geo_dist_to_boundary_batched(batch: Batch, x, y, z, dx, dy, dz, step=None, hit=None, stream=None):
     """One persistent launch over every basket of the batch (FP32+refine)."""
-    import torch
-
+    torch = _th()
     n = int(x.numel())
     f64 = torch.float64
     if step is None:
@@ -551,8 +560,7 @@ def geo_dist_to_boundary_batched_noalloc(volumes, baskets, x, y, z, dx, dy, dz, 
     fixed scratch array is used instead): for callers that cannot let a
     library allocate while they run.  step / hit must be preallocated CUDA
     tensors.  Calls sharing the scratch must not overlap on the GPU."""
-    import torch
-
+    torch = _th()
     n = int(x.numel())
     f64 = torch.float64
     nv = len(volumes)
@@ -579,23 +587,23 @@ def geo_dist_to_boundary_adjoint(vol: Volume, x, y, z, dx, dy, dz, hit, grad_ste
     """Gradients of sum(grad_step * step): returns grad_p (3, n), grad_d (3, n)
     and, when want_geometry, grad_trans (nd, 3) and grad_params (nd + 1, 5)
     (the mother's parameters last)."""
-    import torch
-
+    torch = _th()
     n = int(x.numel())
     f64 = torch.float64
     nd = vol.n_daughters
     gp = torch.empty((3, n), dtype=f64, device=x.device)
     gd = torch.empty((3, n), dtype=f64, device=x.device)
-    gt = torch.zeros((max(nd, 1), 3), dtype=f64, device=x.device) if want_geometry else None
-    gprm = torch.zeros((nd + 1, 5), dtype=f64, device=x.device) if want_geometry else None
+    # (the reduction writes every element; an empty basket launches nothing)
+    make = torch.empty if n > 0 else torch.zeros
+    gt = make((max(nd, 1), 3), dtype=f64, device=x.device) if want_geometry else None
+    gprm = make((nd + 1, 5), dtype=f64, device=x.device) if want_geometry else None
     ws = torch.empty(max(geo_adjoint_workspace_size(vol, n), 8) // 8 + 1, dtype=f64, device=x.device)
     args = [_dev(a, f64, n, nm) for a, nm in ((x, "x"), (y, "y"), (z, "z"), (dx, "dx"), (dy, "dy"), (dz, "dz"))]
     _check(load().geo_dist_to_boundary_adjoint(
         vol.handle, *args, n, _dev(hit, torch.int32, n, "hit"), _dev(grad_step, f64, n, "grad_step"),
         _dev(gp, f64, 3 * n, "grad_p"), _dev(gd, f64, 3 * n, "grad_d"),
-        ctypes.c_void_p(gt.data_ptr()) if gt is not None else ctypes.c_void_p(0),
-        ctypes.c_void_p(gprm.data_ptr()) if gprm is not None else ctypes.c_void_p(0),
-        ctypes.c_void_p(ws.data_ptr()), ctypes.c_uint64(ws.numel() * 8), _stream(stream)),
+        gt.data_ptr() if gt is not None else None, gprm.data_ptr() if gprm is not None else None, ws.data_ptr(),
+        ws.numel() * 8, _stream(stream)),
         "geo_dist_to_boundary_adjoint")
     if not want_geometry:
         return gp, gd
