@@ -244,6 +244,17 @@ struct ShapeArg {
     ShapeRec64 r;
     double table[kPconTableMax];
 };
+// The same for a box, tube or cone whose FP32 copies decide most of a query:
+// its placed copy (an entry of the filter's tables), the copies shrunk and
+// grown in its own frame, and the largest coordinate of a point they are good for.
+struct ShapeFast {
+    ShapeRec64 m64;
+    ShapeRec32 m32, m32u;
+    FiltHvy h;
+    float reach;
+};
+cudaError_t launch_shape_lists(const ShapeFast& a, int what, const Basket& b, double* out, int32_t* face,
+                               cudaStream_t s, int num_sms);
 cudaError_t launch_shape_query(const ShapeArg& a, int what, const Basket& b, double* out, int32_t* face,
                                cudaStream_t s, int num_sms);
 size_t adjoint_smem_bytes(int nd);

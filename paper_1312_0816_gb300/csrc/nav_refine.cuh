@@ -86,8 +86,9 @@ struct MotherExit {
 // hold then as well (`in`) when the line crosses the shrunk copy's outer
 // surface (it does not graze it) and does not leave through the inner one at
 // its start: it starts off that surface, or moves away from the axis.
-template <bool ENTERED = false>
-__device__ __forceinline__ MotherExit mother_exit32(const VolView& v, const Ray32& r, bool entered = false) {
+// V holds the solid's copies m32 (shrunk), m32u (grown) and its record m64.
+template <bool ENTERED = false, class V>
+__device__ __forceinline__ MotherExit mother_exit32(const V& v, const Ray32& r, bool entered = false) {
     const float *el = v.m32.e, *eh = v.m32u.e, *x = r.p, *u = r.d;
     MotherExit m;
     float second = f_inf(), thi = f_inf();
@@ -260,8 +261,9 @@ __device__ __forceinline__ double eval64(const VolView& v, const ShapeRec64* __r
 //    operation of a root commutes with the change of all signs).
 //  * A plane needs one local coordinate; it is formed where a quadric forms its
 //    first.
+// ahead: (optional) the sign of the plane coordinate's direction.
 __device__ __forceinline__ double surface64(const ShapeRec64& r, int tag, bool exit, double px, double py, double pz,
-                                            double qx, double qy, double qz) {
+                                            double qx, double qy, double qz, bool* ahead = nullptr) {
     const double* d = r.d;
     const bool quad = tag == kTagOuter || tag == kTagInner, inner = tag == kTagInner;
     const int k = quad ? 0 : (tag >= kTagAxis ? tag - kTagAxis : 2);
@@ -306,6 +308,7 @@ __device__ __forceinline__ double surface64(const ShapeRec64& r, int tag, bool e
         const double c = copysign(h, uk);
         num = SUB(exit ? c : -c, xk);
         den = uk;
+        if (ahead) *ahead = IS_POS(uk);
     }
     // one division for both kinds of lane (the empty statement keeps the
     // compiler from moving a copy of it into each branch)

@@ -162,7 +162,8 @@ __device__ __forceinline__ int entry_zone(const FiltHvy* h, const float* p) {
 }
 
 // The zone of a point surely inside the mother: its nearest surface, by 4 delta.
-__device__ __forceinline__ int mother_zone(const VolView& v, const float* p) {
+template <class V>
+__device__ __forceinline__ int mother_zone(const V& v, const float* p) {
     const float* e = v.m32.e;
     const float d = 4.f * v.m32.delta;
     float s[3];

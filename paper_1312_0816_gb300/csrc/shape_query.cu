@@ -14,6 +14,8 @@
 #include "geo_internal.h"
 #include "launch.cuh"
 #include "nav_common.cuh"
+#include "nav_refine.cuh"
+#include "point_pass.cuh"
 #include "shapes64.cuh"
 
 namespace geonav {
@@ -58,6 +60,205 @@ __global__ void __launch_bounds__(256) k_shape(const __grid_constant__ ShapeArg 
         }
         out[i] = v;
         if (face) face[i] = f;
+    }
+}
+
+// Boxes, tubes and cones: FP32 decides misses, points surely inside or
+// outside, and the one surface or nearest feature that FP64 has to evaluate
+// (filter_pass.cuh, point_pass.cuh); the tracks that need FP64 are gathered, up to 128 per
+// warp, so that 32 of one sort run together.  Tracks beyond the copies'
+// reach or of directions outside the FP32 range take the whole routine.
+//
+// What bounds it: the latency of the FP64 chains (FP64 unit 54 %, issue 35 %);
+// 22 FP64 instructions per 32 tracks of a placed cone, of which a quarter hit. DistFromOutside
+// of 2^20 tracks: k_shape 230 us (113 FP64 instructions), 72 us so.
+constexpr int kSoloWarps = 8;
+constexpr int kSoloBatch = 128;
+constexpr int kSoloSorts = 4;   // plane, quadric or radius, edge or corner, whole solid
+struct __align__(16) SoloBatch {   // one warp's
+    double p[6][kSoloBatch];
+    signed char tag[kSoloBatch];
+    unsigned char list[kSoloSorts][kSoloBatch];
+};
+
+// the whole routine (k_shape's)
+template <int WHAT>
+static __device__ __noinline__ double solo64(const ShapeRec64& r, double px, double py, double pz, double qx, double qy,
+                                             double qz, int* f) {
+    double x[3], u[3];
+    to_local64(r, px, py, pz, qx, qy, qz, x, u);
+    *f = -1;
+    if (WHAT == GEO_Q_DIST_OUT) return dist_out64<true, false>(r, x, u, f);
+    if (WHAT == GEO_Q_DIST_IN) return contains64<false>(r, x) ? dist_in64<true, false>(r, x, u, f) : 0.0;
+    if (WHAT == GEO_Q_CONTAINS) return contains64<false>(r, x) ? 1.0 : 0.0;
+    return safety64<false>(r, x, WHAT == GEO_Q_SAFETY_IN);
+}
+
+template <int WHAT>
+__global__ void __launch_bounds__(kSoloWarps * 32, 4) k_shape_lists(const __grid_constant__ ShapeFast a, Basket b,
+                                                                    double* __restrict__ out, int32_t* __restrict__ face,
+                                                                    int per) {
+    constexpr bool kDist = WHAT == GEO_Q_DIST_OUT || WHAT == GEO_Q_DIST_IN;
+    extern __shared__ __align__(128) unsigned char smem_raw[];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    SoloBatch& B = reinterpret_cast<SoloBatch*>(smem_raw)[warp];
+    const int64_t nbatch = (b.n + per - 1) / per;
+    const int64_t stride = int64_t(gridDim.x) * kSoloWarps;
+    for (int64_t q = int64_t(blockIdx.x) * kSoloWarps + warp; q < nbatch; q += stride) {
+        const int64_t first = q * per;
+        int cnt[kSoloSorts] = {0, 0, 0, 0};
+        for (int o = lane; o < per; o += 32) {
+            const int64_t i = first + o;
+            if (i - lane >= b.n) break;   // warp-uniform
+            int sort = -1, tag = 0;
+            if (i < b.n) {
+                const double px = b.x[i], py = b.y[i], pz = b.z[i];
+                double qx = 1.0, qy = 0.0, qz = 0.0;
+                if (kDist) {
+                    qx = b.dx[i]; qy = b.dy[i]; qz = b.dz[i];
+                }
+                Ray32 r;
+                r.p[0] = f64_to_f32_trunc(px); r.p[1] = f64_to_f32_trunc(py); r.p[2] = f64_to_f32_trunc(pz);
+                double v = 0.0;   // where no FP64 is needed
+                bool near = fmaxf(fabsf(r.p[0]), fmaxf(fabsf(r.p[1]), fabsf(r.p[2]))) <= a.reach;
+                if (!valid_track(px, py, pz, qx, qy, qz)) {
+                    v = d_nan();
+                } else {
+                    if (kDist) {
+                        r.d[0] = f64_to_f32_trunc(qx); r.d[1] = f64_to_f32_trunc(qy); r.d[2] = f64_to_f32_trunc(qz);
+                        const float dd = fmaf(r.d[0], r.d[0], fmaf(r.d[1], r.d[1], r.d[2] * r.d[2]));
+                        near = near && dd > 1e-30f && dd < 1e30f;
+                        const float inv_dd = frcp(dd);
+                        r.inv_dn = rsqrtf(dd) * (1.f + 4.f * kEps32f);
+#pragma unroll
+                        for (int k = 0; k < 3; ++k) r.e[k] = -r.d[k] * inv_dd;
+                    }
+                    if (!near) {
+                        sort = 3;
+                    } else if (WHAT == GEO_Q_CONTAINS) {
+                        const int in = entry_holds(&a.h, r.p);
+                        if (in == 2) sort = 3;
+                        else v = in ? 1.0 : 0.0;
+                    } else if (WHAT == GEO_Q_SAFETY_OUT) {
+                        tag = entry_zone(&a.h, r.p);
+                        if (tag != kZoneInside) sort = zone_sort(tag);
+                    } else if (WHAT == GEO_Q_DIST_OUT) {
+                        Cands c;
+                        cands_clear(c);
+                        if (a.h.flags & kFiltBox) bound_box(&a.h, r, f_inf(), c);
+                        else bound_quad(&a.h, r, f_inf(), c);
+                        if (!(c.L[0] < f_inf())) {
+                            v = d_inf();
+                        } else {
+                            tag = c.j[0] >> kTagShift;
+                            if (tag != kTagNone) sort = tag == kTagOuter || tag == kTagInner ? 1 : 0;
+                            else if (entry_holds(&a.h, r.p) != 1) sort = 3;   // (surely inside: 0)
+                        }
+                    } else {   // from inside: in the solid's own frame
+                        const float4* H = hvy_words(&a.h);
+                        float x[3];
+                        point_to_entry(H, H[0], a.h.flags, H[3].x, r.p, x);
+                        const bool surely = contains32(a.m32, x);
+                        if (surely && WHAT == GEO_Q_SAFETY_IN) {
+                            tag = mother_zone(a, x);
+                            sort = zone_sort(tag);
+                        } else if (surely) {
+                            float u[3];
+                            if (a.h.flags & kFiltIdentity) {
+                                u[0] = r.d[0]; u[1] = r.d[1]; u[2] = r.d[2];
+                            } else {
+                                rotate_in(H[1], H[2], H[3].x, r.d, u);
+                            }
+#pragma unroll
+                            for (int k = 0; k < 3; ++k) {
+                                r.p[k] = x[k];
+                                r.d[k] = u[k];
+                            }
+                            tag = mother_exit32(a, r).tag;
+                            sort = tag == kTagNone ? 3 : (tag == kTagOuter || tag == kTagInner ? 1 : 0);
+                        } else if (contains32(a.m32u, x)) {
+                            sort = 3;   // (surely outside: 0)
+                        }
+                    }
+                }
+                if (sort < 0) {
+                    out[i] = v;
+                    if (face) face[i] = -1;
+                } else {
+                    B.p[0][o] = px; B.p[1][o] = py; B.p[2][o] = pz;
+                    if (kDist) {
+                        B.p[3][o] = qx; B.p[4][o] = qy; B.p[5][o] = qz;
+                    }
+                    B.tag[o] = (signed char)tag;
+                    if (per <= 32 && sort < 3) sort = 0;   // (32 tracks are not worth several runs)
+                }
+            }
+#pragma unroll
+            for (int s = 0; s < kSoloSorts; ++s) {
+                const unsigned same = __ballot_sync(0xffffffffu, sort == s);
+                if (sort == s) B.list[s][cnt[s] + __popc(same & ((1u << lane) - 1u))] = (unsigned char)o;
+                cnt[s] += __popc(same);
+            }
+        }
+        __syncwarp();
+        for (int sort = 0, c = 0; sort < kSoloSorts;) {
+            const int n = sort == 0 ? cnt[0] : (sort == 1 ? cnt[1] : (sort == 2 ? cnt[2] : cnt[3]));
+            if (c >= n) {
+                ++sort;
+                c = 0;
+                continue;
+            }
+            if (c + lane < n) {
+                const int o = B.list[sort][c + lane], tag = B.tag[o];
+                const double px = B.p[0][o], py = B.p[1][o], pz = B.p[2][o];
+                const double qx = kDist ? B.p[3][o] : 0.0, qy = kDist ? B.p[4][o] : 0.0, qz = kDist ? B.p[5][o] : 0.0;
+                double v;
+                int f = -1;
+                if (sort == 3) {
+                    v = solo64<WHAT>(a.m64, px, py, pz, qx, qy, qz, &f);
+                } else if (kDist) {
+                    bool up = false;
+                    constexpr bool kExit = WHAT == GEO_Q_DIST_IN;
+                    v = surface64(a.m64, tag, kExit, px, py, pz, qx, qy, qz, &up);
+                    f = tag == kTagOuter ? 6 : (tag == kTagInner ? 7 : (tag >= kTagAxis ? 2 * (tag - kTagAxis) : 4) +
+                                                                           (up == kExit ? 1 : 0));
+                } else {
+                    v = zone64(a.m64, tag, WHAT == GEO_Q_SAFETY_IN, px, py, pz);
+                }
+                out[first + o] = v;
+                if (face) face[first + o] = f;
+            }
+            __syncwarp();
+            c += 32;
+        }
+        __syncwarp();
+    }
+}
+
+template <int WHAT>
+static cudaError_t launch_lists_q(const ShapeFast& a, const Basket& b, double* out, int32_t* face, cudaStream_t s,
+                                  int num_sms) {
+    // the basket spread over all resident warps, 32 to 128 tracks each
+    const int64_t warps = int64_t(4) * num_sms * kSoloWarps;
+    const int64_t share = (b.n + warps * 32 - 1) / (warps * 32) * 32;
+    const int per = int(share < kSoloBatch ? share : kSoloBatch);
+    const int smem = kSoloWarps * int(sizeof(SoloBatch));
+    cudaError_t e = prep(k_shape_lists<WHAT>, smem);
+    if (e != cudaSuccess) return e;
+    k_shape_lists<WHAT><<<blocks_for(k_shape_lists<WHAT>, b.n, smem, num_sms), kSoloWarps * 32, smem, s>>>(a, b, out, face,
+                                                                                                         per);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_shape_lists(const ShapeFast& a, int what, const Basket& b, double* out, int32_t* face,
+                               cudaStream_t s, int num_sms) {
+    switch (what) {
+        case GEO_Q_DIST_OUT: return launch_lists_q<GEO_Q_DIST_OUT>(a, b, out, face, s, num_sms);
+        case GEO_Q_DIST_IN: return launch_lists_q<GEO_Q_DIST_IN>(a, b, out, face, s, num_sms);
+        case GEO_Q_SAFETY_OUT: return launch_lists_q<GEO_Q_SAFETY_OUT>(a, b, out, face, s, num_sms);
+        case GEO_Q_SAFETY_IN: return launch_lists_q<GEO_Q_SAFETY_IN>(a, b, out, face, s, num_sms);
+        case GEO_Q_CONTAINS: return launch_lists_q<GEO_Q_CONTAINS>(a, b, out, face, s, num_sms);
+        default: return cudaErrorInvalidValue;
     }
 }
 

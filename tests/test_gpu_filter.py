@@ -187,3 +187,51 @@ def test_world_states_equal_fp64_bitwise(g, n):
         if rng.random() < 0.5:   # scattered: another direction from the boundary
             t = t[:3] + [torch.from_numpy(f).cuda() for f in scenes.isotropic(rng, n)]
         node = node2
+
+
+@pytest.mark.parametrize("n", [1, 33, 4099, 200003, 700001])
+@pytest.mark.parametrize("kind,prm", [(scenes.BOX, (3.0, 20.0, 11.0)), (scenes.TUBE, (0.0, 9.0, 14.0)),
+                                      (scenes.TUBE, (8.9, 9.0, 4.0)), (scenes.CONE, (5.0, 1.0, 30.0, 20.0, 21.0)),
+                                      (scenes.CONE, (30.0, 2.0, 4.0, 9.0, 9.0))])
+def test_solid_queries_equal_fp64_bitwise(g, kind, prm, n):
+    """One solid's queries against the FP64 kernels of a volume that holds it
+    (DistFromOutside) or is it (the others): points near and far beyond the
+    reach of its FP32 copies, on its rims and corners and a little beside
+    them; 32, 64 and 128 points a warp."""
+    rng = np.random.default_rng(n)
+    rot, t = scenes.haar_rotation(rng), np.array([7.0, -3.0, 5.0])
+    size = max(prm)
+    p = rng.uniform(-2.0, 2.0, (n, 3)) * size * np.where(rng.random((n, 1)) < 0.1, 30.0, 1.0)
+    m = n // 2
+    if kind == scenes.BOX:
+        q = np.array(prm) * rng.choice([-1.0, 1.0, 0.4], (m, 3))
+    else:
+        e, ph = rng.choice([-1.0, 1.0], m), rng.uniform(0.0, 2.0 * np.pi, m)
+        ends = (prm[0], prm[1], prm[0], prm[1], prm[2]) if kind == scenes.TUBE else (*prm[1:], prm[0])
+        lo, hi = rng.integers(2, size=m), e > 0
+        r = np.where(hi, np.where(lo, ends[2], ends[3]), np.where(lo, ends[0], ends[1]))
+        q = np.stack([r * np.cos(ph), r * np.sin(ph), e * ends[4]], axis=1)
+    p[:m] = q * (1.0 + rng.choice([0.0, 1e-8, 1e-6, 1e-4], (m, 1)) * rng.uniform(-1.0, 1.0, (m, 3)))
+    d = np.stack(scenes.isotropic(rng, n), axis=1)
+    p -= d * rng.uniform(0.0, 3.0, (n, 1)) * size * rng.integers(0, 2, (n, 1))
+
+    def cuda(a):
+        return [torch.from_numpy(np.ascontiguousarray(a[:, k])).cuda() for k in range(3)]
+
+    R = rot.reshape(3, 3)
+    placed = cuda(p @ R.T + t) + cuda(d @ R.T)
+    hall = g.geo_build_volume(scenes._scene("hall", scenes.BOX, (1e4, 1e4, 1e4), [(kind, prm, rot, t)]))
+    step, hit = g.geo_dist_to_boundary(hall, *placed, mode=g.GEO_FP64)
+    out, face = g.geo_shape_query(kind, prm, g.GEO_Q_DIST_OUT, *placed, rot=rot, trans=t, want_face=True)
+    assert torch.equal(torch.where(hit == 0, step, torch.inf).view(torch.int64), out.view(torch.int64))
+    assert torch.equal((face >= 0), (hit == 0) & (step > 0))
+    own = cuda(p) + cuda(d)
+    solid = g.geo_build_volume(scenes.leaf(kind, prm))
+    inside = g.geo_contains(solid, *own[:3], mode=g.GEO_FP64) == -1
+    assert torch.equal(g.geo_shape_query(kind, prm, g.GEO_Q_CONTAINS, *own[:3]) == 1.0, inside)
+    step, _ = g.geo_dist_to_boundary(solid, *own, mode=g.GEO_FP64)
+    out, face = g.geo_shape_query(kind, prm, g.GEO_Q_DIST_IN, *own, want_face=True)
+    assert torch.equal(step.view(torch.int64), out.view(torch.int64))
+    assert torch.equal(face >= 0, inside)
+    saf = g.geo_shape_query(kind, prm, g.GEO_Q_SAFETY_IN, *own[:3])
+    assert torch.equal(g.geo_safety(solid, *own[:3], mode=g.GEO_FP64).view(torch.int64), saf.view(torch.int64))
