@@ -376,6 +376,53 @@ bool make_rec32(const geo_placed_shape& s, double grow, double delta, ShapeRec32
 
 bool needs_segs_code(const geo_placed_shape& s);
 
+// The plain FP64 step's cull table in the filter's order (`hvy`: its entries).
+std::vector<Cull64> make_cull(const geo_placed_shape* in, const std::vector<ShapeRec64>& d,
+                              const std::vector<FiltHvy>& hvy, int32_t nq1) {
+    std::vector<Cull64> out(hvy.size());
+    for (size_t k = 0; k < hvy.size(); ++k) {
+        Cull64& c = out[k];
+        std::memset(&c, 0, sizeof c);
+        const bool annulus = int(k) < nq1;
+        c.id = hvy[k].brad > 0.f ? hvy[k].id : -1;
+        c.axis = 1;
+        if (c.id < 0) {   // no track meets it
+            c.a = -1.0;
+            continue;
+        }
+        const ShapeRec64& r = d[size_t(c.id)];
+        const geo_placed_shape& s = in[c.id];
+        for (int q = 0; q < 3; ++q) c.t[q] = r.t[q];
+        c.a = r.brad * r.brad * (1.0 + 1e-12);
+        c.b = r.brad;
+        if (!annulus) continue;
+        double hi, lo, h;   // of the solid, or the tube that holds a segment or polycone
+        if (s.kind == GEO_CONE) {
+            hi = std::max(s.p[2], s.p[4]);
+            lo = std::min(s.p[1], s.p[3]);
+            h = s.p[0];
+        } else if (s.kind == GEO_PCON) {
+            const geo_placed_shape t = bounding_tube(s, false);
+            hi = t.p[1];
+            lo = t.p[0];
+            h = t.p[2];
+            for (int q = 0; q < 3; ++q) c.t[q] = t.trans[q];
+        } else {
+            hi = s.p[1];
+            lo = s.p[0];
+            h = s.p[2];
+        }
+        // enlarged as brad is: the cull's own FP64 rounding, relative to the
+        // distances a track covers, stays far below
+        const double grow = 1e-9 + 1e-12 * (r.brad + std::fabs(c.t[0]) + std::fabs(c.t[1]) + std::fabs(c.t[2]));
+        c.a = hi + grow;
+        c.b = lo - grow;
+        c.h = h + grow;
+        c.axis = k % 32 == 0 || c.t[0] != out[k - 1].t[0] || c.t[1] != out[k - 1].t[1] ? 1 : 0;
+    }
+    return out;
+}
+
 // The filter's tables (layout in geo_internal.h) from the daughters `in` and
 // their FP32 copies: sorted by class, the daughters of a class in index order.
 void make_filter(const geo_placed_shape* in, const std::vector<ShapeRec32>& d, std::vector<FiltSph>& sph,
@@ -809,8 +856,10 @@ geo_status geo_build_volume(const geo_placed_shape* mother, const geo_placed_sha
     // the FP32 records, then the filter's two tables
     const size_t b32 = sizeof(ShapeRec32) * size_t(std::max(n_daughters, 1));
     vw.nf = int32_t(hsph.size());
+    const std::vector<Cull64> hcull = make_cull(daughters, h64, hhvy, vw.nq1);
     const size_t bsph = sizeof(FiltSph) * hsph.size(), bhvy = sizeof(FiltHvy) * hhvy.size();
-    if ((e = lib_malloc(&v->d64, b64)) != cudaSuccess || (e = lib_malloc(&v->d32, b32 + bsph + bhvy)) != cudaSuccess ||
+    const size_t bcull = sizeof(Cull64) * hcull.size();
+    if ((e = lib_malloc(&v->d64, b64)) != cudaSuccess || (e = lib_malloc(&v->d32, b32 + bsph + bhvy + bcull)) != cudaSuccess ||
         (e = lib_malloc(&v->status, sizeof(unsigned int))) != cudaSuccess) {
         geo_destroy_volume(v);
         return cuda_status(e);
@@ -829,7 +878,9 @@ geo_status geo_build_volume(const geo_placed_shape* mother, const geo_placed_sha
             (e = cudaMemcpyAsync(reinterpret_cast<char*>(v->d32) + b32, hsph.data(), bsph, cudaMemcpyHostToDevice, s)) !=
                 cudaSuccess ||
             (e = cudaMemcpyAsync(reinterpret_cast<char*>(v->d32) + b32 + bsph, hhvy.data(), bhvy, cudaMemcpyHostToDevice,
-                                 s)) != cudaSuccess) {
+                                 s)) != cudaSuccess ||
+            (e = cudaMemcpyAsync(reinterpret_cast<char*>(v->d32) + b32 + bsph + bhvy, hcull.data(), bcull,
+                                 cudaMemcpyHostToDevice, s)) != cudaSuccess) {
             geo_destroy_volume(v);
             return cuda_status(e);
         }
@@ -843,6 +894,7 @@ geo_status geo_build_volume(const geo_placed_shape* mother, const geo_placed_sha
     vw.d32 = v->d32;
     vw.fsph = reinterpret_cast<const FiltSph*>(reinterpret_cast<char*>(v->d32) + b32);
     vw.fhvy = reinterpret_cast<const FiltHvy*>(reinterpret_cast<char*>(v->d32) + b32 + bsph);
+    vw.cull = reinterpret_cast<const Cull64*>(reinterpret_cast<char*>(v->d32) + b32 + bsph + bhvy);
     vw.status = v->status;
     v->h64 = std::move(h64);
     if (opts && opts->voxelize) {

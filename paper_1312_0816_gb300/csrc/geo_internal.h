@@ -125,6 +125,20 @@ struct __align__(16) FiltHvy {
 };
 static_assert(sizeof(FiltSph) == 32 && sizeof(FiltHvy) == 112, "filter table layout");
 
+// What the plain FP64 step needs of a daughter to pass it over, in the filter's
+// order and with its filling entries (id -1): its bounding sphere, enlarged as
+// brad is, or (unrotated whole tubes and cones) its bounding annulus, enlarged
+// alike.
+struct __align__(16) Cull64 {
+    double t[3];
+    double a;       // sphere: brad^2; annulus: Rmax
+    double b;       // sphere: brad;   annulus: Rmin
+    double h;       // annulus: half-length
+    int32_t id;
+    int32_t axis;   // annulus: 1 where its axis differs from the entry before or the index is a multiple of 32
+};
+static_assert(sizeof(Cull64) == 64, "Cull64 layout");
+
 // Everything a kernel needs about one volume, passed by value (or copied
 // from a device array of views by the batched kernel).
 struct __align__(16) VolView {
@@ -135,11 +149,12 @@ struct __align__(16) VolView {
     const ShapeRec32* d32;     // [nd] device
     const FiltSph* fsph;       // [nf] device, in the filter's order
     const FiltHvy* fhvy;       // [nf] device, likewise
+    const Cull64* cull;        // [nf] device, likewise
     int32_t nq1;               // unrotated quadrics of the filter's order
     int32_t nq;                // quadrics of the filter's order
     int32_t nf;                // entries of the filter's tables
     int32_t nd;
-    int32_t smem64;            // 1 if the FP64 table fits the shared-memory budget
+    int32_t smem64;            // 1 if the FP64 records fit the shared-memory budget
     int32_t smem_refine;       // tables the refine kernel stages: 0 none, 1 the filter's, 2 the FP64 records too
     // voxel grid (uniform over the mother's bounding box)
     int32_t voxelized;

@@ -3,32 +3,22 @@
 // minimum), and the navigator-level Contains and Safety of Sec. 3.1.
 //
 // One thread per track (grid-stride over the basket).  The basket is read as
-// coalesced FP64 structure-of-arrays.  The volume's FP64 daughter table is
-// staged once per block into shared memory with the bulk-copy engine and read
-// warp-uniformly (every lane of a warp visits daughter j together, so each
-// record field is a broadcast).  Per daughter: a bounding-sphere test against
-// the current best step, the master->local transform, DistFromOutside, and a
-// running (step, index) minimum with strict '<' (mother first, then lowest
-// index win ties).
+// coalesced FP64 structure-of-arrays.  Mother first, then the daughters that a
+// cull in FP64 does not exclude, a running (step, index) minimum (mother, then the
+// lowest index win ties).
 #include <cuda_runtime.h>
+
 #include "geo_internal.h"
+#include "launch.cuh"
 #include "nav_common.cuh"
 #include "shapes64.cuh"
 #include "stage.cuh"
-#include "launch.cuh"
 
 namespace geonav {
 
-template <bool SMEM>
-__global__ void __launch_bounds__(256) k_dist_fp64(VolView v, Basket b, double* __restrict__ step,
-                                                   int32_t* __restrict__ hit, double* __restrict__ bpoint) {
-    extern __shared__ __align__(128) unsigned char smem_raw[];
-    __shared__ uint64_t bar;
-    const ShapeRec64* tab = v.d64;
-    if (SMEM) {
-        if (!stage_table(smem_raw, v.d64, uint32_t(v.nd) * sizeof(ShapeRec64), &bar, v.status)) return;
-        tab = reinterpret_cast<const ShapeRec64*>(smem_raw);
-    }
+// Voxelised volumes: the grid's walk (nav_vox64).
+__global__ void __launch_bounds__(256) k_dist_vox64(VolView v, Basket b, double* __restrict__ step,
+                                                    int32_t* __restrict__ hit, double* __restrict__ bpoint) {
     const int64_t stride = int64_t(gridDim.x) * blockDim.x;
     for (int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < b.n; i += stride) {
         const double px = b.x[i], py = b.y[i], pz = b.z[i];
@@ -42,10 +32,208 @@ __global__ void __launch_bounds__(256) k_dist_fp64(VolView v, Basket b, double* 
         } else if (!contains64(v.m64, p)) {
             best = 0.0;
             h = -2;
-        } else if (v.voxelized) {
-            nav_vox64(v, tab, px, py, pz, qx, qy, qz, best, h);
         } else {
-            nav_all64(v.m64, tab, v.nd, px, py, pz, qx, qy, qz, best, h);
+            nav_vox64(v, v.d64, px, py, pz, qx, qy, qz, best, h);
+        }
+        store_result(i, b.n, best, h, px, py, pz, qx, qy, qz, step, hit, bpoint);
+    }
+}
+
+// tube_out64 and cone_out64 (no apex on an end plane) in one path, so that
+// lanes with either kind run it together: a tube is a cone of slope 0 whose
+// outer and inner C keep the rounded squares of its radii (surface64 in
+// nav_refine.cuh has the argument that the bits are the same).
+__device__ __forceinline__ double quad_out64(const ShapeRec64& r, const double* x, const double* u) {
+    const double* d = r.d;
+    const bool tube = r.kind == KTUBE;
+    const double dz = tube ? d[2] : d[0], bo = tube ? 0.0 : d[2], bi = tube ? 0.0 : d[4];
+    const double rho2 = rho2_of(x);
+    // -1 * R^2 (tube), -R * R (cone)
+    const double ro0 = tube ? 1.0 : FMA(bo, x[2], d[1]), ri0 = tube ? 1.0 : FMA(bi, x[2], d[3]);
+    const double ro1 = tube ? d[4] : ro0, ri1 = tube ? d[3] : ri0;
+    const bool hole = tube ? IS_POS(d[0]) : !IS_ZERO(d[11]);
+    if (ABS_LE(x[2], dz) && LE(rho2, MUL(ro0, ro1)) && (!hole || LE(MUL(ri0, ri1), rho2))) return 0.0;
+    double best = d_inf();
+    const bool zc = ABS_GT(x[2], dz) && OPPOSITE(x[2], u[2]);
+    if (zc) {   // the z-plane the track approaches from outside the slab
+        const double t = DIV(SUB(copysign(dz, x[2]), x[2]), u[2]);
+        const double xh = FMA(t, u[0], x[0]), yh = FMA(t, u[1], x[1]);
+        const double r2 = DOT2(xh, xh, yh, yh);
+        const double lo2 = tube ? d[3] : (IS_POS(x[2]) ? d[7] : d[5]);
+        const double hi2 = tube ? d[4] : (IS_POS(x[2]) ? d[8] : d[6]);
+        if (LE(r2, hi2) && LE(lo2, r2)) best = t;
+    }
+    const double A0 = DOT2(u[0], u[0], u[1], u[1]);
+    const double B0 = DOT2(x[0], u[0], x[1], u[1]);
+    {   // outer surface, crossed inwards
+        const double rs = MUL(bo, u[2]);
+        const double s = root_falling(FMA(-rs, rs, A0), FMA(-ro0, rs, B0), FMA(-ro0, ro1, rho2));
+        if (NONNEG(s) && LT(s, best) && ABS_LE(FMA(s, u[2], x[2]), dz)) best = s;
+    }
+    if (hole) {   // inner surface, crossed outwards (out of the hole)
+        const double rs = MUL(bi, u[2]);
+        const double s = root_rising(FMA(-rs, rs, A0), FMA(-ri0, rs, B0), FMA(-ri0, ri1, rho2));
+        if (NONNEG(s) && LT(s, best) && ABS_LE(FMA(s, u[2], x[2]), dz)) best = s;
+    }
+    return best;
+}
+
+template <bool SEGS>
+static __device__ __noinline__ void nav_all64_far(const ShapeRec64& m, const ShapeRec64* __restrict__ tab, int nd,
+                                                  double px, double py, double pz, double qx, double qy, double qz,
+                                                  double& best, int& h) {
+    nav_all64<SEGS>(m, tab, nd, px, py, pz, qx, qy, qz, best, h);
+}
+
+// Every daughter, all in FP64, in the filter's order (filter_pass.cuh has the
+// scheme and its reasons): culls for all lanes together -- bounding spheres,
+// and bounding annuli of unrotated tubes and cones -- then each lane its own
+// daughters, of the annuli the two that start nearest first.  The culls
+// compare on bit patterns, so an annulus costs 8 FP64 instructions and a
+// sphere 12.  `tab`: the FP64 records.
+template <bool SEGS>
+__device__ __forceinline__ void nav_lists64(const VolView& v, const Cull64* __restrict__ C,
+                                            const ShapeRec64* __restrict__ tab, double px, double py, double pz,
+                                            double qx, double qy, double qz, double& best, int& h) {
+    const double p[3] = {px, py, pz}, q[3] = {qx, qy, qz};
+    best = dist_in64<false, SEGS>(v.m64, p, q);
+    h = -1;
+    const double perp2 = DOT2(qx, qx, qy, qy), dd = FMA(qz, qz, perp2), dn = SQRT(dd);
+    if (!(LT(1e-200, dd) && LT(dd, 1e200))) {   // the culls' squares could leave the range of a double
+        nav_all64_far<SEGS>(v.m64, v.d64, v.nd, px, py, pz, qx, qy, qz, best, h);
+        return;
+    }
+    double inv_z = 0.0, inv_r = 0.0;
+    if (v.nq1 > 0) {
+        // lowered below any rounding of the products; no radial bound along the axis
+        constexpr double kLow = 1.0 - 0x1p-48;
+        inv_z = MUL(DIV(1.0, fabs(qz)), kLow);
+        inv_r = LT(MUL(dd, 1e-24), perp2) ? MUL(DIV(1.0, SQRT(perp2)), kLow) : 0.0;
+    }
+    auto eval = [&](int j) {
+        const ShapeRec64& r = tab[j];
+        double x[3], u[3];
+        to_local64(r, px, py, pz, qx, qy, qz, x, u);
+        double s;
+        if (!SEGS && r.kind != KBOX) s = quad_out64(r, x, u);
+        else s = dist_out64<false, SEGS>(r, x, u);
+        if (LT(s, best) || (BITS(s) == BITS(best) && h >= 0 && j < h)) {
+            best = s;
+            h = j;
+        }
+    };
+    double rho = 0.0, rr = 0.0;   // distance to the axis: the start's, the forward ray's least
+    auto to_axis = [&](const Cull64& c) {
+        const double wx = SUB(px, c.t[0]), wy = SUB(py, c.t[1]);
+        rho = SQRT(DOT2(wx, wx, wy, wy));
+        const double away = DOT2(wx, qx, wy, qy);
+        rr = NONNEG(away) ? rho : MUL(fabs(FMA(wx, qy, -MUL(wy, qx))), inv_r);
+    };
+    auto pos = [](double a) { return BITS(a) < 0 ? 0.0 : a; };   // max(a, 0)
+    // start of the annulus' part of the track, +inf when it is missed or starts beyond best
+    auto annulus = [&](const Cull64& c) {
+        const double wz = SUB(pz, c.t[2]), wzs = BITS(qz) < 0 ? -wz : wz;
+        const double t_in = pos(MUL(SUB(-c.h, wzs), inv_z)), t_out = MUL(SUB(c.h, wzs), inv_z);
+        const double t_r = MUL(MAXP(pos(SUB(rho, c.a)), pos(SUB(c.b, rho))), inv_r);
+        const double L = MAXP(t_in, t_r);
+        // (t_out is lowered like L: compared with a margin of its own)
+        const bool miss = BITS(t_out) < 0 || BITS(t_out) + (1LL << 8) < BITS(L) || LT(c.a, rr) || LT(best, L);
+        return miss ? d_inf() : L;
+    };
+    for (int base = 0; base < v.nf; base += 32) {
+        const Cull64* S = C + base;
+        const int cnt = min(32, v.nf - base), n1 = max(0, min(cnt, v.nq1 - base));
+        unsigned m = 0;
+        double l1 = d_inf(), l2 = d_inf();
+        int k1 = -1, k2 = -1, k = 0;
+        for (; k < n1; ++k) {
+            if (S[k].axis) to_axis(S[k]);   // warp-uniform: another axis than the solid before
+            const double L = annulus(S[k]);
+            if (!LT(L, d_inf())) continue;
+            m |= 1u << k;
+            if (LT(L, l1)) {
+                l2 = l1;
+                k2 = k1;
+                l1 = L;
+                k1 = k;
+            } else if (LT(L, l2)) {
+                l2 = L;
+                k2 = k;
+            }
+        }
+        for (; k < cnt; ++k) {
+            const double w0 = SUB(S[k].t[0], px), w1 = SUB(S[k].t[1], py), w2 = SUB(S[k].t[2], pz);
+            const double proj = FMA(w2, qz, FMA(w1, qy, MUL(w0, qx)));
+            const double ww = FMA(w2, w2, FMA(w1, w1, MUL(w0, w0)));
+            // squared distance of the line times dd against the radius' (a filling entry's is negative)
+            const double far2 = FMA(-proj, proj, MUL(ww, dd)), rb2 = MUL(S[k].a, dd);
+            if (BITS(rb2) < 0 || LT(rb2, pos(far2))) continue;
+            const double rb = MUL(S[k].b, dn);
+            if (BITS(ADD(proj, rb)) < 0 || LT(MUL(best, dd), pos(SUB(proj, rb)))) continue;   // behind, beyond
+            m |= 1u << k;
+        }
+        if (k1 >= 0) m &= ~(1u << k1);
+        if (k2 >= 0) m &= ~(1u << k2);
+        for (;;) {
+            int w = k1;
+            k1 = k2;
+            k2 = -1;
+            if (w >= 0 && LT(best, l1)) w = -1;
+            l1 = l2;
+            if (w < 0) {
+                if (k1 >= 0) continue;
+                if (!m) break;
+                w = __ffs(m) - 1;
+                m &= m - 1;
+                if (w < n1) {
+                    to_axis(S[w]);
+                    if (!LT(annulus(S[w]), d_inf())) continue;
+                }
+            }
+            eval(S[w].id);
+        }
+    }
+}
+
+// What bounds it: the FP64 unit (66 %; 1050 FP64 warp instructions per 32 tracks
+// of the toy detector, 2200 when the warp walked the daughters together).
+// 100003 tracks: 484 -> 242 us.  Blocks of 64 threads, eight per SM: the last
+// wave's imbalance costs least (128 x 5 259 us, 128 x 8 258, 32 x 20 238).
+constexpr int kFp64Threads = 64, kFp64Blocks = 8;
+constexpr int kFp64Tables = 24 * 1024;   // bytes staged per block
+
+// STAGED: 1 the cull table, 2 the FP64 records too
+template <int STAGED, bool SEGS>
+__global__ void __launch_bounds__(kFp64Threads, kFp64Blocks)
+    k_dist_fp64(const __grid_constant__ VolView v, Basket b, double* __restrict__ step, int32_t* __restrict__ hit,
+                double* __restrict__ bpoint) {
+    extern __shared__ __align__(128) unsigned char smem_raw[];
+    __shared__ uint64_t bar;
+    const Cull64* C = v.cull;
+    const ShapeRec64* tab = v.d64;
+    if (STAGED) {
+        const uint32_t bc = uint32_t(v.nf) * uint32_t(sizeof(Cull64));
+        if (!stage_tables(smem_raw, v.cull, bc, smem_raw + bc, v.d64,
+                          STAGED == 2 ? uint32_t(v.nd) * uint32_t(sizeof(ShapeRec64)) : 0, &bar, v.status))
+            return;
+        C = reinterpret_cast<const Cull64*>(smem_raw);
+        if (STAGED == 2) tab = reinterpret_cast<const ShapeRec64*>(smem_raw + bc);
+    }
+    const int64_t stride = int64_t(gridDim.x) * kFp64Threads;
+    for (int64_t i = int64_t(blockIdx.x) * kFp64Threads + threadIdx.x; i < b.n; i += stride) {
+        const double px = b.x[i], py = b.y[i], pz = b.z[i];
+        const double qx = b.dx[i], qy = b.dy[i], qz = b.dz[i];
+        double best;
+        int h;
+        const double p[3] = {px, py, pz};
+        if (!valid_track(px, py, pz, qx, qy, qz)) {
+            best = d_nan();
+            h = -2;
+        } else if (!contains64<SEGS>(v.m64, p)) {
+            best = 0.0;
+            h = -2;
+        } else {
+            nav_lists64<SEGS>(v, C, tab, px, py, pz, qx, qy, qz, best, h);
         }
         store_result(i, b.n, best, h, px, py, pz, qx, qy, qz, step, hit, bpoint);
     }
@@ -219,10 +407,34 @@ cudaError_t launch_dist_warp(const VolView& v, const Basket& b, double* step, in
     return cudaGetLastError();
 }
 
+template <int STAGED, bool SEGS>
+static cudaError_t launch_fp64(const VolView& v, const Basket& b, double* step, int32_t* hit, double* bpoint, int smem,
+                               cudaStream_t s, int num_sms) {
+    cudaError_t e = prep(k_dist_fp64<STAGED, SEGS>, smem);
+    if (e != cudaSuccess) return e;
+    k_dist_fp64<STAGED, SEGS><<<blocks_for(k_dist_fp64<STAGED, SEGS>, b.n, smem, num_sms, kFp64Threads), kFp64Threads, smem,
+                                s>>>(v, b, step, hit, bpoint);
+    return cudaGetLastError();
+}
+
 cudaError_t launch_dist_fp64(const VolView& v, const Basket& b, double* step, int32_t* hit, double* bpoint,
                              cudaStream_t s, int num_sms) {
     if (small_basket(v, b.n, num_sms)) return launch_dist_warp(v, b, step, hit, bpoint, s, num_sms);
-    GEO_LAUNCH(k_dist_fp64, v, b, step, hit, bpoint);
+    if (v.voxelized) {
+        k_dist_vox64<<<blocks_for(k_dist_vox64, b.n, 0, num_sms), 256, 0, s>>>(v, b, step, hit, bpoint);
+        return cudaGetLastError();
+    }
+    const int64_t bc = int64_t(v.nf) * int64_t(sizeof(Cull64)), br = bc + int64_t(v.nd) * int64_t(sizeof(ShapeRec64));
+    const int staged = br <= kFp64Tables ? 2 : (bc <= kFp64Tables ? 1 : 0);
+    const int smem = staged == 2 ? int(br) : (staged == 1 ? int(bc) : 0);
+    switch (2 * staged + (v.segs ? 1 : 0)) {
+        case 0: return launch_fp64<0, false>(v, b, step, hit, bpoint, smem, s, num_sms);
+        case 1: return launch_fp64<0, true>(v, b, step, hit, bpoint, smem, s, num_sms);
+        case 2: return launch_fp64<1, false>(v, b, step, hit, bpoint, smem, s, num_sms);
+        case 3: return launch_fp64<1, true>(v, b, step, hit, bpoint, smem, s, num_sms);
+        case 4: return launch_fp64<2, false>(v, b, step, hit, bpoint, smem, s, num_sms);
+        default: return launch_fp64<2, true>(v, b, step, hit, bpoint, smem, s, num_sms);
+    }
 }
 
 cudaError_t launch_contains(const VolView& v, const Basket& b, int32_t* where, int mode, cudaStream_t s,

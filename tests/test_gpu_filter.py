@@ -130,6 +130,21 @@ def test_grid_equals_fp64_bitwise(g, counts, grid):
     assert g.geo_check_device_status(vol) == 0
 
 
+@pytest.mark.parametrize("mother,apex", [("box", False), ("tube", False), ("box", True)])
+@pytest.mark.parametrize("counts", COUNTS)
+def test_fp64_lists_equal_the_single_cell_walk(g, counts, mother, apex):
+    """The FP64 step's culls and lists per lane against a grid of one cell, whose
+    walk looks at every daughter with the shapes' own functions."""
+    sc = filter_scene(*counts, mother, seed=sum(counts) + 7, apex=apex)
+    flat, walk = g.geo_build_volume(sc), g.geo_build_volume(sc, voxelize=True, grid=(1, 1, 1))
+    for n in (63, 5003, 70001):
+        t = tracks(sc, n, n)
+        s0, h0 = g.geo_dist_to_boundary(walk, *t, mode=g.GEO_FP64)
+        s1, h1 = g.geo_dist_to_boundary(flat, *t, mode=g.GEO_FP64)
+        assert torch.equal(h0, h1)
+        assert torch.equal(s0.view(torch.int64), s1.view(torch.int64))
+
+
 @pytest.mark.parametrize("mother", ["box", "tube"])
 @pytest.mark.parametrize("counts", COUNTS)
 def test_point_queries_equal_fp64_bitwise(g, counts, mother):
