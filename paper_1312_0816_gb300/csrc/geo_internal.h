@@ -225,6 +225,8 @@ cudaError_t launch_dist_refine_split(const VolView& v, const Basket& b, double* 
                                      int32_t* nref, cudaStream_t s);
 
 // one thread per track (volumes without segments and polycones)
+cudaError_t launch_dist_grid(const VolView& v, const Basket& b, double* step, int32_t* hit, double* bpoint, int32_t* nref,
+                             cudaStream_t s, int num_sms);
 cudaError_t launch_dist_direct(const VolView& v, const Basket& b, double* step, int32_t* hit, double* bpoint,
                                int32_t* nref, cudaStream_t s, int num_sms);
 
@@ -240,6 +242,8 @@ cudaError_t launch_dist_warp(const VolView& v, const Basket& b, double* step, in
                              cudaStream_t s, int num_sms);
 cudaError_t launch_dist_refine_stats(const VolView& v, const Basket& b, double* step, int32_t* hit,
                                      double* bpoint, int32_t* nref, cudaStream_t s, int num_sms);
+cudaError_t launch_batched_direct(const BatchView& bv, const Basket& b, double* step, int32_t* hit, int blocks_per_sm,
+                                  int tile_tracks, cudaStream_t s, int num_sms);
 cudaError_t launch_dist_batched(const BatchView& bv, const Basket& b, double* step, int32_t* hit,
                                 int blocks_per_sm, int tile_tracks, cudaStream_t s, int num_sms);
 cudaError_t launch_contains(const VolView& v, const Basket& b, int32_t* where, int mode, cudaStream_t s,

@@ -78,85 +78,6 @@ __global__ void __launch_bounds__(kDirect, kDirectBlocks)
     }
 }
 
-// The same with the uniform grid.  STAGED: the grid's short form and the
-// filter's records in shared memory, one block of kGridStaged threads per SM
-// (the tables are staged once per SM); otherwise they are read through L1, by
-// blocks of kDirect threads.
-//
-// What bounds it: the FP64 unit (67 %) and issue slots (78 %); 5200 warp
-// instructions per 32 tracks with 8.5 of 32 lanes active, since a warp walks as
-// long as its longest track (22 cells, the mean is 7).  512 daughters, 2^22
-// tracks: 1745 us with the walk to the mother's exit in the pipelined kernel,
-// 754 us here (896 threads per block 776, 768 at 80 registers 875 with an earlier
-// form of the walk that took 829 with 1024).
-constexpr int kGridStaged = 1024;
-
-template <bool STAGED, int T>
-__global__ void __launch_bounds__(T, STAGED ? 1 : kDirectBlocks)
-    k_dist_grid(const __grid_constant__ VolView v, Basket b, double* __restrict__ step, int32_t* __restrict__ hit,
-                double* __restrict__ bpoint, int32_t* __restrict__ nref) {
-    extern __shared__ __align__(128) unsigned char smem_raw[];
-    __shared__ uint64_t bar;
-    __shared__ ShapeRec64 m64;
-    double(*pd)[T] = reinterpret_cast<double(*)[T]>(smem_raw);   // each thread's track
-    GridTab g = grid_lists(v);
-    const int t = threadIdx.x;
-    if (t < int(sizeof(ShapeRec64) / sizeof(double)))
-        reinterpret_cast<double*>(&m64)[t] = reinterpret_cast<const double*>(&v.m64)[t];
-    if (STAGED) {
-        unsigned char* tab = smem_raw + 6 * sizeof(double) * T;
-        const uint32_t bh = uint32_t(v.nf) * uint32_t(sizeof(FiltHvy));
-        if (!stage_tables(tab, v.fhvy, bh, tab + bh, v.vox_small, v.vox_small_bytes, &bar, v.status)) return;
-        g.hvy = reinterpret_cast<const FiltHvy*>(tab);
-        g.cells = reinterpret_cast<const uint32_t*>(tab + bh);
-        g.ids16 = reinterpret_cast<const uint16_t*>(tab + bh + v.vox_small_cells);
-    }
-    __syncthreads();
-    const int64_t stride = int64_t(gridDim.x) * T;
-    for (int64_t i = int64_t(blockIdx.x) * T + t; i < b.n; i += stride) {
-        RefineState rs;
-        double best = 0.0;
-        int h = -2, nev = 0;
-        {
-            const double px = b.x[i], py = b.y[i], pz = b.z[i];
-            const double qx = b.dx[i], qy = b.dy[i], qz = b.dz[i];
-            pd[0][t] = px; pd[1][t] = py; pd[2][t] = pz;
-            pd[3][t] = qx; pd[4][t] = qy; pd[5][t] = qz;
-            asm volatile("" ::: "memory");   // read again below
-            refine_pass1<STAGED ? kTravGridSmall : kTravGrid, false>(v, FiltTab{}, g, v.d64, px, py, pz, qx, qy, qz,
-                                                                     [&](int c) { return pd[c][t]; }, rs, best, h, nev);
-        }
-        const double px = pd[0][t], py = pd[1][t], pz = pd[2][t], qx = pd[3][t], qy = pd[4][t], qz = pd[5][t];
-        finish_direct(v, v.d64, m64, rs, px, py, pz, qx, qy, qz, best, h, nev);
-        store_result(i, b.n, best, h, px, py, pz, qx, qy, qz, step, hit, bpoint);
-        if (nref) nref[i] = nev;
-    }
-}
-
-template <bool STAGED, int T>
-static cudaError_t launch_grid(const VolView& v, const Basket& b, double* step, int32_t* hit, double* bpoint,
-                               int32_t* nref, int smem, cudaStream_t s, int num_sms) {
-    auto kernel = k_dist_grid<STAGED, T>;
-    cudaError_t e = prep(kernel, smem);
-    if (e != cudaSuccess) return e;
-    kernel<<<blocks_for(kernel, b.n, smem, num_sms, T), T, smem, s>>>(v, b, step, hit, bpoint, nref);
-    return cudaGetLastError();
-}
-
-// Staged from one full wave of tracks on: per call, staged against read
-// through L1, 65536 tracks 47.5 / 35.6 us, 155648 (a wave) 49.1 / 49.7, 2^20
-// 222 / 250.
-static cudaError_t launch_dist_grid(const VolView& v, const Basket& b, double* step, int32_t* hit, double* bpoint,
-                                    int32_t* nref, cudaStream_t s, int num_sms) {
-    const int64_t staged = int64_t(6 * sizeof(double)) * kGridStaged + int64_t(v.nf) * int64_t(sizeof(FiltHvy)) +
-                           int64_t(v.vox_small_bytes);
-    int dev = 0, most = 0;
-    if (v.vox_small && b.n >= int64_t(num_sms) * kGridStaged && cudaGetDevice(&dev) == cudaSuccess &&
-        cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) == cudaSuccess && staged + 1024 <= most)
-        return launch_grid<true, kGridStaged>(v, b, step, hit, bpoint, nref, int(staged), s, num_sms);
-    return launch_grid<false, kDirect>(v, b, step, hit, bpoint, nref, int(6 * sizeof(double)) * kDirect, s, num_sms);
-}
-
 template <int SMEM>
 static cudaError_t launch_direct(const VolView& v, const Basket& b, double* step, int32_t* hit, double* bpoint,
                                  int32_t* nref, cudaStream_t s, int num_sms) {
