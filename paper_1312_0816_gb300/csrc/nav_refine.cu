@@ -30,7 +30,8 @@ namespace geonav {
 size_t refine_stage_bytes() { return 2 * (sizeof(Stage<kProd>) + sizeof(Answers<kProd>)); }
 
 // ---------------------------------------------------------------------------
-// Batched persistent launch: tiles of many logical volumes, claimed in order
+// Batched persistent launch of volumes with a tube segment, a polycone or a cone
+// with an apex among them: tiles of many logical volumes, claimed in order
 // from a device counter (largest estimated cost first when the host sorted
 // them so), with the same producer / consumer pipeline.  The tile header of a
 // stage carries a copy of the tile's volume view.  The filter's tables of a
@@ -64,14 +65,13 @@ struct NextTile {
     const void* src;
 };
 
-// SEGS = false: no volume of the batch holds a tube segment or a polycone.
 // GLOB = false: no volume has a uniform grid and every volume's filter tables
 // fit the table area (`room` bytes); the kernel carries only the all-daughter
 // FP32 pass over staged tables (10 % faster on the 64-volume batch than with
 // the grid walk's code beside it).  GLOB = true: the tables are read from
 // global memory, a volume's grid is walked where it has one.  P producer
 // threads (one track each of a tile of P) and C consumer threads.
-template <bool SEGS, bool GLOB, int P, int C>
+template <bool GLOB, int P, int C>
 __global__ void __launch_bounds__(P + C, 2) k_dist_batched(BatchView bv, Basket b, double* __restrict__ step,
                                                               int32_t* __restrict__ hit, uint32_t room) {
     extern __shared__ __align__(128) unsigned char smem_raw[];
@@ -192,12 +192,12 @@ __global__ void __launch_bounds__(P + C, 2) k_dist_batched(BatchView bv, Basket 
                 int h = -2, nev = 0;
                 rs.status = 1;
                 if (live)
-                    refine_pass1<GLOB ? kTravEither : kTravAll, SEGS>(v, f, GridTab{}, v.d64, px, py, pz, qx, qy, qz,
-                                                                      [&](int c) { return st_.pd[c][t]; }, rs, best, h, nev);
+                    refine_pass1<GLOB ? kTravEither : kTravAll>(v, f, GridTab{}, v.d64, px, py, pz, qx, qy, qz,
+                                                                [&](int c) { return st_.pd[c][t]; }, rs, best, h, nev);
                 int task = 0, bin = -1;
                 if (rs.status == 0) {
                     task = first_task(rs);
-                    bin = task_bin<SEGS || GLOB>(rs.tag, task, v.d64);
+                    bin = task_bin<true>(rs.tag, task, v.d64);
                 }
                 const int slot = bin >= 0 ? atomicAdd(&st_.cnt[bin], 1) : 0;
                 producer_barrier<P>();
@@ -235,7 +235,7 @@ __global__ void __launch_bounds__(P + C, 2) k_dist_batched(BatchView bv, Basket 
             const int64_t* idx = bv.idx;
             // the outputs are in device memory: each track is stored as it is
             // finished (staging the tile's answers was 4 % slower here)
-            drain_tasks<SEGS, P, false>(v, v.d64, v.m64, st_, nullptr, [=](int o) { return packed ? idx[base + o] : base + o; },
+            drain_tasks<true, P, false>(v, v.d64, v.m64, st_, nullptr, [=](int o) { return packed ? idx[base + o] : base + o; },
                                         b.n, step, hit);
             __syncwarp();
             if (lane == 0) mbar_arrive(&done[k & 1]);
@@ -292,16 +292,16 @@ static uint32_t table_room(int max_nf) {
     return uint32_t(std::max<int64_t>(std::min(2 * one, avail) & ~int64_t(15), 16));
 }
 
-template <bool SEGS, bool GLOB, int P, int C>
+template <bool GLOB, int P, int C>
 static cudaError_t launch_batched(const BatchView& bv, const Basket& b, double* step, int32_t* hit, int blocks_per_sm,
                                   uint32_t room, cudaStream_t s, int num_sms) {
     const int smem = 2 * int(sizeof(Stage<P>) + sizeof(TileHdr)) + (GLOB ? 0 : int(room));
     cudaError_t e =
-        cudaFuncSetAttribute(k_dist_batched<SEGS, GLOB, P, C>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        cudaFuncSetAttribute(k_dist_batched<GLOB, P, C>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
-    const int maxb = resident_blocks(reinterpret_cast<const void*>(k_dist_batched<SEGS, GLOB, P, C>), P + C, smem);
+    const int maxb = resident_blocks(reinterpret_cast<const void*>(k_dist_batched<GLOB, P, C>), P + C, smem);
     const int per_sm = (blocks_per_sm <= 0 || blocks_per_sm > maxb) ? maxb : blocks_per_sm;
-    k_dist_batched<SEGS, GLOB, P, C><<<per_sm * num_sms, P + C, smem, s>>>(bv, b, step, hit, room);
+    k_dist_batched<GLOB, P, C><<<per_sm * num_sms, P + C, smem, s>>>(bv, b, step, hit, room);
     return cudaGetLastError();
 }
 
@@ -309,18 +309,17 @@ template <int P, int C>
 static cudaError_t launch_batched_shape(const BatchView& bv, const Basket& b, double* step, int32_t* hit,
                                         int blocks_per_sm, cudaStream_t s, int num_sms) {
     const uint32_t room = bv.vox ? 0 : table_room<P>(bv.max_nf);
-    if (room == 0)
-        return bv.segs ? launch_batched<true, true, P, C>(bv, b, step, hit, blocks_per_sm, room, s, num_sms)
-                       : launch_batched<false, true, P, C>(bv, b, step, hit, blocks_per_sm, room, s, num_sms);
-    return bv.segs ? launch_batched<true, false, P, C>(bv, b, step, hit, blocks_per_sm, room, s, num_sms)
-                   : launch_batched<false, false, P, C>(bv, b, step, hit, blocks_per_sm, room, s, num_sms);
+    return room == 0 ? launch_batched<true, P, C>(bv, b, step, hit, blocks_per_sm, room, s, num_sms)
+                     : launch_batched<false, P, C>(bv, b, step, hit, blocks_per_sm, room, s, num_sms);
 }
 
-// Two tile shapes, the autotuner's choice per batch: tiles of kTileTracks =
+// Volumes of boxes, tubes and cones take the kernel without producers and
+// consumers (nav_batched_direct.cu).  For the others two tile shapes, the autotuner's choice per batch: tiles of kTileTracks =
 // 384 tracks with 12 producer + 4 consumer warps, or tiles of 256 with 8 + 4.
 cudaError_t launch_dist_batched(const BatchView& bv, const Basket& b, double* step, int32_t* hit, int blocks_per_sm,
                                 int tile_tracks, cudaStream_t s, int num_sms) {
     static_assert(sizeof(TileHdr) % 16 == 0 && sizeof(VolView) % 16 == 0, "16-byte copies");
+    if (!bv.segs) return launch_batched_direct(bv, b, step, hit, blocks_per_sm, tile_tracks, s, num_sms);
     if (tile_tracks == kLatProd)
         return launch_batched_shape<kLatProd, kLatCons>(bv, b, step, hit, blocks_per_sm, s, num_sms);
     return launch_batched_shape<kProd, kCons>(bv, b, step, hit, blocks_per_sm, s, num_sms);

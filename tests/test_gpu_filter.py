@@ -93,14 +93,14 @@ def test_filter_equals_fp64_bitwise(g, counts, mother, apex):
     assert g.geo_check_device_status(vol) == 0
 
 
+@pytest.mark.parametrize("n", [60013, 600011, 1200007])
 @pytest.mark.parametrize("which", [(1, 4, 10), (0, 11, 9, 10)])
-def test_batched_filter_equals_fp64_bitwise(g, which):
-    """Volumes whose tables fit side by side in the batch's table area, and
-    volumes that only fit one after the other or not at all."""
+def test_batched_filter_equals_fp64_bitwise(g, which, n):
+    """Small and large volumes, in baskets from 17 tracks to a third of the
+    batch; sizes at which a warp takes 32, 64 and 128 tracks of a tile at a time."""
     vols = [g.geo_build_volume(filter_scene(*COUNTS[w], "box", seed=100 + w)) for w in which]
-    n = 60013
     t = tracks(None, n, 5)
-    cuts = [0, 17, 400, 20000, 20384, 45000, n]
+    cuts = [0, 17, 400, n // 3, n // 3 + 384, 3 * n // 4, n]
     rows = [(k % len(vols), a, b - a) for k, (a, b) in enumerate(zip(cuts, cuts[1:]))]
     for tile in (384, 256):
         batch = g.geo_build_batch(vols, rows, tile_tracks=tile)
@@ -116,12 +116,12 @@ def test_batched_filter_equals_fp64_bitwise(g, which):
 @pytest.mark.parametrize("grid", [(0, 0, 0), (1, 1, 1), (7, 3, 40)])
 @pytest.mark.parametrize("counts", [(1, 1, 1), (34, 31, 1), (0, 150, 130)])
 def test_grid_equals_fp64_bitwise(g, counts, grid):
-    """The grid's walk over the lists in global memory (one wave of tracks or
-    less) and over the short form staged in shared memory (beyond)."""
+    """The grid's walk with one thread per track (up to 1.25 waves of tracks), and
+    with a warp's tracks sorted for FP64, over the staged short form (beyond)."""
     sc = filter_scene(*counts, "box", seed=sum(counts) + 7)
     vol = g.geo_build_volume(sc, voxelize=True, grid=grid)
     wave = 1024 * torch.cuda.get_device_properties(0).multi_processor_count
-    for n in (30011, wave - 1, wave, wave + 333):
+    for n in (30011, wave * 5 // 4 - 1, wave * 5 // 4, wave * 4 + 333):
         t = tracks(sc, n, n)
         s0, h0 = g.geo_dist_to_boundary(vol, *t, mode=g.GEO_FP64)
         s1, h1 = g.geo_dist_to_boundary(vol, *t, mode=g.GEO_FP32_REFINE)
