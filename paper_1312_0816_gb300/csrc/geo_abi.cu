@@ -1023,7 +1023,7 @@ geo_status geo_dist_to_boundary_host(geo_volume v, const double* x, const double
         // kernel's loads and stores cross the host link; no staging copies)
         const Basket b{static_cast<const double*>(mp[0]), static_cast<const double*>(mp[1]),
                        static_cast<const double*>(mp[2]), static_cast<const double*>(mp[3]),
-                       static_cast<const double*>(mp[4]), static_cast<const double*>(mp[5]), n};
+                       static_cast<const double*>(mp[4]), static_cast<const double*>(mp[5]), n, 1};
         double* ostep = const_cast<double*>(static_cast<const double*>(mp[6]));
         int32_t* ohit = const_cast<int32_t*>(static_cast<const int32_t*>(mp[7]));
         e = (mode == GEO_FP64) ? launch_dist_fp64(v->view, b, ostep, ohit, nullptr, s, sms)

@@ -180,6 +180,7 @@ struct __align__(16) VolView {
 struct Basket {
     const double *x, *y, *z, *dx, *dy, *dz;
     int64_t n;
+    int64_t link = 0;   // 1: the arrays are host memory, so that each is best read once and stored in order
 };
 
 // One tile of the batched launch: up to kTileTracks consecutive tracks of one

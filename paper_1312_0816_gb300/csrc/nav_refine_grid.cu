@@ -102,10 +102,11 @@ static cudaError_t launch_sheets(const VolView& v, const Basket& b, double* step
 
 // k_grid_sheets from 1.25 waves of its tracks on, with the tables in shared memory
 // if they fit (us, k_dist_grid against it: 155648 tracks, a wave, 48.8 / 60.6, 200000
-// 73.9 / 65.7, 311000 85.4 / 87.6, 500000 133 / 125, 2^20 244 / 210).
+// 73.9 / 65.7, 311000 85.4 / 87.6, 500000 133 / 125, 2^20 244 / 210).  Not over
+// host memory: it reads a track twice.
 cudaError_t launch_dist_grid(const VolView& v, const Basket& b, double* step, int32_t* hit, double* bpoint, int32_t* nref,
                              cudaStream_t s, int num_sms) {
-    if (4 * b.n >= int64_t(num_sms) * kStaged * 5) {
+    if (!b.link && 4 * b.n >= int64_t(num_sms) * kStaged * 5) {
         const int64_t own = int64_t(sizeof(Sheet<kOnSheet>)) * (kStaged / 32);
         const int64_t staged = own + int64_t(v.nf) * int64_t(sizeof(FiltHvy)) + int64_t(v.vox_small_bytes);
         int dev = 0, most = 0;

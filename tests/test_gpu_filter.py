@@ -127,6 +127,10 @@ def test_grid_equals_fp64_bitwise(g, counts, grid):
         s1, h1 = g.geo_dist_to_boundary(vol, *t, mode=g.GEO_FP32_REFINE)
         assert torch.equal(h0, h1)
         assert torch.equal(s0.view(torch.int64), s1.view(torch.int64))
+    # host arrays in place: one thread per track whatever the size
+    host = [x.cpu().pin_memory() for x in t]
+    s2, h2 = g.geo_dist_to_boundary_host(vol, *host, mode=g.GEO_FP32_REFINE)
+    assert torch.equal(h2, h0.cpu()) and torch.equal(s2.view(torch.int64), s0.cpu().view(torch.int64))
     assert g.geo_check_device_status(vol) == 0
 
 
