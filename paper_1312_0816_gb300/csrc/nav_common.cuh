@@ -88,45 +88,55 @@ __device__ __forceinline__ void nav_vox64(const VolView& v, const ShapeRec64* __
     setup(2, i2, s2, m2, e2);
     const int g0 = v.grid[0], g1 = v.grid[1], g2 = v.grid[2];
     int mb0 = -1, mb1 = -1, mb2 = -1, mb3 = -1;
-    const int maxit = g0 + g1 + g2 + 3;
-    for (int it = 0; it < maxit; ++it) {
-        const int c = (i0 * g1 + i1) * g2 + i2;
-        const int q1 = v.vox_off[c + 1];
-        for (int e = v.vox_off[c]; e < q1; ++e) {
-            const int j = v.vox_ids[e];
-            if (j == mb0 || j == mb1 || j == mb2 || j == mb3) continue;
-            mb3 = mb2; mb2 = mb1; mb1 = mb0; mb0 = j;
-            const ShapeRec64& r = tab[j];
-            const double w0 = r.t[0] - px, w1 = r.t[1] - py, w2 = r.t[2] - pz;
-            const double proj = w0 * qx + w1 * qy + w2 * qz;
-            const double rb = r.brad * dn;
-            if (proj + rb < 0.0) continue;
-            if (proj - rb > best * dd) continue;
-            const double ww = w0 * w0 + w1 * w1 + w2 * w2;
-            if (ww * dd - proj * proj > rb * rb) continue;
+    int left = g0 + g1 + g2 + 3;   // cells at most
+    int c = (i0 * g1 + i1) * g2 + i2, e = v.vox_off[c], q1 = v.vox_off[c + 1];
+    // A flat walk: every lane goes on by itself, a list entry or a cell a turn, until it
+    // holds a daughter whose sphere it meets, and all lanes evaluate theirs together.
+    // (As two nested loops the lanes' evaluations were together or apart as the
+    // compiler happened to place them: 512 daughters, 2^20 tracks, 3.6 to 5.3 ms
+    // for 2.94 so.)
+    bool more = true;
+    while (more) {
+        int j = -1;
+        do {
+            if (e < q1) {
+                const int k = v.vox_ids[e++];
+                if (k != mb0 && k != mb1 && k != mb2 && k != mb3) {
+                    mb3 = mb2; mb2 = mb1; mb1 = mb0; mb0 = k;
+                    const ShapeRec64& r = tab[k];
+                    const double w0 = r.t[0] - px, w1 = r.t[1] - py, w2 = r.t[2] - pz;
+                    const double proj = w0 * qx + w1 * qy + w2 * qz;
+                    const double rb = r.brad * dn;
+                    const double ww = w0 * w0 + w1 * w1 + w2 * w2;
+                    if (!(proj + rb < 0.0) && !(proj - rb > best * dd) && !(ww * dd - proj * proj > rb * rb)) j = k;
+                }
+            } else {
+                // the cell is left at min(m0, m1, m2): nothing entered later can win
+                const double mn = fmin(m0, fmin(m1, m2));
+                const bool a0 = m0 <= m1 && m0 <= m2, a1 = !a0 && m1 <= m2, a2 = !a0 && !a1;
+                i0 += a0 ? s0 : 0;
+                i1 += a1 ? s1 : 0;
+                i2 += a2 ? s2 : 0;
+                m0 = a0 ? m0 + e0 : m0;
+                m1 = a1 ? m1 + e1 : m1;
+                m2 = a2 ? m2 + e2 : m2;
+                more = !(best < mn * (1.0 - 9.094947017729282e-13)) && i0 >= 0 && i0 < g0 && i1 >= 0 && i1 < g1 && i2 >= 0 &&
+                       i2 < g2 && --left > 0;
+                if (more) {
+                    c = (i0 * g1 + i1) * g2 + i2;
+                    e = v.vox_off[c];
+                    q1 = v.vox_off[c + 1];
+                }
+            }
+        } while (j < 0 && more);
+        if (j >= 0) {
             double x[3], u[3];
-            to_local64(r, px, py, pz, qx, qy, qz, x, u);
-            const double s = dist_out64(r, x, u);
+            to_local64(tab[j], px, py, pz, qx, qy, qz, x, u);
+            const double s = dist_out64(tab[j], x, u);
             if (LT(s, best) || (BITS(s) == BITS(best) && h >= 0 && j < h)) {
                 best = s;
                 h = j;
             }
-        }
-        // the cell is left at min(m0, m1, m2): nothing entered later can win
-        const double mn = fmin(m0, fmin(m1, m2));
-        if (best < mn * (1.0 - 9.094947017729282e-13)) break;
-        if (m0 <= m1 && m0 <= m2) {
-            i0 += s0;
-            if (i0 < 0 || i0 >= g0) break;
-            m0 += e0;
-        } else if (m1 <= m2) {
-            i1 += s1;
-            if (i1 < 0 || i1 >= g1) break;
-            m1 += e1;
-        } else {
-            i2 += s2;
-            if (i2 < 0 || i2 >= g2) break;
-            m2 += e2;
         }
     }
 }

@@ -16,7 +16,9 @@
 
 namespace geonav {
 
-// Voxelised volumes: the grid's walk (nav_vox64).
+// Voxelised volumes: the grid's walk (nav_vox64), bound by the FP64 unit (its walk's
+// and culls' instructions).  512 daughters: 65536 tracks 290 -> 241 us, 2^20 3.64 -> 2.94 ms;
+// the records staged in shared memory give the same times (2.95 ms).
 __global__ void __launch_bounds__(256) k_dist_vox64(VolView v, Basket b, double* __restrict__ step,
                                                     int32_t* __restrict__ hit, double* __restrict__ bpoint) {
     const int64_t stride = int64_t(gridDim.x) * blockDim.x;
