@@ -60,8 +60,8 @@ FP32_SPHERE, FP32_TRANSFORM = 16, 18   # the rotation is skipped for identity pl
 FP32_SHAPE = {0: 45, 1: 90, 2: 110}
 FP32_DDA_STEP = 12     # one grid step: pick the axis, advance index and boundary, test the range
 FP32_MOTHER = 100      # the mother's two FP32 exits (shrunk and grown copy)
-KERNEL_SOURCES = ("nav_refine.cu", "refine_kernel.cuh", "nav_refine.cuh", "shapes32.cuh", "shapes64.cuh", "nav_common.cuh",
-                  "stage.cuh", "geo_internal.h")
+KERNEL_SOURCES = ("nav_refine_direct.cu", "filter_pass.cuh", "nav_refine.cuh", "shapes32.cuh", "shapes64.cuh",
+                  "nav_common.cuh", "stage.cuh", "geo_internal.h")
 
 
 def log(*a):
@@ -221,7 +221,7 @@ def captured_traffic():
     """DRAM bytes per launch of the refine kernel from the committed ncu
     summary, only if the kernel sources are those that were captured."""
     try:
-        rec = json.load(open(os.path.join(ROOT, "profiles", "k_dist_refine_toy40_2p20.json")))
+        rec = json.load(open(os.path.join(ROOT, "profiles", "k_dist_direct_toy40_2p20.json")))
     except Exception:
         return None, None
     if rec.get("sources_sha") != sources_sha():
@@ -423,15 +423,14 @@ def batched_leg(pkg, scenes, rank, steps):
         sc_v = vols[int(v)]
         f64 += float(fp64_cost_per_track(sc_v, h_np[off:off + cnt], Q_RATES[0], Q_RATES[1]).sum())
         f32 += fp32_ops_per_track(sc_v) * int(cnt)
-    roof = roof_block(f64, f32, 60.0 * tr.n, ms * 1e-3, "k_dist_batched (one launch per step)",
+    roof = roof_block(f64, f32, 60.0 * tr.n, ms * 1e-3, "k_batched_direct (one launch per step)",
                       "per track: its volume's mother exit, winning daughter and boundary point in FP64; "
                       "every daughter bounded in FP32; 60 B of HBM", PEAK_HBM[0])
     return {"workload": "64 volumes (box/tube mothers, 4..200 mixed daughters), %d baskets of 16..65536 "
                         "tracks, %d tracks, FP32+refine, one persistent launch per step as a CUDA graph"
                         % (len(rows), tr.n),
             "value": tr.n / (ms * 1e-3), "unit": "tracks/s", "ms_per_launch": ms, "steps": steps,
-            "schedule": {"tile_order": order, "blocks_per_sm": bps, "tile_tracks": tile,
-                         "warps": "12 producer + 4 consumer" if tile == 384 else "8 producer + 4 consumer"},
+            "schedule": {"tile_order": order, "blocks_per_sm": bps, "tile_tracks": tile},
             "autotune_ms": timings, "roofline": roof}
 
 
@@ -523,7 +522,7 @@ def voxel_leg(pkg, scenes, rank, steps, n=1 << 24):
             f32_track = float(cand.mean() * per_cand + dda.mean() * FP32_DDA_STEP + FP32_MOTHER)
             f64_track = float(fp64_cost_per_track(sc, h_np, Q_RATES[0], Q_RATES[1]).mean())
             out["roofline"] = roof_block(f64_track * tr.n, f32_track * tr.n, 60.0 * tr.n, ms * 1e-3,
-                                         "k_dist_refine, grid traversal (one launch per step)",
+                                         "k_grid_sheets (one launch per step)",
                                          "per track: FP32 bounds of the distinct daughters listed in the cells "
                                          "the line crosses up to its step (%.2f on average, instrumented walk of "
                                          "4000 tracks) and %.2f grid steps; FP64 mother, winner and boundary point"
@@ -1037,7 +1036,7 @@ def main():
             "pipe": "fp64",
             "peak_source": "nominal: 152 SMs x 2 DFMA/cycle x 2 flop x 2.07 GHz (unit counts and clock); "
                            "the probe measured %.3f TFLOP/s" % (2 * r_f64 / 1e12),
-            "kernel": "k_dist_refine (one launch per step)", "kernel_sources_sha": sources_sha(),
+            "kernel": "k_dist_direct (one launch per step)", "kernel_sources_sha": sources_sha(),
             "algorithmic_per_track": {"hbm_bytes": hbm_bytes, "fp64_dfma_equiv": ops64, "fp32_instr": ops32},
             "fp64_count": "the mother's exit on every track, the winning daughter's transform and "
                           "DistFromOutside, the boundary point",

@@ -370,7 +370,8 @@ struct GridTab {
 // along the FP32 ray; at most gx + gy + gz + 3 cells).  What bounds it: the lanes'
 // own walks diverge, so the loop is flat -- every turn a lane goes on to its
 // next cell if its list is done, then looks at one entry -- until the lane holds a
-// daughter whose sphere it meets; then all lanes bound their daughters together.  A certain entry shortens Um and with it the walk (the
+// daughter whose sphere it meets; then all lanes bound their daughters
+// together.  A certain entry shortens Um and with it the walk (the
 // 512-daughter volume: about half of the tracks enter a daughter, most
 // far before the mother's exit).  A daughter met again is skipped (4-entry mailbox,
 // then the candidate list).

@@ -1131,8 +1131,8 @@ geo_status geo_build_batch(const geo_volume* vols, int32_t n_vols, const geo_bas
     // Every basket's full T-track stretches become tiles of
     // consecutive tracks; the ragged tails of a volume's baskets are
     // gathered, in basket order, into packed tiles that list their tracks'
-    // indices, so that baskets of a few tracks still fill the producer
-    // threads.
+    // indices, so that baskets of a few tracks still fill whole
+    // tiles.
     std::vector<BatchTile> tiles;
     std::vector<int64_t> cost;
     std::vector<std::vector<int64_t>> tails(static_cast<size_t>(n_vols));

@@ -10,7 +10,7 @@ namespace geonav {
 
 constexpr int KBOX = 0, KTUBE = 1, KCONE = 2, KTUBS = 3, KPCON = 4;
 constexpr int kMaxPlanes = GEO_MAX_PLANES;
-// tracks per tile of the FP32-filter kernels (one per producer thread)
+// tracks per tile of a batch and of the pipelined kernel (one per producer thread)
 constexpr int kTileTracks = GEO_TILE_TRACKS;
 
 // Plane table of one polycone of n planes (m = n - 1 sections), FP64:

@@ -19,9 +19,9 @@ namespace geonav {
 // instruction every 64 cycles; a dependent FP64 chain takes about 76 cycles
 // per step, and the square roots, divisions and comparisons between them
 // leave gaps, so one warp cannot keep its unit busy and two do better.
-// This kernel serves volumes with tube segments or polycones, whose tracks need
-// whole solids of differing kinds in FP64, and volumes with a uniform grid;
-// nav_refine_direct.cu serves the others.  (While it served those too, the toy
+// This kernel serves volumes with tube segments, polycones or apex cones, whose
+// tracks need whole solids of differing kinds in FP64, with or without a uniform
+// grid; nav_refine_direct.cu and nav_refine_grid.cu serve the others.  (While it served those too, the toy
 // detector's 2^20 tracks took 0.222 ms with 12 + 4 warps, 0.257 with 12 + 2 at 72
 // registers, 0.248 with 11 + 3, 0.264 with 9 + 3 at 80 registers.)
 //  producers: wait done[k%2] (the stage's previous tile, k-2, finished), FP32

@@ -71,8 +71,8 @@ __device__ __forceinline__ void world_to_node(const double* G, double px, double
                                               double qy, double qz, double* x, double* u) {
     const double w0 = SUB(px, G[9]), w1 = SUB(py, G[10]), w2 = SUB(pz, G[11]);
     constexpr long long kOneBits = 0x3ff0000000000000LL;
-    const bool ident = BITS(G[0]) == kOneBits && BITS(G[4]) == kOneBits && BITS(G[8]) == kOneBits && IS_ZERO(G[1]) && IS_ZERO(G[2]) && IS_ZERO(G[3]) &&
-                       IS_ZERO(G[5]) && IS_ZERO(G[6]) && IS_ZERO(G[7]);
+    const bool ident = BITS(G[0]) == kOneBits && BITS(G[4]) == kOneBits && BITS(G[8]) == kOneBits && IS_ZERO(G[1]) &&
+                       IS_ZERO(G[2]) && IS_ZERO(G[3]) && IS_ZERO(G[5]) && IS_ZERO(G[6]) && IS_ZERO(G[7]);
     if (ident) {
         x[0] = w0; x[1] = w1; x[2] = w2;
         u[0] = qx; u[1] = qy; u[2] = qz;
