@@ -244,10 +244,12 @@ typedef struct {
 
 /* tile_order: 0 = largest estimated cost first (tracks x daughters), 1 = in
  * basket order (the packed tiles of ragged tails after the baskets' full
- * tiles, volume by volume).  blocks_per_sm: resident blocks of the persistent launch
- * (0 = as many as fit).  tile_tracks: tracks per tile, 0 or GEO_TILE_TRACKS
- * (384) or 256 (a batch with tube segments, polycones or apex cones runs 12
- * producer and 4 consumer warps on the former, 8 and 4 on the latter).  Values other than these give GEO_ERR_INVALID_ARG. */
+ * tiles, volume by volume).  blocks_per_sm: resident blocks of the persistent
+ * launch, of 512 threads (0 = as many as fit; two fill an SM).  tile_tracks:
+ * tracks per tile, 0 or GEO_TILE_TRACKS (384) or 256 (a batch with tube
+ * segments, polycones or apex cones runs 12 producer and 4 consumer warps on
+ * the former, 8 and 4 on the latter).  Values other than these give
+ * GEO_ERR_INVALID_ARG. */
 typedef struct {
     int32_t tile_order;
     int32_t blocks_per_sm;

@@ -9,8 +9,8 @@
 // What bounds it: latency of the lanes' record gathers through L1 (a third of
 // the warps' time) with issue slots at 60 % and the FP64 unit at 55 %.  64
 // volumes of 4 to 200 daughters, 2^22 tracks: 675 us with producer and consumer warps over
-// tables staged per tile, 616 us here (32 warps per SM 660, 24 657; parts of
-// 192 tracks 630, of 64 644; chunks of 14 parts claimed by a block, so that an SM's
+// tables staged per tile, 616 us here (32 warps per SM 660, 24 657; two blocks of
+// 448 threads 641; parts of 192 tracks 630, of 64 644; chunks of 14 parts claimed by a block, so that an SM's
 // warps share a volume, 734: the last chunks run alone).
 #include <cuda_runtime.h>
 
@@ -64,7 +64,9 @@ template <bool VOX>
 static cudaError_t launch(const BatchView& bv, const Basket& b, double* step, int32_t* hit, int blocks_per_sm, int tile_tracks,
                           cudaStream_t s, int num_sms) {
     const int most = resident_blocks(reinterpret_cast<const void*>(k_batched_direct<VOX>), kBatchThreads, 0);
-    const int per_sm = (blocks_per_sm <= 0 || blocks_per_sm > most) ? most : blocks_per_sm;
+    // the caller's limit counts blocks of 512 threads (k_dist_batched's): four of
+    // these each, so that two are the whole SM for either kernel
+    const int per_sm = (blocks_per_sm <= 0 || 4 * int64_t(blocks_per_sm) > most) ? most : 4 * blocks_per_sm;
     // Parts of 128 tracks sort best, but a warp takes 80 us for one: while there are
     // fewer than two for each warp, smaller ones (us for parts of 32 / 64 / 128, 64 volumes:
     // 4096 tracks 45 / 60 / 83, 300000 85 / 89 / 117, 600000 124 / 118 / 138,
