@@ -425,7 +425,8 @@ def batched_leg(pkg, scenes, rank, steps):
         f32 += fp32_ops_per_track(sc_v) * int(cnt)
     roof = roof_block(f64, f32, 60.0 * tr.n, ms * 1e-3, "k_batched_direct (one launch per step)",
                       "per track: its volume's mother exit, winning daughter and boundary point in FP64; "
-                      "every daughter bounded in FP32; 60 B of HBM", PEAK_HBM[0])
+                      "every daughter bounded in FP32 (the plain algorithm's count: the kernel bounds "
+                      "only the daughters that a cheap test leaves, so frac may exceed 1); 60 B of HBM", PEAK_HBM[0])
     return {"workload": "64 volumes (box/tube mothers, 4..200 mixed daughters), %d baskets of 16..65536 "
                         "tracks, %d tracks, FP32+refine, one persistent launch per step as a CUDA graph"
                         % (len(rows), tr.n),
