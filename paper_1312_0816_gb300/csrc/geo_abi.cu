@@ -376,9 +376,28 @@ bool make_rec32(const geo_placed_shape& s, double grow, double delta, ShapeRec32
 
 bool needs_segs_code(const geo_placed_shape& s);
 
-// The plain FP64 step's cull table in the filter's order (`hvy`: its entries).
+// Reach of a daughter's FP64 rounding (mm): its whole routine may accept a line
+// this far beside the solid.  The crossings of a quadric are formed about the
+// start, whose distance W to the solid's origin is at most S + |t| in a mother
+// of extent S, and carry an error of about 1e-15 W^2 (1 + slope^2) in the
+// squared radius: 3e-8 W beside a thin solid, and as much along the track where it
+// is tangent.  The culls have to let every line pass that the routine accepts, so
+// the bounding spheres and annuli reach six times as far (0.4 um more in a
+// detector of 1 m).
+double reach64(const geo_placed_shape& s, double S) {
+    const double W = S + std::sqrt(s.trans[0] * s.trans[0] + s.trans[1] * s.trans[1] + s.trans[2] * s.trans[2]);
+    double slope2 = 0.0;
+    if (s.kind == GEO_CONE) {
+        const double bo = (s.p[4] - s.p[2]) / (2.0 * s.p[0]), bi = (s.p[3] - s.p[1]) / (2.0 * s.p[0]);
+        slope2 = std::max(bo * bo, bi * bi);
+    }
+    return 2e-7 * W * std::sqrt(1.0 + slope2);
+}
+
+// The plain FP64 step's cull table in the filter's order (`hvy`: its entries) for
+// daughters whose records already hold the enlarged bounding radius.
 std::vector<Cull64> make_cull(const geo_placed_shape* in, const std::vector<ShapeRec64>& d,
-                              const std::vector<FiltHvy>& hvy, int32_t nq1) {
+                              const std::vector<FiltHvy>& hvy, int32_t nq1, double S) {
     std::vector<Cull64> out(hvy.size());
     for (size_t k = 0; k < hvy.size(); ++k) {
         Cull64& c = out[k];
@@ -412,9 +431,8 @@ std::vector<Cull64> make_cull(const geo_placed_shape* in, const std::vector<Shap
             lo = s.p[0];
             h = s.p[2];
         }
-        // enlarged as brad is: the cull's own FP64 rounding, relative to the
-        // distances a track covers, stays far below
-        const double grow = 1e-9 + 1e-12 * (r.brad + std::fabs(c.t[0]) + std::fabs(c.t[1]) + std::fabs(c.t[2]));
+        // enlarged as brad is
+        const double grow = 1e-9 + reach64(s, S);
         c.a = hi + grow;
         c.b = lo - grow;
         c.h = h + grow;
@@ -828,6 +846,7 @@ geo_status geo_build_volume(const geo_placed_shape* mother, const geo_placed_sha
     std::vector<ShapeRec32> h32(n_daughters);
     for (int j = 0; j < n_daughters; ++j) {
         h64[j] = make_rec64(daughters[j], table_of(j));
+        h64[j].brad += reach64(daughters[j], S);
         const double dl = inflation(daughters[j], S);
         if (!make_rec32(daughters[j], dl, dl, h32[j])) {
             geo_destroy_volume(v);
@@ -856,7 +875,7 @@ geo_status geo_build_volume(const geo_placed_shape* mother, const geo_placed_sha
     // the FP32 records, then the filter's two tables
     const size_t b32 = sizeof(ShapeRec32) * size_t(std::max(n_daughters, 1));
     vw.nf = int32_t(hsph.size());
-    const std::vector<Cull64> hcull = make_cull(daughters, h64, hhvy, vw.nq1);
+    const std::vector<Cull64> hcull = make_cull(daughters, h64, hhvy, vw.nq1, S);
     const size_t bsph = sizeof(FiltSph) * hsph.size(), bhvy = sizeof(FiltHvy) * hhvy.size();
     const size_t bcull = sizeof(Cull64) * hcull.size();
     if ((e = lib_malloc(&v->d64, b64)) != cudaSuccess || (e = lib_malloc(&v->d32, b32 + bsph + bhvy + bcull)) != cudaSuccess ||

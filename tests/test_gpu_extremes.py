@@ -1,0 +1,73 @@
+"""Inputs at the ends of their ranges: both modes and every kernel give the
+plain FP64 routines' bits there too."""
+import numpy as np
+import pytest
+
+from paper_1312_0816_gb300 import scenes
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+EYE = np.eye(3).reshape(9)
+
+
+@pytest.fixture(scope="module")
+def g():
+    import paper_1312_0816_gb300 as pkg
+
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    pkg.load()
+    return pkg
+
+
+def cuda(*arrays):
+    return [torch.from_numpy(np.ascontiguousarray(a)).cuda() for a in arrays]
+
+
+def same(a, b):
+    return torch.equal(a[0].view(torch.int64), b[0].view(torch.int64)) and all(torch.equal(x, y) for x, y in zip(a[1:], b[1:]))
+
+
+@pytest.mark.parametrize("extent", [1e3, 1e4, 1e5, 1e6, 1e7])
+@pytest.mark.parametrize("rotated", [False, True])
+def test_small_solids_in_a_large_mother(g, extent, rotated):
+    """Tracks from far away that graze small solids, within the rounding of the
+    quadrics' crossings and beyond: the FP64 culls (annuli and spheres, lists
+    and the walk of a one-cell grid) pass every line that the whole routine
+    accepts, so the modes and the kernels agree."""
+    rng = np.random.default_rng(int(extent) + rotated)
+    n = 200003
+    kinds = [(scenes.TUBE, (0.0, 5.0, 100.0)), (scenes.CONE, (100.0, 1.0, 4.0, 2.0, 6.0)), (scenes.TUBE, (4.0, 5.0, 50.0)),
+             (scenes.CONE, (0.5, 2.0, 4.0, 3.0, 9.0)), (scenes.TUBE, (0.0, 0.1, 80.0)), (scenes.TUBE, (0.0, 5.0, 0.05))]
+    rows = [(*kinds[k % 6], scenes.haar_rotation(rng) if rotated else EYE,
+             (0.0, 0.0, 0.0) if k % 4 == 0 else (30.0 * k - 500.0, 3.0 * k, 0.0)) for k in range(36)]
+    sc = scenes._scene("far", scenes.BOX, (extent,) * 3, rows)
+    flat, walk = g.geo_build_volume(sc), g.geo_build_volume(sc, voxelize=True, grid=(1, 1, 1))
+    j = rng.integers(0, len(rows), n)
+    prm, cone = sc.params[j], sc.kinds[j] == scenes.CONE
+    half = np.where(cone, prm[:, 0], prm[:, 2])
+    z = rng.uniform(-1.01, 1.01, n) * half
+    slope = np.where(cone, (prm[:, 4] - prm[:, 2]) / (2.0 * half), 0.0)
+    radius = np.where(cone, 0.5 * (prm[:, 2] + prm[:, 4]), prm[:, 1]) + slope * z
+    radius = np.where(rng.random(n) < 0.2, np.where(cone, 1.5, np.maximum(prm[:, 0], 0.05)), radius)
+    b = radius * (1.0 + 10.0 ** rng.uniform(-14.0, -2.0, n) * rng.choice([-1.0, 1.0], n))
+    ph = rng.uniform(0.0, 2.0 * np.pi, n)
+    u = np.stack([np.cos(ph), np.sin(ph), slope * 0.0 + rng.normal(0.0, 0.3, n) * rng.integers(0, 2, n)])
+    u /= np.linalg.norm(u, axis=0)
+    foot = np.stack([-b * np.sin(ph), b * np.cos(ph), z])
+    local = foot - u * rng.uniform(0.05, 0.65, n) * (extent - 600.0)
+    R = sc.rot[j].reshape(n, 3, 3)
+    p = np.einsum("nab,bn->an", R, local) + sc.trans[j].T
+    t = cuda(*p, *np.einsum("nab,bn->an", R, u))
+    f0 = g.geo_dist_to_boundary(flat, *t, mode=g.GEO_FP64)
+    assert int((f0[1] >= 0).sum()) > n // 4
+    assert same(f0, g.geo_dist_to_boundary(walk, *t, mode=g.GEO_FP64))
+    for v in (flat, walk):
+        assert same(f0, g.geo_dist_to_boundary(v, *t, mode=g.GEO_FP32_REFINE))
+    # the step of a track and the whole routine of the solid it enters
+    for k in range(6):
+        i = torch.nonzero(f0[1] == k).flatten()
+        kind, q = rows[k][0], rows[k][1]
+        own = g.geo_shape_query(kind, q, g.GEO_Q_DIST_OUT, *[x[i].contiguous() for x in t], rot=rows[k][2], trans=rows[k][3])
+        assert torch.equal(own.view(torch.int64), f0[0][i].view(torch.int64))
