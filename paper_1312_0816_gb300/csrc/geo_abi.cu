@@ -575,6 +575,24 @@ double inflation(const geo_placed_shape& s, double S) {
     return d;
 }
 
+// Least |d|^2 that the FP32 pass takes in an extent S: no square of it that the
+// margins resolve may fall below the normal FP32 range (1.2e-38), where the
+// filter's roots and reciprocals give 0 and infinity (shapes32.cuh).
+//  - The annulus test divides by the squared part across the axis down to
+//    1e-12 |d|^2:                                                   |d|^2 > 1e-25.
+//  - A discriminant that is lost changes a quadric's radius r by
+//    1.2e-38 / (2 s^2 |d|^2 r) for a track inclined by s.  It matters from s =
+//    delta / 2 S = 1.5e-6 on (below, the track covers less than delta across the
+//    axis) and r = delta (the copy's), and is to be small against delta:
+//                                                        |d|^2 delta^2 > 1e-24.
+// Shorter directions take the whole FP64 routines; a unit vector is never
+// short down to extents of 1e-6 mm.
+float dd_limit(double S) {
+    const double delta = 48.0 * kEps32 * S;   // the least inflation of any solid
+    const double lim = std::max(1e-25, 1e-24 / (delta * delta));
+    return lim < 1e30 ? float_up(lim) : HUGE_VALF;
+}
+
 // The one-solid query's FP32 copies, good for points within 16 times the solid's
 // own reach; false where they do not decide anything (other kinds, an apex, a
 // hole or a solid no larger than the inflation).
@@ -598,6 +616,7 @@ bool make_fast(const geo_placed_shape& s, ShapeFast& f) {
     if (f.h.flags & kFiltLoose) return false;
     f.m64 = make_rec64(s);
     f.reach = float(S / 1.8);   // |p| <= sqrt(3) max |p_k| < S
+    f.dd_min = dd_limit(S);
     return true;
 }
 
@@ -862,6 +881,7 @@ geo_status geo_build_volume(const geo_placed_shape* mother, const geo_placed_sha
         return GEO_ERR_SHAPE_PARAMS;
     }
     vw.nd = n_daughters;
+    vw.dd_min = dd_limit(S);
     // the kernels' instantiation with the out-of-line code of tube segments,
     // polycones and cones through an apex on an end plane
     vw.segs = needs_segs_code(*mother) ? 1 : 0;

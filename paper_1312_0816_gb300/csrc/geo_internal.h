@@ -161,7 +161,7 @@ struct __align__(16) VolView {
     int32_t grid[3];
     int32_t segs;              // 1 if the mother or a daughter is a tube segment or a polycone, or a cone with an
                                // apex on an end plane (needs_segs_code)
-    int32_t pad_;
+    float dd_min;              // least |d|^2 that the FP32 pass takes (shapes32.cuh)
     double lo[3];
     double cell[3];
     double inv_cell[3];
@@ -266,12 +266,14 @@ struct ShapeArg {
 };
 // The same for a box, tube or cone whose FP32 copies decide most of a query:
 // its placed copy (an entry of the filter's tables), the copies shrunk and
-// grown in its own frame, and the largest coordinate of a point they are good for.
+// grown in its own frame, and the largest coordinate of a point and the least
+// |d|^2 they are good for.
 struct ShapeFast {
     ShapeRec64 m64;
     ShapeRec32 m32, m32u;
     FiltHvy h;
     float reach;
+    float dd_min;
 };
 cudaError_t launch_shape_lists(const ShapeFast& a, int what, const Basket& b, double* out, int32_t* face,
                                cudaStream_t s, int num_sms);

@@ -194,7 +194,7 @@ __device__ __forceinline__ void refine_pass1(const VolView& v, const FiltTab& f,
     r.p[0] = f64_to_f32_trunc(px); r.p[1] = f64_to_f32_trunc(py); r.p[2] = f64_to_f32_trunc(pz);
     r.d[0] = f64_to_f32_trunc(qx); r.d[1] = f64_to_f32_trunc(qy); r.d[2] = f64_to_f32_trunc(qz);
     const float dd = fmaf(r.d[0], r.d[0], fmaf(r.d[1], r.d[1], r.d[2] * r.d[2]));
-    if (!(dd > 1e-30f && dd < 1e30f)) {
+    if (!(dd > v.dd_min && dd < 1e30f)) {
         // direction magnitude outside the range the FP32 bounds assume
         const double p[3] = {src(0), src(1), src(2)};
         if (contains64<SEGS>(v.m64, p))

@@ -127,7 +127,7 @@ __global__ void __launch_bounds__(kSoloWarps * 32, 4) k_shape_lists(const __grid
                     if (kDist) {
                         r.d[0] = f64_to_f32_trunc(qx); r.d[1] = f64_to_f32_trunc(qy); r.d[2] = f64_to_f32_trunc(qz);
                         const float dd = fmaf(r.d[0], r.d[0], fmaf(r.d[1], r.d[1], r.d[2] * r.d[2]));
-                        near = near && dd > 1e-30f && dd < 1e30f;
+                        near = near && dd > a.dd_min && dd < 1e30f;
                         const float inv_dd = frcp(dd);
                         r.inv_dn = rsqrtf(dd) * (1.f + 4.f * kEps32f);
 #pragma unroll

@@ -236,7 +236,7 @@ static __device__ __forceinline__ void world_pass1(const VolView& v, const doubl
         r.d[k] = f64_to_f32_trunc(u[k]);
     }
     const float dd = fmaf(r.d[0], r.d[0], fmaf(r.d[1], r.d[1], r.d[2] * r.d[2]));
-    if (!(dd > 1e-30f && dd < 1e30f)) {
+    if (!(dd > v.dd_min && dd < 1e30f)) {
         world_nav64(v, x, u, skip, entered, best, h);
         return;
     }

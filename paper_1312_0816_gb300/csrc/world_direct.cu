@@ -46,7 +46,7 @@ __device__ __forceinline__ void world_pass_lists(const VolView& v, const double*
         r.d[k] = f64_to_f32_trunc(u[k]);
     }
     const float dd = fmaf(r.d[0], r.d[0], fmaf(r.d[1], r.d[1], r.d[2] * r.d[2]));
-    if (!(dd > 1e-30f && dd < 1e30f)) {
+    if (!(dd > v.dd_min && dd < 1e30f)) {
         const double xx[3] = {src(0), src(1), src(2)}, uu[3] = {src(3), src(4), src(5)};
         world_nav64(v, xx, uu, skip, entered, best, h);
         return;

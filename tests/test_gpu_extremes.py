@@ -71,3 +71,61 @@ def test_small_solids_in_a_large_mother(g, extent, rotated):
         kind, q = rows[k][0], rows[k][1]
         own = g.geo_shape_query(kind, q, g.GEO_Q_DIST_OUT, *[x[i].contiguous() for x in t], rot=rows[k][2], trans=rows[k][3])
         assert torch.equal(own.view(torch.int64), f0[0][i].view(torch.int64))
+
+
+@pytest.mark.parametrize("scene", ["shells", "thin"])
+@pytest.mark.parametrize("length", [1.0, 1e-6, 1e-9, 1e-10, 1e-11, 1e-12, 1e-13, 1e-14, 1.2e-15])
+def test_short_directions(g, scene, length):
+    """Directions from units down to where their squares leave the normal FP32
+    range, inclined to the solids' axis by anything from 1e-6 on."""
+    rng = np.random.default_rng(5)
+    n = 60007
+    if scene == "shells":
+        cone = (5.0, 1.0, 12.0, 2.0, 20.0)
+        rows = [(scenes.TUBE, (0.0, 10.0, 5.0), EYE, (0.0, 0.0, 40.0 * k)) for k in range(-4, 5)]
+        rows += [(scenes.CONE, cone, EYE, (60.0, 0.0, 40.0 * k)) for k in range(-8, 9)]
+        rows += [(scenes.TUBE, (3.0, 10.0, 5.0), EYE, (-60.0, 0.0, 40.0 * k)) for k in range(-8, 9)]
+        sc = scenes._scene("shells", scenes.BOX, (400.0,) * 3, rows)
+        p = np.stack([rng.choice([0.0, 60.0, -60.0], n) + rng.uniform(-9.0, 9.0, n), rng.uniform(-9.0, 9.0, n),
+                      rng.uniform(-390.0, 390.0, n)])
+    else:
+        rows = [(scenes.TUBE, (2e-3, 4e-3, 1.0), EYE, (0.0, 0.0, 2.0)),
+                (scenes.CONE, (1.0, 1e-3, 2e-3, 3e-3, 5e-3), EYE, (0.0, 0.0, -2.0))] * 17
+        sc = scenes._scene("thin", scenes.TUBE, (0.0, 1e-2, 5.0), rows)
+        p = np.stack([rng.uniform(-6e-3, 6e-3, n), rng.uniform(-6e-3, 6e-3, n), rng.uniform(-4.9, 4.9, n)])
+    s, ph = 10.0 ** rng.uniform(-6.0, -0.1, n), rng.uniform(0.0, 2.0 * np.pi, n)
+    t = cuda(*p, *(np.stack([s * np.cos(ph), s * np.sin(ph), rng.choice([-1.0, 1.0], n)]) * length))
+    flat, grid = g.geo_build_volume(sc), g.geo_build_volume(sc, voxelize=True)
+    ref = g.geo_dist_to_boundary(flat, *t, mode=g.GEO_FP64)
+    assert same(ref, g.geo_dist_to_boundary(flat, *t, mode=g.GEO_FP32_REFINE))
+    assert same(ref, g.geo_dist_to_boundary(grid, *t, mode=g.GEO_FP32_REFINE))
+    batch = g.geo_build_batch([flat], [(0, 0, n)])
+    assert same(ref, g.geo_dist_to_boundary_batched(batch, *t))
+    few = [x[:1000].contiguous() for x in t]   # the small-basket kernel
+    assert same([x[:1000] for x in ref], g.geo_dist_to_boundary(flat, *few, mode=g.GEO_FP32_REFINE))
+    # the tree: the volume in a hall, its daughters leaves
+    leaves = [g.geo_build_volume(scenes.leaf(int(k), q)) for k, q in zip(sc.kinds, sc.params)]
+    hall = g.geo_build_volume(scenes._scene("hall", scenes.BOX, (500.0,) * 3, [(sc.mother_kind, sc.mother_params, EYE, (0, 0, 0))]))
+    m = len(leaves)
+    world = g.geo_build_world(leaves + [flat, hall], [[] for _ in leaves] + [list(range(m)), [m]], m + 1)
+    node = torch.full((n,), 1, dtype=torch.int32, device="cuda")
+    a = g.geo_world_step(world, *t, node, mode=g.GEO_FP64)
+    assert same(a, g.geo_world_step(world, *t, node, mode=g.GEO_FP32_REFINE))
+
+
+@pytest.mark.parametrize("length", [1.0, 1e-9, 1e-11, 1e-13, 1.2e-15])
+@pytest.mark.parametrize("kind,prm", [(scenes.TUBE, (3.0, 10.0, 5.0)), (scenes.CONE, (5.0, 1.0, 12.0, 2.0, 20.0)),
+                                      (scenes.TUBE, (0.0, 1e-2, 5.0)), (scenes.BOX, (3.0, 10.0, 5.0))])
+def test_short_directions_of_one_solid(g, kind, prm, length):
+    """The list kernel (from 98304 tracks on) against the whole routine's."""
+    rng = np.random.default_rng(6)
+    n, m = 98304, 90000
+    s, ph = 10.0 ** rng.uniform(-6.0, -0.1, n), rng.uniform(0.0, 2.0 * np.pi, n)
+    size = 1.2 * np.array({scenes.BOX: prm[:3], scenes.TUBE: (prm[1], prm[1], prm[-1])}.get(kind, (20.0, 20.0, 5.0)))
+    p = rng.uniform(-1.0, 1.0, (3, n)) * size[:, None]
+    p[2] += 10.0 * rng.integers(-1, 2, n)
+    t = cuda(*p, *(np.stack([s * np.cos(ph), s * np.sin(ph), rng.choice([-1.0, 1.0], n)]) * length))
+    for what in (g.GEO_Q_DIST_OUT, g.GEO_Q_DIST_IN):
+        a = g.geo_shape_query(kind, prm, what, *t, want_face=True)
+        b = g.geo_shape_query(kind, prm, what, *[x[:m].contiguous() for x in t], want_face=True)
+        assert same([x[:m] for x in a], b)
