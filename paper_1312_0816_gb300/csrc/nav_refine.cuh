@@ -86,6 +86,10 @@ struct MotherExit {
 // hold then as well (`in`) when the line crosses the shrunk copy's outer
 // surface (it does not graze it) and does not leave through the inner one at
 // its start: it starts off that surface, or moves away from the axis.
+// A hole bounds the exit from above only for starts surely off its surface.  On
+// it, FP64 may find its crossing a rounding behind the start and pass over it
+// (a cone's, or any entered mother's), so that the exact exit is the next one,
+// beyond the hole.
 // V holds the solid's copies m32 (shrunk), m32u (grown) and its record m64.
 template <bool ENTERED = false, class V>
 __device__ __forceinline__ MotherExit mother_exit32(const V& v, const Ray32& r, bool entered = false) {
@@ -124,7 +128,8 @@ __device__ __forceinline__ MotherExit mother_exit32(const V& v, const Ray32& r, 
         auto inner = [&](float Al, float Bl, float Cl, bool hole, float Ah, float Bh, float Ch) {
             const float lo = root_falling32(Al, Bl, Cl), hi = hole ? root_falling32(Ah, Bh, Ch) : f_inf();
             if (ENTERED) crosses = crosses && (Cl >= 0.f || Bl > 64.f * kEps32f * fsqrt(Al > 0.f ? Al * rho2 : f_inf()));
-            take(lo >= 0.f ? lo : f_inf(), hi >= 0.f ? hi : f_inf(), kTagInner);
+            const bool off = Cl >= 0.f || (ENTERED && entered && crosses);
+            take(lo >= 0.f ? lo : f_inf(), off && hi >= 0.f ? hi : f_inf(), kTagInner);
         };
         if (kind == KTUBE) {
             m.in = fabsf(x[2]) <= el[2] && rho2 <= el[1] && (el[3] == 0.f || rho2 >= el[0]);

@@ -222,7 +222,12 @@ __device__ __forceinline__ float enter32(const ShapeRec32& r, const float* x, co
 // ------------------------------------------------------- mother exit -------
 // Exit distance of a start point x inside the (shrunk or grown) mother, in the
 // mother's own frame (no shift).  Also reports whether x is inside it.
-__device__ __forceinline__ float exit32(const ShapeRec32& r, const float* x, const float* u, bool& inside) {
+// UPPER: an upper bound from the grown copy, in which the hole counts only
+// (`hole`) for starts 2 delta off the copy's, so off the mother's own surface (see
+// mother_exit32 in nav_refine.cuh).
+template <bool UPPER = false>
+__device__ __forceinline__ float exit32(const ShapeRec32& r, const float* x, const float* u, bool& inside,
+                                        bool hole = true) {
     const float* e = r.e;
     if (r.kind == KBOX) {
         inside = fabsf(x[0]) <= e[0] && fabsf(x[1]) <= e[1] && fabsf(x[2]) <= e[2];
@@ -237,7 +242,8 @@ __device__ __forceinline__ float exit32(const ShapeRec32& r, const float* x, con
         t = u[2] != 0.f ? fdiv(copysignf(e[2], u[2]) - x[2], u[2]) : f_inf();
         s = root_rising32(A0, B0, rho2 - e[1]);
         if (s >= 0.f) t = fminf(t, s);
-        if (e[3] != 0.f) {
+        const float ro = fmaf(2.f, r.delta, e[8]);
+        if (e[3] != 0.f && (!UPPER || (hole && rho2 >= ro * ro))) {
             s = root_falling32(A0, B0, rho2 - e[0]);
             if (s >= 0.f) t = fminf(t, s);
         }
@@ -255,7 +261,8 @@ __device__ __forceinline__ float exit32(const ShapeRec32& r, const float* x, con
         s = root_rising32(fmaf(-rs, rs, A0), fmaf(-ro0, rs, B0), co);
         if (s >= 0.f) t = fminf(t, s);
     }
-    if (e[5] != 0.f) {
+    const float ro = fmaxf(fmaf(2.f * r.delta, sqrtf(fmaf(e[4], e[4], 1.f)), ri0), 0.f);
+    if (e[5] != 0.f && (!UPPER || (hole && rho2 >= ro * ro))) {
         const float rs = e[4] * u[2];
         s = root_falling32(fmaf(-rs, rs, A0), fmaf(-ri0, rs, B0), ci);
         if (s >= 0.f) t = fminf(t, s);

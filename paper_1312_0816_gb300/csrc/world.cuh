@@ -254,7 +254,8 @@ static __device__ __forceinline__ void world_pass1(const VolView& v, const doubl
     }
     st.Lm = in_shrunk ? fmaxf(lower_bound(e_lo, v.m32.delta, r.inv_dn), 0.f) : 0.f;
     bool dummy;
-    const float e_hi = exit32(v.m32u, r.p, r.d, dummy);
+    // (a polycone's bounding tube says nothing of its sections' holes)
+    const float e_hi = exit32<true>(v.m32u, r.p, r.d, dummy, in_shrunk || v.m64.kind != KPCON);
     const float Um = e_hi + 16.f * kEps32f * e_hi + v.m32u.delta * r.inv_dn;
     for (int j = 0; j < v.nd; ++j)
         if (j != skip) bound_daughter(v.d32[j], j, r, Um, st.c);

@@ -129,3 +129,58 @@ def test_short_directions_of_one_solid(g, kind, prm, length):
         a = g.geo_shape_query(kind, prm, what, *t, want_face=True)
         b = g.geo_shape_query(kind, prm, what, *[x[:m].contiguous() for x in t], want_face=True)
         assert same([x[:m] for x in a], b)
+
+
+HOLED = {"cone": (scenes.CONE, (100.0, 30.0, 90.0, 50.0, 120.0)), "tube": (scenes.TUBE, (40.0, 90.0, 100.0)),
+         "tubs": (scenes.TUBS, (40.0, 90.0, 100.0, 0.2, 5.0)),
+         "pcon": (scenes.PCON, scenes.Pcon((-100.0, -20.0, 20.0, 100.0), (20.0, 38.0, 42.0, 30.0), (90.0, 95.0, 95.0, 90.0)))}
+
+
+@pytest.mark.parametrize("copies", [1, 3])   # 12 daughters, 36
+@pytest.mark.parametrize("mother", sorted(HOLED))
+def test_starts_on_the_surface_of_the_mothers_hole(g, mother, copies):
+    """Tracks that start within a rounding of the hole of their mother and move
+    into it: FP64 may pass over the crossing at the start, and the daughters
+    beyond the hole then decide the step."""
+    rng = np.random.default_rng(copies)
+    n = 200003
+    kind, prm = HOLED[mother]
+    a = 2.0 * np.pi / 12 * np.arange(12)
+    rows = [(scenes.BOX, (6.0, 6.0, 20.0), scenes._rot_z(p), (70.0 * np.cos(p), 70.0 * np.sin(p), 0.0)) for p in a] * copies
+    sc = scenes._scene("holed", kind, prm, rows)
+    ph = rng.uniform(0.0, 2.0 * np.pi, n)
+    z = rng.uniform(-90.0, 90.0, n) if mother == "pcon" else rng.uniform(-30.0, 30.0, n)
+    if mother == "cone":
+        ri = 40.0 + 0.1 * z
+    elif mother == "pcon":
+        zp, rn, _ = sc.planes_of(sc.mother_params)
+        ri = np.interp(z, zp, rn)
+    else:
+        ri = np.full(n, 40.0)
+    r = ri * (1.0 + rng.integers(-2, 3, n) * 2.0 ** -53)
+    d = -np.stack([np.cos(ph + rng.normal(0.0, 0.3, n)), np.sin(ph + rng.normal(0.0, 0.3, n)), rng.normal(0.0, 0.1, n)])
+    t = cuda(r * np.cos(ph), r * np.sin(ph), z, *d)
+    flat = g.geo_build_volume(sc)
+    ref = g.geo_dist_to_boundary(flat, *t, mode=g.GEO_FP64)
+    assert int((ref[1] > -2).sum()) > n // 4
+    assert same(ref, g.geo_dist_to_boundary(flat, *t, mode=g.GEO_FP32_REFINE))
+    grid = g.geo_build_volume(sc, voxelize=True)
+    assert same(ref, g.geo_dist_to_boundary(grid, *t, mode=g.GEO_FP32_REFINE))
+    assert same(ref, g.geo_dist_to_boundary_batched(g.geo_build_batch([flat], [(0, 0, n)]), *t))
+    few = [x[:1000].contiguous() for x in t]
+    assert same([x[:1000] for x in ref], g.geo_dist_to_boundary(flat, *few, mode=g.GEO_FP32_REFINE))
+    # the tree: tracks in the volume, or just entered and scattered back
+    seg = (scenes.TUBS, (1.0, 2.0, 3.0, 0.0, 1.0))
+    for other in ([], [(*seg, EYE, (300.0, 0.0, 0.0))]):   # with a segment: the tiled kernel
+        hall = scenes._scene("hall", scenes.BOX, (500.0,) * 3, [(kind, prm, EYE, (0.0, 0.0, 0.0))] + other)
+        vols = [g.geo_build_volume(s) for s in (scenes.leaf(scenes.BOX, (6.0, 6.0, 20.0)), sc, hall)]
+        child = [[], [0] * len(rows), [1]]
+        if other:
+            vols.append(g.geo_build_volume(scenes.leaf(*seg)))
+            child = child[:2] + [[1, 3], []]
+        world = g.geo_build_world(vols, child, 2)
+        node = torch.ones(n, dtype=torch.int32, device="cuda")
+        for f in (-1, -2):
+            flag = torch.full((n,), f, dtype=torch.int32, device="cuda")
+            assert same(g.geo_world_step(world, *t, node, flag, mode=g.GEO_FP64),
+                        g.geo_world_step(world, *t, node, flag, mode=g.GEO_FP32_REFINE))
