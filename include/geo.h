@@ -427,12 +427,21 @@ geo_status geo_check_device_status(geo_volume v, uint32_t* word, void* stream);
  * context stays usable.  Asynchronous on `stream`; read the word with
  * geo_check_device_status.
  *
+ * geo_selftest_batch_timeout: geo_dist_to_boundary_batched in which every wait
+ * for a tile's tables (a batch with tube segments, polycones or apex cones
+ * stages them in shared memory) gives up at once.  The tracks then take the
+ * whole FP64 routines, so the answers are the same, and the timeout (bit 1)
+ * stands in the status word of every volume of the batch.
+ *
  * geo_debug_fail_alloc: host-side fault injection.  With nth > 0, the nth
  * allocation the library makes from now on (host objects of volumes, batches
  * and trees, and their device memory) fails as if memory had run out: the
  * building call frees what it had taken and returns GEO_ERR_OOM.  0 turns it
  * off; negative values give GEO_ERR_INVALID_ARG.  Process-wide. */
 geo_status geo_selftest_wait_timeout(geo_volume v, uint32_t polls, void* stream);
+geo_status geo_selftest_batch_timeout(geo_batch b, const double* x, const double* y, const double* z, const double* dx,
+                                      const double* dy, const double* dz, int64_t n_total, double* step, int32_t* hit,
+                                      void* stream);
 geo_status geo_debug_fail_alloc(int32_t nth);
 
 /* Measurement support (not part of the navigator): issue rate in operations

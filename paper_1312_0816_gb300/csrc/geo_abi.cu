@@ -1265,9 +1265,9 @@ geo_status geo_destroy_batch(geo_batch b) {
     return GEO_OK;
 }
 
-geo_status geo_dist_to_boundary_batched(geo_batch b, const double* x, const double* y, const double* z,
-                                        const double* dx, const double* dy, const double* dz, int64_t n_total,
-                                        double* step, int32_t* hit, void* stream) {
+static geo_status run_batched(geo_batch b, const double* x, const double* y, const double* z, const double* dx,
+                              const double* dy, const double* dz, int64_t n_total, double* step, int32_t* hit,
+                              uint32_t table_polls, void* stream) {
     if (!b) return GEO_ERR_INVALID_ARG;
     int dev = -1;
     if (cudaGetDevice(&dev) != cudaSuccess) return GEO_ERR_CUDA;
@@ -1289,10 +1289,23 @@ geo_status geo_dist_to_boundary_batched(geo_batch b, const double* x, const doub
     bv.nvols = b->n_vols;
     bv.vox = b->vox;
     bv.max_nf = b->max_nf;
+    bv.table_polls = table_polls;
     bv.idx = b->d_idx;
     const Basket bk{x, y, z, dx, dy, dz, n_total};
     return cuda_status(
         launch_dist_batched(bv, bk, step, hit, b->blocks_per_sm, b->tile_tracks, s, num_sms_of(b->device)));
+}
+
+geo_status geo_dist_to_boundary_batched(geo_batch b, const double* x, const double* y, const double* z,
+                                        const double* dx, const double* dy, const double* dz, int64_t n_total,
+                                        double* step, int32_t* hit, void* stream) {
+    return run_batched(b, x, y, z, dx, dy, dz, n_total, step, hit, kWaitLimit, stream);
+}
+
+geo_status geo_selftest_batch_timeout(geo_batch b, const double* x, const double* y, const double* z, const double* dx,
+                                      const double* dy, const double* dz, int64_t n_total, double* step, int32_t* hit,
+                                      void* stream) {
+    return run_batched(b, x, y, z, dx, dy, dz, n_total, step, hit, 0, stream);
 }
 
 geo_status geo_adjoint_workspace_size(geo_volume v, int64_t n, uint64_t* bytes) {

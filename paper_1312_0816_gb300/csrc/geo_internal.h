@@ -177,6 +177,9 @@ struct __align__(16) VolView {
     unsigned int* status;      // device error word (0 = ok)
 };
 
+// polls of a wait for a bulk copy, after which the kernel gives it up
+constexpr uint32_t kWaitLimit = 1u << 22;
+
 struct Basket {
     const double *x, *y, *z, *dx, *dy, *dz;
     int64_t n;
@@ -204,6 +207,7 @@ struct BatchView {
     int32_t vox;              // 1 if a volume has a uniform grid
     int32_t max_nf;           // filter entries of the largest volume
     const int64_t* idx;       // track indices of packed tiles (count < 0), or null
+    uint32_t table_polls = kWaitLimit;   // of a wait for a tile's tables in shared memory
 };
 
 // device error codes written to VolView::status

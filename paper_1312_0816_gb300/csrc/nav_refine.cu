@@ -47,22 +47,31 @@ size_t refine_stage_bytes() { return 2 * (sizeof(Stage<kProd>) + sizeof(Answers<
 // L1 (each track reads one).  A packed tile (negative count) lists its
 // tracks' indices in bv.idx from its base on (the ragged tails of a volume's
 // baskets gathered into full tiles).
+//
+// A wait that runs out is recorded and never followed by a read of what it waited
+// for: tracks whose tables did not arrive take the whole FP64 routines, as do those
+// of the block's later tiles, and a stage whose consumers did not finish is left
+// to them (the block ends).
 struct __align__(16) TileHdr {
     VolView vol;
     int64_t base;
     int count;
     int tile;   // -1: the queue is empty
     int vol_index;
-    int pad[3];
+    int staged;          // the tile's tables were sent to the table area
+    int pad[2];
 };
 
-// the next tile, as claimed by producer thread 0
+// the next tile, as claimed by producer thread 0 (which alone uses it)
 struct NextTile {
     int64_t base;
     int tile, count, vol_index;
+    int staged;          // its tables go to the table area
     uint32_t bytes;      // of its filter tables
     int pending;         // 1: their copy is not issued yet
     const void* src;
+    int staging;         // tiles' tables are still copied
+    uint32_t owed;       // bit p: a copy on tabs[p] that was not seen to end (bit 2 + p: its parity)
 };
 
 // GLOB = false: no volume has a uniform grid and every volume's filter tables
@@ -84,6 +93,8 @@ __global__ void __launch_bounds__(P + C, 2) k_dist_batched(BatchView bv, Basket 
     const int lane = t & 31;
     bool healthy = true;
     if (t == 0) {
+        N.staging = !GLOB;
+        N.owed = 0;
         mbar_init(&full[0], P / 32);
         mbar_init(&full[1], P / 32);
         mbar_init(&done[0], C / 32);
@@ -114,6 +125,7 @@ __global__ void __launch_bounds__(P + C, 2) k_dist_batched(BatchView bv, Basket 
         auto claim = [&](int k, uint32_t used) {
             const unsigned q = atomicAdd(bv.counter, 1u);
             N.pending = 0;
+            N.staged = 0;
             N.bytes = 0;
             if (int64_t(q) < bv.ntiles) {
                 const BatchTile tl = bv.tiles[q];
@@ -121,7 +133,8 @@ __global__ void __launch_bounds__(P + C, 2) k_dist_batched(BatchView bv, Basket 
                 N.base = tl.base;
                 N.count = tl.count;
                 N.vol_index = tl.vol;
-                if (!GLOB) {
+                if (!GLOB && N.staging) {
+                    N.staged = 1;
                     const VolView& nv = bv.vols[tl.vol];
                     N.bytes = uint32_t(nv.nf) * uint32_t(sizeof(FiltSph) + sizeof(FiltHvy));
                     N.src = nv.fsph;
@@ -140,13 +153,18 @@ __global__ void __launch_bounds__(P + C, 2) k_dist_batched(BatchView bv, Basket 
             // have finished
             if (k >= 2) mbar_wait_bounded(&done[k & 1], uint32_t(((k - 2) >> 1) & 1), bv.status, healthy);
             if (t == 0) {
-                hd.tile = N.tile;
-                hd.base = N.base;
-                hd.count = N.count;
-                hd.vol_index = N.vol_index;
+                hd.tile = healthy ? N.tile : -1;
+                if (healthy) {
+                    hd.base = N.base;
+                    hd.count = N.count;
+                    hd.vol_index = N.vol_index;
+                    hd.staged = N.staged;
 #pragma unroll
-                for (int q = 0; q < kTaskBins; ++q) st_.cnt[q] = 0;
-                st_.next = 0;
+                    for (int q = 0; q < kTaskBins; ++q) st_.cnt[q] = 0;
+                    st_.next = 0;
+                } else if (N.staged) {
+                    N.owed |= (1u | uint32_t((k >> 1) & 1) << 2) << (k & 1);
+                }
             }
             producer_barrier<P>();
             const int tile = hd.tile;
@@ -162,9 +180,16 @@ __global__ void __launch_bounds__(P + C, 2) k_dist_batched(BatchView bv, Basket 
                 FiltTab f = {v.fsph, v.fhvy, v.nq1, v.nq, v.nf};
                 if (!GLOB) {
                     // every tile's copy is waited for, so none is in flight when the block ends
-                    if (!mbar_wait_limited(&tabs[k & 1], uint32_t((k >> 1) & 1), kWaitLimit)) {
+                    if (!hd.staged) {
+                        hd.vol.dd_min = f_inf();   // no direction is long enough for the FP32 pass
+                    } else if (!mbar_wait_limited(&tabs[k & 1], uint32_t((k >> 1) & 1), bv.table_polls)) {
+                        hd.vol.dd_min = f_inf();
                         atomicOr(bv.status, ST_TMA_TIMEOUT);
-                        healthy = false;
+                        atomicOr(v.status, ST_TMA_TIMEOUT);
+                        if (t == 0) {
+                            N.staging = 0;
+                            N.owed |= (1u | uint32_t((k >> 1) & 1) << 2) << (k & 1);
+                        }
                     }
                     const unsigned char* tab =
                         (k & 1) ? area + (room - uint32_t(v.nf) * uint32_t(sizeof(FiltSph) + sizeof(FiltHvy))) : area;
@@ -201,7 +226,10 @@ __global__ void __launch_bounds__(P + C, 2) k_dist_batched(BatchView bv, Basket 
                 }
                 const int slot = bin >= 0 ? atomicAdd(&st_.cnt[bin], 1) : 0;
                 producer_barrier<P>();
-                if (!GLOB && t == 0 && N.pending) copy_tables(k + 1);   // nobody reads the current tables any more
+                if (!GLOB && t == 0 && N.pending) {   // nobody reads the current tables any more
+                    if (N.staging) copy_tables(k + 1);
+                    else N.staged = 0;
+                }
                 if (bin >= 0) st_.task[bin_start(st_.cnt, bin) + slot] = t | ((task + 1) << kOwnerBits);
                 pad_bins<P>(st_, t);
                 if (rs.status == 0) {
@@ -220,6 +248,12 @@ __global__ void __launch_bounds__(P + C, 2) k_dist_batched(BatchView bv, Basket 
             __syncwarp();
             if (lane == 0) mbar_arrive(&full[k & 1]);
             if (tile < 0) break;
+        }
+        if (t == 0 && N.owed) {
+            for (int q = 0; q < bv.nvols; ++q) atomicOr(bv.vols[q].status, ST_TMA_TIMEOUT);
+            // do not leave while a late copy may still write this block's memory
+            for (int p = 0; p < 2; ++p)
+                if (N.owed >> p & 1u) mbar_wait_limited(&tabs[p], N.owed >> (2 + p) & 1u, kWaitLimit);
         }
     } else {
         // ------------------------------------------------------ consumers --

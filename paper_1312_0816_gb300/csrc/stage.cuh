@@ -11,7 +11,6 @@
 
 namespace geonav {
 
-constexpr uint32_t kWaitLimit = 1u << 22;
 constexpr uint32_t kChunk = 32768;   // bytes per bulk copy instruction
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) {

@@ -58,7 +58,7 @@ EXPORTS = ("geo_build_volume", "geo_destroy_volume", "geo_volume_info", "geo_dis
            "geo_dist_to_boundary_batched", "geo_dist_to_boundary_batched_noalloc", "geo_adjoint_workspace_size",
            "geo_dist_to_boundary_adjoint", "geo_shape_query", "geo_build_world", "geo_destroy_world",
            "geo_world_info", "geo_world_nodes", "geo_world_locate", "geo_world_step", "geo_selftest_wait_timeout",
-           "geo_debug_fail_alloc", "geo_status_string")
+           "geo_selftest_batch_timeout", "geo_debug_fail_alloc", "geo_status_string")
 
 
 def library_path() -> str:
@@ -99,6 +99,7 @@ def load(build_if_stale: bool = True):
                                   ctypes.POINTER(geo_batch_opts), vp, ctypes.POINTER(vp)]
     L.geo_destroy_batch.argtypes = [vp]
     L.geo_dist_to_boundary_batched.argtypes = [vp, dp, dp, dp, dp, dp, dp, i64, dp, ip, vp]
+    L.geo_selftest_batch_timeout.argtypes = L.geo_dist_to_boundary_batched.argtypes
     L.geo_dist_to_boundary_batched_noalloc.argtypes = [ctypes.POINTER(vp), i32, ctypes.POINTER(geo_basket), i32,
                                                        dp, dp, dp, dp, dp, dp, i64, dp, ip, vp]
     L.geo_adjoint_workspace_size.argtypes = [vp, i64, ctypes.POINTER(ctypes.c_uint64)]
@@ -474,6 +475,21 @@ def geo_selftest_wait_timeout(vol: Volume, polls: int = 256, stream=None):
     """Runs the failure path of a bounded wait (a barrier nobody arrives at);
     the volume's status word then holds bit 4 (see geo.h)."""
     _check(load().geo_selftest_wait_timeout(vol.handle, int(polls), _stream(stream)), "geo_selftest_wait_timeout")
+
+
+def geo_selftest_batch_timeout(batch: Batch, x, y, z, dx, dy, dz, stream=None):
+    """geo_dist_to_boundary_batched with every wait for a tile's tables given up
+    at once: the same answers, and bit 1 in the volumes' status words (see
+    geo.h)."""
+    torch = _th()
+    n = int(x.numel())
+    f64 = torch.float64
+    step = torch.empty(n, dtype=f64, device=x.device)
+    hit = torch.empty(n, dtype=torch.int32, device=x.device)
+    args = [_dev(a, f64, n, nm) for a, nm in ((x, "x"), (y, "y"), (z, "z"), (dx, "dx"), (dy, "dy"), (dz, "dz"))]
+    _check(load().geo_selftest_batch_timeout(batch.handle, *args, n, step.data_ptr(), hit.data_ptr(), _stream(stream)),
+           "geo_selftest_batch_timeout")
+    return step, hit
 
 
 def geo_debug_fail_alloc(nth: int):
