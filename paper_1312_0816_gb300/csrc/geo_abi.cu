@@ -214,15 +214,18 @@ bool inscribed_tube(const geo_placed_shape& s, geo_placed_shape& t) {
 }
 
 // plane table of a polycone (layout in geo_internal.h)
-std::vector<double> pcon_table_host(const geo_placed_shape& s) {
+void pcon_table_into(const geo_placed_shape& s, double* T) {
     const int n = pcon_nz(s);
-    std::vector<double> T(size_t(pcon_table_len(n)));
-    std::copy(s.planes, s.planes + 3 * n, T.begin());
+    std::copy(s.planes, s.planes + 3 * n, T);
     const double *z = s.planes, *rn = z + n, *rx = rn + n;
     for (int k = 0; k + 1 < n; ++k) {
         T[3 * n + k] = (rn[k + 1] - rn[k]) / (z[k + 1] - z[k]);
         T[3 * n + (n - 1) + k] = (rx[k + 1] - rx[k]) / (z[k + 1] - z[k]);
     }
+}
+std::vector<double> pcon_table_host(const geo_placed_shape& s) {
+    std::vector<double> T(size_t(pcon_table_len(pcon_nz(s))));
+    pcon_table_into(s, T.data());
     return T;
 }
 
@@ -441,6 +444,50 @@ std::vector<Cull64> make_cull(const geo_placed_shape* in, const std::vector<Shap
     return out;
 }
 
+// The filter's gathered record of daughter `id`, solid sh, whose FP32 copy is r
+// (layout in geo_internal.h).  hi, lo: of a quadric, the squared acceptance limits
+// of the end annuli at -dz, +dz.
+void filter_entry(const geo_placed_shape& sh, const ShapeRec32& r, int32_t id, FiltHvy& h, float* hi, float* lo) {
+    std::memset(&h, 0, sizeof h);
+    std::memcpy(h.t, r.t, sizeof h.t);
+    std::memcpy(h.R, r.R, sizeof h.R);
+    h.brad = r.brad;
+    h.delta = r.delta;
+    h.id = id;
+    h.flags = (r.flags & kRec32Identity) ? kFiltIdentity : 0;
+    if (r.kind == KBOX) {
+        std::memcpy(h.e, r.e, 3 * sizeof(float));
+        h.e[3] = r.delta;
+        h.flags |= kFiltBox;
+        return;
+    }
+    if (r.kind == KTUBE) {
+        const float e[5] = {r.e[2], r.e[7], 0.f, r.e[8], 0.f};
+        std::memcpy(h.e, e, sizeof e);
+        h.h = r.e[6];
+        hi[0] = hi[1] = r.e[4];
+        lo[0] = lo[1] = r.e[5];
+        if (r.e[3] != 0.f) h.flags |= kFiltHole;
+    } else {
+        std::memcpy(h.e, r.e, 5 * sizeof(float));
+        h.h = r.e[14];
+        hi[0] = r.e[10]; hi[1] = r.e[11];
+        lo[0] = r.e[12]; lo[1] = r.e[13];
+        if (r.e[5] != 0.f) h.flags |= kFiltHole;
+    }
+    h.e[5] = hi[0]; h.e[6] = hi[1]; h.e[7] = lo[0]; h.e[8] = lo[1];
+    const double slope = std::max(std::fabs(double(h.e[2])), std::fabs(double(h.e[4])));
+    h.g = float_up(2.0 * double(r.delta) * std::sqrt(1.0 + slope * slope));
+    const bool has_hole = sh.kind == GEO_TUBE ? sh.p[0] > 0 : (sh.kind == GEO_CONE && (sh.p[1] > 0 || sh.p[3] > 0));
+    if (sh.kind == GEO_CONE) {
+        const double r[5] = {sh.p[1], sh.p[2], sh.p[4], sh.p[3], sh.p[1]};
+        bool exact = true;
+        for (int q = 0; q < 4; ++q) exact = exact && r[q] + (r[q + 1] - r[q]) == r[q + 1];
+        if (exact) h.flags |= kFiltVertex;
+    }
+    if (needs_segs_code(sh) || (has_hole && !(h.flags & kFiltHole))) h.flags |= kFiltLoose;
+}
+
 // The filter's tables (layout in geo_internal.h) from the daughters `in` and
 // their FP32 copies: sorted by class, the daughters of a class in index order.
 void make_filter(const geo_placed_shape* in, const std::vector<ShapeRec32>& d, std::vector<FiltSph>& sph,
@@ -474,45 +521,8 @@ void make_filter(const geo_placed_shape* in, const std::vector<ShapeRec32>& d, s
             continue;
         }
         const ShapeRec32& r = d[order[k]];
-        std::memcpy(h.t, r.t, sizeof h.t);
-        std::memcpy(h.R, r.R, sizeof h.R);
-        h.brad = r.brad;
-        h.delta = r.delta;
-        h.id = order[k];
-        h.flags = (r.flags & kRec32Identity) ? kFiltIdentity : 0;
-        if (r.kind == KBOX) {
-            std::memcpy(h.e, r.e, 3 * sizeof(float));
-            h.e[3] = r.delta;
-            h.flags |= kFiltBox;
-            continue;
-        }
-        float hi[2], lo[2];   // squared acceptance limits of the end annuli at -dz, +dz
-        if (r.kind == KTUBE) {
-            const float e[5] = {r.e[2], r.e[7], 0.f, r.e[8], 0.f};
-            std::memcpy(h.e, e, sizeof e);
-            h.h = r.e[6];
-            hi[0] = hi[1] = r.e[4];
-            lo[0] = lo[1] = r.e[5];
-            if (r.e[3] != 0.f) h.flags |= kFiltHole;
-        } else {
-            std::memcpy(h.e, r.e, 5 * sizeof(float));
-            h.h = r.e[14];
-            hi[0] = r.e[10]; hi[1] = r.e[11];
-            lo[0] = r.e[12]; lo[1] = r.e[13];
-            if (r.e[5] != 0.f) h.flags |= kFiltHole;
-        }
-        h.e[5] = hi[0]; h.e[6] = hi[1]; h.e[7] = lo[0]; h.e[8] = lo[1];
-        const double slope = std::max(std::fabs(double(h.e[2])), std::fabs(double(h.e[4])));
-        h.g = float_up(2.0 * double(r.delta) * std::sqrt(1.0 + slope * slope));
-        const geo_placed_shape& sh = in[order[k]];
-        const bool has_hole = sh.kind == GEO_TUBE ? sh.p[0] > 0 : (sh.kind == GEO_CONE && (sh.p[1] > 0 || sh.p[3] > 0));
-        if (sh.kind == GEO_CONE) {
-            const double r[5] = {sh.p[1], sh.p[2], sh.p[4], sh.p[3], sh.p[1]};
-            bool exact = true;
-            for (int q = 0; q < 4; ++q) exact = exact && r[q] + (r[q + 1] - r[q]) == r[q + 1];
-            if (exact) h.flags |= kFiltVertex;
-        }
-        if (needs_segs_code(sh) || (has_hole && !(h.flags & kFiltHole))) h.flags |= kFiltLoose;
+        float hi[2], lo[2];
+        filter_entry(in[order[k]], r, order[k], h, hi, lo);
         if (k < nq1) {
             const bool axis = k % 32 == 0 || r.t[0] != sph[k - 1].a.x || r.t[1] != sph[k - 1].a.y;
             s.a = make_float4(r.t[0], r.t[1], r.t[2], axis ? 1.f : 0.f);
@@ -606,13 +616,10 @@ bool make_fast(const geo_placed_shape& s, ShapeFast& f) {
     geo_placed_shape own = s;   // in its own frame
     for (int k = 0; k < 9; ++k) own.rot[k] = k % 4 == 0 ? 1.0 : 0.0;
     for (int k = 0; k < 3; ++k) own.trans[k] = 0.0;
-    std::vector<ShapeRec32> r(1);
-    if (!make_rec32(s, dl, dl, r[0]) || !make_rec32(own, -dl, dl, f.m32) || !make_rec32(own, dl, dl, f.m32u)) return false;
-    std::vector<FiltSph> sph;
-    std::vector<FiltHvy> hvy;
-    int32_t nq1, nq;
-    make_filter(&s, r, sph, hvy, nq1, nq);
-    f.h = hvy[size_t(hvy[0].entry)];
+    ShapeRec32 r;   // (nothing is allocated here: the call takes place per query)
+    if (!make_rec32(s, dl, dl, r) || !make_rec32(own, -dl, dl, f.m32) || !make_rec32(own, dl, dl, f.m32u)) return false;
+    float hi[2], lo[2];
+    filter_entry(s, r, 0, f.h, hi, lo);
     if (f.h.flags & kFiltLoose) return false;
     f.m64 = make_rec64(s);
     f.reach = float(S / 1.8);   // |p| <= sqrt(3) max |p_k| < S
@@ -1364,10 +1371,7 @@ geo_status geo_shape_query(const geo_placed_shape* shape, int32_t what, const do
     ShapeArg a;
     std::memset(&a, 0, sizeof a);
     a.r = make_rec64(*shape);
-    if (shape->kind == GEO_PCON) {
-        const std::vector<double> T = pcon_table_host(*shape);
-        std::copy(T.begin(), T.end(), a.table);
-    }
+    if (shape->kind == GEO_PCON) pcon_table_into(*shape, a.table);
     const Basket b{x, y, z, dist ? dx : nullptr, dist ? dy : nullptr, dist ? dz : nullptr, n};
     return cuda_status(launch_shape_query(a, what, b, out, face, static_cast<cudaStream_t>(stream),
                                           num_sms_of(dev)));
