@@ -141,7 +141,10 @@ typedef enum {
  * queries.  A polycone's plane table travels in the kernel's parameters (the
  * call allocates nothing).  dx,dy,dz may be NULL for the safeties and Contains.
  * Non-finite input, or a zero direction for a distance: NaN.  The values are
- * those of the navigator's FP64 routines.  Errors: bad kind or parameters of
+ * those of the navigator's FP64 routines, bit for bit.  For boxes, tubes and
+ * cones FP32 may decide, by margins, which of a routine's surfaces the answer
+ * lies on and whether the solid is missed, holds the point or does not
+ * (Contains, and the others from 98304 points on); every number is FP64.  Errors: bad kind or parameters of
  * the solid (as geo_build_volume), bad query, host pointers. */
 geo_status geo_shape_query(const geo_placed_shape* shape, int32_t what, const double* x, const double* y,
                            const double* z, const double* dx, const double* dy, const double* dz, int64_t n,

@@ -624,6 +624,9 @@ bool make_fast(const geo_placed_shape& s, ShapeFast& f) {
     f.m64 = make_rec64(s);
     f.reach = float(S / 1.8);   // |p| <= sqrt(3) max |p_k| < S
     f.dd_min = dd_limit(S);
+    // FP32: 5e-6 of the largest coordinate; FP64's crossings (reach64): 3e-8 of the distance
+    f.grow = float(2.0 / f.reach);
+    f.far = float(3e-5 * reach64(s, S) / (2e-7 * (S + tn)));
     return true;
 }
 
@@ -1357,11 +1360,15 @@ geo_status geo_shape_query(const geo_placed_shape* shape, int32_t what, const do
     if (!is_device_ptr(out) || (face && !is_device_ptr(face))) return GEO_ERR_INVALID_ARG;
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return GEO_ERR_CUDA;
-    // the list kernel from 98304 points on (2^20: cone DistFromOutside 227 -> 65
-    // us, tube 202 -> 66, box 148 -> 30; safeties and DistFromInside 1.05 to 2.1
-    // times faster); below, its FP32 pass before the FP64 chain is the longer way
-    // (1024: tube 9.0 -> 12.2 us; 65536 about equal), except for Contains, which
-    // needs no FP64 (2.7 -> 2.3 and 39 -> 11 us)
+    // the list kernel from 98304 points on (k_shape -> k_shape_lists, us of 2^20 points
+    // within 1.5 radii: DistFromOutside box 149 -> 29, tube 203 -> 68, cone 229 -> 66;
+    // from inside 108 -> 27, 184 -> 62, 196 -> 57; the safeties 84 -> 70, 100 -> 84,
+    // 324 -> 140 and 55 -> 18, 78 -> 32, 100 -> 33; 30 radii away it is further ahead
+    // but for the tube's safety, 100 -> 98; on the surface, where FP32 decides least, from
+    // 12 % slower, box DistFromOutside 66 -> 74, to 16 % faster); below, its FP32 pass before the FP64
+    // chain is the longer way (1024: tube 9.0 -> 12.2 us; 65536 about equal), except
+    // for Contains, which needs almost no FP64 (1024 points 4.2 -> 4.1, 2^20 41 -> 10,
+    // on the surface 22.5 for both)
     ShapeFast fast;
     if ((what == GEO_Q_CONTAINS || n >= 98304) && make_fast(*shape, fast)) {
         const Basket b{x, y, z, dist ? dx : nullptr, dist ? dy : nullptr, dist ? dz : nullptr, n};

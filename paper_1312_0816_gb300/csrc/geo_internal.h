@@ -270,14 +270,16 @@ struct ShapeArg {
 };
 // The same for a box, tube or cone whose FP32 copies decide most of a query:
 // its placed copy (an entry of the filter's tables), the copies shrunk and
-// grown in its own frame, and the largest coordinate of a point and the least
-// |d|^2 they are good for.
+// grown in its own frame, the largest coordinate of a point and the least |d|^2
+// they are good for.  Beyond the reach, by the start's largest coordinate: the
+// rounding of a line that passes the solid, and the growth of the copies' margins.
 struct ShapeFast {
     ShapeRec64 m64;
     ShapeRec32 m32, m32u;
     FiltHvy h;
     float reach;
     float dd_min;
+    float far, grow;
 };
 cudaError_t launch_shape_lists(const ShapeFast& a, int what, const Basket& b, double* out, int32_t* face,
                                cudaStream_t s, int num_sms);

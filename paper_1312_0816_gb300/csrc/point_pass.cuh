@@ -101,15 +101,16 @@ __device__ __forceinline__ float entry_distance(const FiltHvy* h, const float* p
 
 // The zone of a point outside solid h (or surely inside it).  Every comparison
 // keeps 2 delta (times the slope's factor) from the solid's own limit, which
-// is the copy's less delta.
-__device__ __forceinline__ int entry_zone(const FiltHvy* h, const float* p) {
+// is the copy's less delta.  Of a point `grow` times beyond the extent that the copy
+// was made for, the FP32 rounding is that much larger, and so is what they keep.
+__device__ __forceinline__ int entry_zone(const FiltHvy* h, const float* p, const float grow = 1.f) {
     const float4* H = hvy_words(h);
     const float4 h0 = H[0], h3 = H[3], h4 = H[4];
     const int flags = __float_as_int(h3.y);
     float x[3];
     point_to_entry(H, h0, flags, h3.x, p, x);
     if (flags & kFiltBox) {
-        const float d = h4.w;
+        const float d = h4.w * grow;
         const float e[3] = {fabsf(x[0]) - h4.x, fabsf(x[1]) - h4.y, fabsf(x[2]) - h4.z};   // less delta
         int out = 0, in = 0, k = 0;
 #pragma unroll
@@ -125,11 +126,11 @@ __device__ __forceinline__ int entry_zone(const FiltHvy* h, const float* p) {
     }
     if (flags & kFiltLoose) return kZoneNone;
     const float4 h5 = H[5], h6 = H[6];
-    const float d = h6.z, m = h6.y;   // delta; 2 delta sqrt(1 + slope^2)
+    const float m = h6.y * grow;   // 2 delta sqrt(1 + slope^2)
     const bool hole = (flags & kFiltHole) != 0;
     const float rho = fsqrt(fmaf(x[0], x[0], x[1] * x[1]));
-    const float z = x[2], az = fabsf(z), dz = h4.x - d;
-    const float bo = h4.z, bi = h5.x, half = 0.5f * m;
+    const float z = x[2], az = fabsf(z), dz = h4.x - h6.z;
+    const float bo = h4.z, bi = h5.x, half = 0.5f * h6.y;
     const float ao = h4.y - half, ai = h4.w + half;   // the solid's own radius lines, to delta
     const float no = rho - fmaf(bo, z, ao), ni = hole ? fmaf(bi, z, ai) - rho : -1e30f;   // > 0: outside, in the hole
     const float zc = az - dz;

@@ -184,3 +184,49 @@ def test_starts_on_the_surface_of_the_mothers_hole(g, mother, copies):
             flag = torch.full((n,), f, dtype=torch.int32, device="cuda")
             assert same(g.geo_world_step(world, *t, node, flag, mode=g.GEO_FP64),
                         g.geo_world_step(world, *t, node, flag, mode=g.GEO_FP32_REFINE))
+
+
+@pytest.mark.parametrize("kind,prm", [(scenes.BOX, (3.0, 20.0, 11.0)), (scenes.TUBE, (0.0, 9.0, 14.0)),
+                                      (scenes.TUBE, (8.9, 9.0, 4.0)), (scenes.CONE, (5.0, 1.0, 30.0, 20.0, 21.0)),
+                                      (scenes.CONE, (30.0, 2.0, 4.0, 9.0, 9.0)), (scenes.CONE, (0.5, 2.0, 4.0, 30.0, 40.0))])
+@pytest.mark.parametrize("reach", [2.0, 9.0, 30.0, 1e3, 1e6, 1e12, 1e17, 1e200])
+def test_one_solid_from_afar(g, kind, prm, reach):
+    """Points up to `reach` times the solid's size away, half of them on its
+    surface or on lines that graze it, through the list kernels (from 98304 points
+    on; Contains always) against the whole routines'."""
+    rng = np.random.default_rng(int(np.log10(reach) * 10.0))
+    n, m = 98304, 90000
+    R, shift = scenes.haar_rotation(rng), np.array([7.0, -3.0, 5.0])
+    size = max(prm)
+    # points on the faces, and directions along them or anywhere
+    if kind == scenes.BOX:
+        q = rng.uniform(-1.0, 1.0, (n, 3))
+        q[np.arange(n), rng.integers(0, 3, n)] = rng.choice([-1.0, 1.0], n)
+        q *= np.array(prm)
+    else:
+        ends = (prm[0], prm[1], prm[0], prm[1], prm[2]) if kind == scenes.TUBE else (*prm[1:], prm[0])
+        f, ph = rng.uniform(0.0, 1.0, n), rng.uniform(0.0, 2.0 * np.pi, n)
+        f = np.where(rng.random(n) < 0.2, rng.integers(0, 2, n), f)
+        lo, hi = ends[0] + f * (ends[2] - ends[0]), ends[1] + f * (ends[3] - ends[1])
+        r = np.where(rng.random(n) < 0.5, hi, np.where(rng.random(n) < 0.5, lo, rng.uniform(0.0, 1.0, n) * (hi - lo) + lo))
+        q = np.stack([r * np.cos(ph), r * np.sin(ph), (2.0 * f - 1.0) * ends[4]], axis=1)
+    d = np.stack(scenes.isotropic(rng, n), axis=1)
+    graze = rng.random(n) < 0.3
+    d[graze, 2] = 0.0 if kind == scenes.TUBE else d[graze, 2]
+    radial = np.stack([-q[:, 1], q[:, 0], np.zeros(n)], axis=1) / np.maximum(np.hypot(q[:, 0], q[:, 1]), 1e-300)[:, None]
+    d[graze] = radial[graze] + 1e-3 * rng.normal(0.0, 1.0, (int(graze.sum()), 3)) * rng.integers(0, 2, (int(graze.sum()), 1))
+    away = size * reach ** rng.uniform(0.0, 1.0, (n, 1)) * rng.choice([0.0, 1.0, 1.0, 1.0], (n, 1)) * rng.choice([-1.0, 1.0], (n, 1))
+    p = q - d * away
+    anywhere = rng.random(n) < 0.4
+    p[anywhere] = rng.normal(0.0, 1.0, (int(anywhere.sum()), 3)) * size * reach ** rng.uniform(0.0, 1.0, (int(anywhere.sum()), 1))
+    A = R.reshape(3, 3)
+    t = cuda(*(p @ A.T + shift).T, *(d @ A.T).T)
+    for what in (g.GEO_Q_DIST_OUT, g.GEO_Q_DIST_IN, g.GEO_Q_SAFETY_OUT, g.GEO_Q_SAFETY_IN):
+        dist = what in (g.GEO_Q_DIST_OUT, g.GEO_Q_DIST_IN)
+        a = g.geo_shape_query(kind, prm, what, *t[:6 if dist else 3], rot=R, trans=shift, want_face=True)
+        b = g.geo_shape_query(kind, prm, what, *[x[:m].contiguous() for x in t[:6 if dist else 3]], rot=R, trans=shift,
+                              want_face=True)
+        assert same([x[:m] for x in a], b)
+        if what == g.GEO_Q_DIST_IN:   # the whole routine's face tells whether it holds the point
+            inside = g.geo_shape_query(kind, prm, g.GEO_Q_CONTAINS, *t[:3], rot=R, trans=shift) == 1.0
+            assert torch.equal(inside[:m] & ~torch.isnan(b[0]), b[1] >= 0)   # (NaN: no direction, on the axis)
