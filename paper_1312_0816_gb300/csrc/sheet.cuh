@@ -28,7 +28,7 @@ constexpr int kTaskNone = -1;
 // A track that its first task (solid h, value s) does not settle (0.02 %, out of
 // line): the FP32 pass again, for its whole list of candidates.  This copy of the
 // pass may round a bound differently (the compiler contracts each copy's expressions
-// by itself) and name another first task; the value is then formed for that one.  (Marking such tracks and
+// by itself) and name another first task; the loop over every daughter then decides.  (Marking such tracks and
 // taking them through the loop a second time: 748 us for 700 in the grid; two more
 // candidates kept per track: 709.)
 template <int TRAV>
@@ -36,13 +36,12 @@ static __device__ __noinline__ void refine_again(const VolView& v, double& s, do
                                                  double qy, double qz, int& h, int& nev) {
     const double pd[6] = {px, py, pz, qx, qy, qz};
     const int first = h;
-    double s_first = s;
+    const double s_first = s;
     RefineState rs;
     refine_pass1<TRAV, false>(v, FiltTab{v.fsph, v.fhvy, v.nq1, v.nq, v.nf}, GridTab{}, v.d64, px, py, pz, qx, qy, qz,
                               [&](int c) { return pd[c]; }, rs, s, h, nev);
     if (rs.status != 0) return;
-    const int task = first_task(rs);
-    if (task != first) s_first = eval64_cold(v, v.d64, task, px, py, pz, qx, qy, qz);
+    if (first_task(rs) != first) rs.c.dropped = 0.f;   // below any value
     refine_rest<false>(v, v.d64, rs, s_first, px, py, pz, qx, qy, qz, s, h, nev);
 }
 
