@@ -655,6 +655,10 @@ geo_status build_voxels(const geo_placed_shape& m, const geo_placed_shape* d, in
     if (mb.kind == GEO_BOX) { half[0] = p[0]; half[1] = p[1]; half[2] = p[2]; }
     else if (mb.kind == GEO_TUBE || mb.kind == GEO_TUBS) { half[0] = half[1] = p[1]; half[2] = p[2]; }
     else { half[0] = half[1] = std::max(p[2], p[4]); half[2] = p[0]; }
+    // A walk ends at the grid's walls.  They stand off the mother by more than the
+    // rounding of an FP32 start, so that a track is out of the mother before it comes
+    // to one; on her own walls a start that moves along one would seem to be through.
+    for (int k = 0; k < 3; ++k) half[k] += 4e-6 * S;
     int g[3];
     const int gauto = std::max(1, std::min(64, int(std::lround(2.0 * std::cbrt(double(std::max(nd, 1)))))));
     for (int k = 0; k < 3; ++k) g[k] = opts->grid[k] > 0 ? opts->grid[k] : gauto;

@@ -230,3 +230,39 @@ def test_one_solid_from_afar(g, kind, prm, reach):
         if what == g.GEO_Q_DIST_IN:   # the whole routine's face tells whether it holds the point
             inside = g.geo_shape_query(kind, prm, g.GEO_Q_CONTAINS, *t[:3], rot=R, trans=shift) == 1.0
             assert torch.equal(inside[:m] & ~torch.isnan(b[0]), b[1] >= 0)   # (NaN: no direction, on the axis)
+
+
+@pytest.mark.parametrize("cells", [(0, 0, 0), (7, 3, 40)])
+@pytest.mark.parametrize("half", [(90.0, 95.0, 100.0), (0.1, 70.0, 1.3)])
+def test_starts_along_a_wall_of_the_grid(g, half, cells):
+    """Tracks a rounding (FP32's or FP64's) inside a wall of the mother's box and
+    of the grid, moving along it and hardly towards it, with daughters flush with
+    the wall ahead."""
+    rng = np.random.default_rng(int(half[1]))
+    n = 200003
+    half = np.array(half)
+    rows = []
+    for k in range(3):
+        for side in (-1.0, 1.0):
+            for _ in range(10):
+                size = half * rng.uniform(0.03, 0.1, 3)
+                size[k] = half[k] / 16
+                at = rng.uniform(-0.85, 0.85, 3) * half
+                at[k] = side * (half[k] - size[k])
+                rows.append((scenes.BOX, size, EYE, at))
+    sc = scenes._scene("flush", scenes.BOX, half, rows)
+    face, side = rng.integers(0, 3, n), rng.choice([-1.0, 1.0], n)
+    i = np.arange(n)
+    p = rng.uniform(-1.0, 1.0, (3, n)) * half[:, None]
+    p[face, i] = side * half[face] * (1.0 - rng.choice([0.0, 1e-15, 1e-14, 1e-12, 1e-9, 1e-8, 1e-7], n))
+    d = np.stack(scenes.isotropic(rng, n))
+    d[face, i] = side * rng.choice([0.0, 1e-20, 1e-18, 1e-16, 1e-14, 1e-12, 1e-10, 1e-8], n)
+    t = cuda(*p, *d)
+    flat, grid = g.geo_build_volume(sc), g.geo_build_volume(sc, voxelize=True, grid=cells)
+    ref = g.geo_dist_to_boundary(flat, *t, mode=g.GEO_FP64)
+    assert int((ref[1] >= 0).sum()) > n // 20
+    assert same(ref, g.geo_dist_to_boundary(flat, *t, mode=g.GEO_FP32_REFINE))
+    assert same(ref, g.geo_dist_to_boundary(grid, *t, mode=g.GEO_FP64))
+    assert same(ref, g.geo_dist_to_boundary(grid, *t, mode=g.GEO_FP32_REFINE))
+    assert same([x[:60000] for x in ref], g.geo_dist_to_boundary(grid, *[x[:60000].contiguous() for x in t]))
+    assert same(ref, g.geo_dist_to_boundary_batched(g.geo_build_batch([grid], [(0, 0, n)]), *t))
