@@ -232,6 +232,67 @@ def test_one_solid_from_afar(g, kind, prm, reach):
             assert torch.equal(inside[:m] & ~torch.isnan(b[0]), b[1] >= 0)   # (NaN: no direction, on the axis)
 
 
+MOTHERS = {**HOLED, "box": (scenes.BOX, (90.0, 95.0, 100.0)), "rod": (scenes.TUBE, (0.0, 90.0, 100.0)),
+           "plug": (scenes.CONE, (100.0, 0.0, 90.0, 0.0, 120.0))}
+
+
+@pytest.mark.parametrize("daughters", ["few", "many", "overlapping"])
+@pytest.mark.parametrize("mother", sorted(MOTHERS))
+def test_starts_on_the_mothers_surface(g, mother, daughters):
+    """Tracks that start on a face of their mother, a rounding or up to 1e-3 of
+    her size inside, in any direction, along the face or nearly so: the mother's
+    exit is bounded there as for a track that has just entered."""
+    rng = np.random.default_rng(len(mother) * 10 + len(daughters))
+    n = 200003
+    kind, prm = MOTHERS[mother]
+    count = {"few": 12, "many": 60, "overlapping": 40}[daughters]
+    rows = []
+    for k in range(count):
+        a, r = 2.0 * np.pi * k / min(count, 12), rng.uniform(60.0, 68.0)
+        size = rng.uniform(2.0, 8.0 if daughters != "overlapping" else 12.0, 3)   # inside the outer surface
+        at = (r * np.cos(a), r * np.sin(a), rng.uniform(-79.0, 79.0))
+        solid = [(scenes.BOX, size), (scenes.TUBE, (0.3 * size[0], size[0], size[1])),
+                 (scenes.CONE, (size[2], 0.1, size[0], 0.2, size[1]))][k % 3]
+        rows.append((*solid, scenes.haar_rotation(rng) if k % 2 else EYE, at))
+    sc = scenes._scene("skin", kind, prm, rows)
+    face, ph = rng.integers(0, 3, n), rng.uniform(0.0, 2.0 * np.pi, n)
+    z = np.where(face == 0, 100.0 * rng.choice([-1.0, 1.0], n), rng.uniform(-100.0, 100.0, n))
+    if kind == scenes.BOX:
+        p = rng.uniform(-1.0, 1.0, (3, n)) * np.array(prm)[:, None]
+        p[face, np.arange(n)] = np.array(prm)[face] * rng.choice([-1.0, 1.0], n)
+        normal = np.zeros((3, n))
+        normal[face, np.arange(n)] = np.sign(p[face, np.arange(n)])
+    else:
+        if kind == scenes.PCON:
+            zp, rn, rx = sc.planes_of(sc.mother_params)
+        else:
+            zp = np.array([-100.0, 100.0])
+            rn, rx = ((np.array([prm[1], prm[3]]), np.array([prm[2], prm[4]])) if kind == scenes.CONE
+                      else (np.full(2, prm[0]), np.full(2, prm[1])))
+        ro, ri = np.interp(z, zp, rx), np.interp(z, zp, rn)
+        r = np.where(face == 0, ri + rng.uniform(0.0, 1.0, n) * (ro - ri), np.where(face == 1, ro, ri))
+        p = np.stack([r * np.cos(ph), r * np.sin(ph), z])
+        side = np.where(face == 1, 1.0, -1.0)
+        normal = np.where(face == 0, np.stack([0.0 * z, 0.0 * z, np.sign(z)]), np.stack([side * np.cos(ph), side * np.sin(ph), 0.0 * z]))
+    depth = rng.choice([0.0, 1e-15, 1e-13, 1e-9, 1e-6, 1e-5, 1e-4, 1e-3], n) * 100.0
+    p = p - normal * depth
+    d = np.stack(scenes.isotropic(rng, n))
+    flat_along = rng.random(n) < 0.3   # along the face, but for a little
+    along = d - normal * (normal * d).sum(axis=0)
+    d = np.where(flat_along, along + normal * rng.choice([0.0, 1e-12, 1e-7, 1e-4], n) * rng.choice([-1.0, 1.0], n), d)
+    t = cuda(*p, *d)
+    flat, grid = g.geo_build_volume(sc), g.geo_build_volume(sc, voxelize=True)
+    ref = g.geo_dist_to_boundary(flat, *t, mode=g.GEO_FP64)
+    assert int((ref[1] > -2).sum()) > n // 4
+    assert same(ref, g.geo_dist_to_boundary(flat, *t, mode=g.GEO_FP32_REFINE))
+    assert same(ref, g.geo_dist_to_boundary(grid, *t, mode=g.GEO_FP64))
+    assert same(ref, g.geo_dist_to_boundary(grid, *t, mode=g.GEO_FP32_REFINE))
+    assert same(ref, g.geo_dist_to_boundary_batched(g.geo_build_batch([flat], [(0, 0, n)]), *t))
+    assert same(ref, g.geo_dist_to_boundary_batched(g.geo_build_batch([grid], [(0, 0, n)]), *t))
+    few = [x[:1000].contiguous() for x in t]
+    assert same([x[:1000] for x in ref], g.geo_dist_to_boundary(flat, *few, mode=g.GEO_FP32_REFINE))
+
+
 @pytest.mark.parametrize("cells", [(0, 0, 0), (7, 3, 40)])
 @pytest.mark.parametrize("half", [(90.0, 95.0, 100.0), (0.1, 70.0, 1.3)])
 def test_starts_along_a_wall_of_the_grid(g, half, cells):
