@@ -41,45 +41,6 @@ __global__ void __launch_bounds__(256) k_dist_vox64(VolView v, Basket b, double*
     }
 }
 
-// tube_out64 and cone_out64 (no apex on an end plane) in one path, so that
-// lanes with either kind run it together: a tube is a cone of slope 0 whose
-// outer and inner C keep the rounded squares of its radii (surface64 in
-// nav_refine.cuh has the argument that the bits are the same).
-__device__ __forceinline__ double quad_out64(const ShapeRec64& r, const double* x, const double* u) {
-    const double* d = r.d;
-    const bool tube = r.kind == KTUBE;
-    const double dz = tube ? d[2] : d[0], bo = tube ? 0.0 : d[2], bi = tube ? 0.0 : d[4];
-    const double rho2 = rho2_of(x);
-    // -1 * R^2 (tube), -R * R (cone)
-    const double ro0 = tube ? 1.0 : FMA(bo, x[2], d[1]), ri0 = tube ? 1.0 : FMA(bi, x[2], d[3]);
-    const double ro1 = tube ? d[4] : ro0, ri1 = tube ? d[3] : ri0;
-    const bool hole = tube ? IS_POS(d[0]) : !IS_ZERO(d[11]);
-    if (ABS_LE(x[2], dz) && LE(rho2, MUL(ro0, ro1)) && (!hole || LE(MUL(ri0, ri1), rho2))) return 0.0;
-    double best = d_inf();
-    const bool zc = ABS_GT(x[2], dz) && OPPOSITE(x[2], u[2]);
-    if (zc) {   // the z-plane the track approaches from outside the slab
-        const double t = DIV(SUB(copysign(dz, x[2]), x[2]), u[2]);
-        const double xh = FMA(t, u[0], x[0]), yh = FMA(t, u[1], x[1]);
-        const double r2 = DOT2(xh, xh, yh, yh);
-        const double lo2 = tube ? d[3] : (IS_POS(x[2]) ? d[7] : d[5]);
-        const double hi2 = tube ? d[4] : (IS_POS(x[2]) ? d[8] : d[6]);
-        if (LE(r2, hi2) && LE(lo2, r2)) best = t;
-    }
-    const double A0 = DOT2(u[0], u[0], u[1], u[1]);
-    const double B0 = DOT2(x[0], u[0], x[1], u[1]);
-    {   // outer surface, crossed inwards
-        const double rs = MUL(bo, u[2]);
-        const double s = root_falling(FMA(-rs, rs, A0), FMA(-ro0, rs, B0), FMA(-ro0, ro1, rho2));
-        if (NONNEG(s) && LT(s, best) && ABS_LE(FMA(s, u[2], x[2]), dz)) best = s;
-    }
-    if (hole) {   // inner surface, crossed outwards (out of the hole)
-        const double rs = MUL(bi, u[2]);
-        const double s = root_rising(FMA(-rs, rs, A0), FMA(-ri0, rs, B0), FMA(-ri0, ri1, rho2));
-        if (NONNEG(s) && LT(s, best) && ABS_LE(FMA(s, u[2], x[2]), dz)) best = s;
-    }
-    return best;
-}
-
 template <bool SEGS>
 static __device__ __noinline__ void nav_all64_far(const ShapeRec64& m, const ShapeRec64* __restrict__ tab, int nd,
                                                   double px, double py, double pz, double qx, double qy, double qz,

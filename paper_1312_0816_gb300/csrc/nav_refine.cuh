@@ -423,10 +423,15 @@ static __device__ __noinline__ void refine_rest(const VolView& v, const ShapeRec
     }
 }
 
-// a track whose first task is not certain: the whole solid (rare, out of line)
+// a track whose first task is not certain: the whole solid (rare, out of line; tubes
+// and cones in one path, since a warp may hold both)
 static __device__ __noinline__ double eval64_cold(const VolView& v, const ShapeRec64* __restrict__ tab64, int j, double px,
                                                   double py, double pz, double qx, double qy, double qz) {
-    return eval64<false>(v, tab64, j, px, py, pz, qx, qy, qz);
+    if (j < 0) return eval64<false>(v, tab64, j, px, py, pz, qx, qy, qz);
+    const ShapeRec64& r = tab64[j];
+    double x[3], u[3];
+    to_local64(r, px, py, pz, qx, qy, qz, x, u);
+    return r.kind == KBOX ? box_out64(r.d, x, u) : quad_out64(r, x, u);
 }
 
 // The FP64 part of a track after its FP32 pass.

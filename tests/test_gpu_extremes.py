@@ -327,3 +327,35 @@ def test_starts_along_a_wall_of_the_grid(g, half, cells):
     assert same(ref, g.geo_dist_to_boundary(grid, *t, mode=g.GEO_FP32_REFINE))
     assert same([x[:60000] for x in ref], g.geo_dist_to_boundary(grid, *[x[:60000].contiguous() for x in t]))
     assert same(ref, g.geo_dist_to_boundary_batched(g.geo_build_batch([grid], [(0, 0, n)]), *t))
+
+
+@pytest.mark.parametrize("scene", ["toy8", "toy40", "grid512"])
+def test_starts_on_the_daughters_surfaces(g, scene):
+    """Tracks that start where an earlier step ended, or a little beside it, in any
+    direction: FP32 is certain of nothing there, and whole solids are evaluated.
+    The reference walks a grid of one cell with the shapes' own functions."""
+    sc = scenes.SCENES[scene]()
+    rng = np.random.default_rng(9)
+    n = 260011
+    tr = scenes.sample_tracks(sc, n, 9)
+    t = cuda(*tr.fields())
+    flat, walk, grid = (g.geo_build_volume(sc, **o) for o in ({}, {"voxelize": True, "grid": (1, 1, 1)}, {"voxelize": True}))
+    s, h = g.geo_dist_to_boundary(walk, *t, mode=g.GEO_FP64)
+    i = torch.nonzero(h >= 0).flatten()
+    i = i[torch.from_numpy(rng.integers(0, i.numel(), n)).cuda()]
+    s = s[i] + torch.from_numpy(rng.choice([0.0, 0.0, -1e-12, 1e-12, -1e-9, 1e-9, -1e-4, 1e-4], n)).cuda()
+    p = [(t[k][i] + s * t[3 + k][i]).contiguous() for k in range(3)]
+    q = p + cuda(*np.stack(scenes.isotropic(rng, n)))
+    ref = g.geo_dist_to_boundary(walk, *q, mode=g.GEO_FP64)
+    for v in (flat, grid):
+        for m in (n, 60011):
+            part = [x[:m].contiguous() for x in q]
+            assert same([x[:m] for x in ref], g.geo_dist_to_boundary(v, *part, mode=g.GEO_FP32_REFINE))
+    assert same(ref, g.geo_dist_to_boundary(flat, *q, mode=g.GEO_FP64))
+    for v in (flat, grid):
+        assert same(ref, g.geo_dist_to_boundary_batched(g.geo_build_batch([v], [(0, 0, n)]), *q))
+    for m in (n, 60011, 1009):
+        part = [x[:m].contiguous() for x in p]
+        assert torch.equal(g.geo_contains(flat, *part, mode=g.GEO_FP64), g.geo_contains(flat, *part))
+        a, b = g.geo_safety(flat, *part, mode=g.GEO_FP64), g.geo_safety(flat, *part)
+        assert torch.equal(a.view(torch.int64), b.view(torch.int64))
