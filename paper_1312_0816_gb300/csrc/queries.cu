@@ -241,10 +241,11 @@ __global__ void __launch_bounds__(256) k_contains_lists(const __grid_constant__ 
     }
 }
 
-// Safety: each warp takes `per` points at a time (128, or fewer where that
-// would leave warps without points); the FP32 pass runs 32 of them at a time
-// and sorts them by their FP64 work (zone_sort), which then runs 32 points
-// of one sort at a time (an FP64 instruction holds its unit for 64 cycles
+// Safety: the basket is shared equally by all resident warps (toy detector, 524288
+// points: 98 us with whole batches of 128 dealt in turn, 88 so; 203 and 176 for points
+// on the daughters' surfaces).  Each takes up to 128 points at a time; the FP32 pass
+// runs 32 of them at a time and sorts them by their FP64 work (zone_sort), which then
+// runs 32 points of one sort at a time (an FP64 instruction holds its unit for 64 cycles
 // however few lanes take part).  Everything is the warp's own, so there is no barrier.
 //
 // What bounds it: issue slots (62 %) and the FP64 unit (50 %): 2260 warp
@@ -279,7 +280,7 @@ static __device__ __noinline__ double safety_all_cold(const VolView& v, double s
 
 template <bool SMEM>
 __global__ void __launch_bounds__(kSafWarps * 32, 4)
-    k_safety_zones(const __grid_constant__ VolView v, const __grid_constant__ Basket b, double* __restrict__ saf, int per) {
+    k_safety_zones(const __grid_constant__ VolView v, const __grid_constant__ Basket b, double* __restrict__ saf) {
     extern __shared__ __align__(128) unsigned char smem_raw[];
     __shared__ uint64_t bar;
     __shared__ ShapeRec64 m64;
@@ -291,16 +292,16 @@ __global__ void __launch_bounds__(kSafWarps * 32, 4)
     __syncthreads();
     SafetyBatch& B = reinterpret_cast<SafetyBatch*>(smem_raw)[warp];
     const float tau = safety_tau(v);
-    const int64_t nbatch = (b.n + per - 1) / per;
-    const int64_t stride = int64_t(gridDim.x) * kSafWarps;
-    for (int64_t q = int64_t(blockIdx.x) * kSafWarps + warp; q < nbatch; q += stride) {
-        const int64_t first = q * per;
+    // an equal share of the basket, in whole groups of 32 points, for every warp
+    const int64_t share = int64_t(blockIdx.x) * kSafWarps + warp, shares = int64_t(gridDim.x) * kSafWarps;
+    const int64_t groups = (b.n + 31) >> 5, end = min((groups * (share + 1) / shares) << 5, b.n);
+    for (int64_t first = (groups * share / shares) << 5; first < end; first += kSafBatch) {
+        const int per = int(min(end - first, int64_t(kSafBatch)));
         int cnt[kZoneSorts] = {0, 0, 0, 0};
-        for (int o = lane; o < per; o += 32) {
+        for (int o = lane; o - lane < per; o += 32) {
             const int64_t i = first + o;
-            if (i - lane >= b.n) break;   // warp-uniform
             int sort = -1;
-            if (i < b.n) {
+            if (o < per) {
                 const double px = b.x[i], py = b.y[i], pz = b.z[i];
                 const float p[3] = {f64_to_f32_trunc(px), f64_to_f32_trunc(py), f64_to_f32_trunc(pz)};
                 const bool surely = contains32(v.m32, p);
@@ -413,13 +414,8 @@ cudaError_t launch_safety_filter(const VolView& v, const Basket& b, double* saf,
     // with k_safety_zones, eight solids of the toy detector 16.0 against 17.3;
     // from 100000 points on 10.7 / 10.8 and 27.6 / 24.2; 40 solids 36.8 / 20.5)
     if (v.nd <= 8 && b.n <= 32768) return launch32(k_safety32<true, false>, k_safety32<false, false>, v, b, s, num_sms, saf);
-    // the basket spread over all resident warps, 32 to 128 points each (toy
-    // detector, 1024 points: 35 us with 128 points each, 18.5 so)
-    const int64_t warps = int64_t(4) * num_sms * kSafWarps;
-    const int64_t share = (b.n + warps * 32 - 1) / (warps * 32) * 32;
-    const int per = int(share < kSafBatch ? share : kSafBatch);
     return launch_lists(k_safety_zones<true>, k_safety_zones<false>, kSafWarps * int(sizeof(SafetyBatch)), v, b, s, num_sms,
-                        saf, per);
+                        saf);
 }
 
 }  // namespace geonav
