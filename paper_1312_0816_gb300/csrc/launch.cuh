@@ -42,11 +42,36 @@ static inline int blocks_for(K kernel, int64_t n, int smem, int num_sms, int thr
 
 // Lets a kernel take `smem` bytes of dynamic shared memory.  The limit that
 // holds without this (48 KB) counts the kernel's static shared memory too, of
-// which the callers' kernels have up to 16 KB.
+// which the callers' kernels have up to 16 KB.  The limit is set to all that the device
+// gives, never to this call's size: it belongs to the kernel, and another thread
+// could lower it to its own size before this one launches.  Each thread keeps the
+// limits it has set.
+static inline cudaError_t raise_smem(const void* kernel, int smem) {
+    struct Entry {
+        const void* kernel;
+        int device, most;
+    };
+    constexpr int kEntries = 64;
+    static thread_local Entry cache[kEntries];
+    static thread_local int used = 0;
+    int device = 0, most = 0;
+    cudaError_t e = cudaGetDevice(&device);
+    if (e != cudaSuccess) return e;
+    for (int k = 0; k < used; ++k)
+        if (cache[k].kernel == kernel && cache[k].device == device)
+            return smem <= cache[k].most ? cudaSuccess : cudaErrorInvalidValue;
+    cudaFuncAttributes a;
+    if ((e = cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, device)) != cudaSuccess ||
+        (e = cudaFuncGetAttributes(&a, kernel)) != cudaSuccess)
+        return e;
+    most -= int(a.sharedSizeBytes);
+    if ((e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, most)) != cudaSuccess) return e;
+    if (used < kEntries) cache[used++] = {kernel, device, most};
+    return smem <= most ? cudaSuccess : cudaErrorInvalidValue;
+}
 template <typename K>
 static inline cudaError_t prep(K kernel, int smem) {
-    if (smem > 32 * 1024) return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    return cudaSuccess;
+    return smem > 32 * 1024 ? raise_smem(reinterpret_cast<const void*>(kernel), smem) : cudaSuccess;
 }
 
 }  // namespace geonav

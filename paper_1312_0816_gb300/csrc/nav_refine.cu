@@ -330,8 +330,7 @@ template <bool GLOB, int P, int C>
 static cudaError_t launch_batched(const BatchView& bv, const Basket& b, double* step, int32_t* hit, int blocks_per_sm,
                                   uint32_t room, cudaStream_t s, int num_sms) {
     const int smem = 2 * int(sizeof(Stage<P>) + sizeof(TileHdr)) + (GLOB ? 0 : int(room));
-    cudaError_t e =
-        cudaFuncSetAttribute(k_dist_batched<GLOB, P, C>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    cudaError_t e = prep(k_dist_batched<GLOB, P, C>, smem);
     if (e != cudaSuccess) return e;
     const int maxb = resident_blocks(reinterpret_cast<const void*>(k_dist_batched<GLOB, P, C>), P + C, smem);
     const int per_sm = (blocks_per_sm <= 0 || blocks_per_sm > maxb) ? maxb : blocks_per_sm;
