@@ -222,7 +222,7 @@ __global__ void __launch_bounds__(P + C, 2) k_dist_batched(BatchView bv, Basket 
                 int task = 0, bin = -1;
                 if (rs.status == 0) {
                     task = first_task(rs);
-                    bin = task_bin<true>(rs.tag, task, v.d64);
+                    bin = task_bin(rs.tag, task, v.d64);
                 }
                 const int slot = bin >= 0 ? atomicAdd(&st_.cnt[bin], 1) : 0;
                 producer_barrier<P>();
@@ -269,7 +269,7 @@ __global__ void __launch_bounds__(P + C, 2) k_dist_batched(BatchView bv, Basket 
             const int64_t* idx = bv.idx;
             // the outputs are in device memory: each track is stored as it is
             // finished (staging the tile's answers was 4 % slower here)
-            drain_tasks<true, P, false>(v, v.d64, v.m64, st_, nullptr, [=](int o) { return packed ? idx[base + o] : base + o; },
+            drain_tasks<P, false>(v, v.d64, v.m64, st_, nullptr, [=](int o) { return packed ? idx[base + o] : base + o; },
                                         b.n, step, hit);
             __syncwarp();
             if (lane == 0) mbar_arrive(&done[k & 1]);

@@ -21,9 +21,8 @@ namespace geonav {
 // leave gaps, so one warp cannot keep its unit busy and two do better.
 // This kernel serves volumes with tube segments, polycones or apex cones, whose
 // tracks need whole solids of differing kinds in FP64, with or without a uniform
-// grid; nav_refine_direct.cu and nav_refine_grid.cu serve the others.  (While it served those too, the toy
-// detector's 2^20 tracks took 0.222 ms with 12 + 4 warps, 0.257 with 12 + 2 at 72
-// registers, 0.248 with 11 + 3, 0.264 with 9 + 3 at 80 registers.)
+// grid; nav_refine_direct.cu and nav_refine_grid.cu serve the others.  (The times
+// below are the toy detector's, of when it took this kernel.)
 //  producers: wait done[k%2] (the stage's previous tile, k-2, finished), FP32
 //             pass of tile k, bin each track's first FP64 task (a sure plane
 //             or quadric, or a whole solid by its kind) into stage k%2, arrive
@@ -57,12 +56,9 @@ static_assert(kProd <= (1 << kOwnerBits) && kProd % 32 == 0 && kLatProd % 32 == 
 // (and tube segment), cone (and polycone).
 constexpr int kTaskBins = 6;
 __device__ __forceinline__ int kind_bin(int kind) { return kind == KTUBS ? 2 : (kind == KPCON ? 3 : 1 + kind); }
-// KINDS = false: whole solids are rare and share one bin (the all-daughter pass
-// in volumes without segments and polycones).
-template <bool KINDS>
 __device__ __forceinline__ int task_bin(int tag, int task, const ShapeRec64* __restrict__ tab64) {
     if (tag != kTagNone) return tag == kTagOuter || tag == kTagInner ? 1 : 0;
-    return !KINDS || task < 0 ? 2 : 2 + kind_bin(tab64[task].kind);
+    return task < 0 ? 2 : 2 + kind_bin(tab64[task].kind);
 }
 
 template <int P>
@@ -141,7 +137,7 @@ __device__ __forceinline__ void mbar_wait_bounded(uint64_t* bar, uint32_t parity
 // consecutive lanes (the tasks themselves are in kind order: their own
 // stores would scatter, which outputs in host memory written over the host
 // link pay for); or it is stored right away to index(o).
-template <bool SEGS, int P, bool STAGED, typename Index>
+template <int P, bool STAGED, typename Index>
 __device__ __forceinline__ void finish_track(const VolView& v, const ShapeRec64* __restrict__ tab64,
                                              const ShapeRec64& m64, const Stage<P>& st, Answers<P>* ans, int o, int jj, Index index,
                                              int64_t n, double* __restrict__ step, int32_t* __restrict__ hit) {
@@ -149,7 +145,7 @@ __device__ __forceinline__ void finish_track(const VolView& v, const ShapeRec64*
     double s_first;
     if (tag == kTagNone) {
         s_first =
-            eval64<SEGS>(v, tab64, jj, st.pd[0][o], st.pd[1][o], st.pd[2][o], st.pd[3][o], st.pd[4][o], st.pd[5][o]);
+            eval64<true>(v, tab64, jj, st.pd[0][o], st.pd[1][o], st.pd[2][o], st.pd[3][o], st.pd[4][o], st.pd[5][o]);
     } else {
         s_first = surface64(jj < 0 ? m64 : tab64[jj], tag, jj < 0, st.pd[0][o], st.pd[1][o], st.pd[2][o], st.pd[3][o],
                             st.pd[4][o], st.pd[5][o]);
@@ -167,7 +163,7 @@ __device__ __forceinline__ void finish_track(const VolView& v, const ShapeRec64*
     double best;
     int h, nev = 1;
     if (!refine_fast(rs, s_first, best, h))
-        refine_rest<SEGS>(v, tab64, rs, s_first, st.pd[0][o], st.pd[1][o], st.pd[2][o], st.pd[3][o], st.pd[4][o],
+        refine_rest<true>(v, tab64, rs, s_first, st.pd[0][o], st.pd[1][o], st.pd[2][o], st.pd[3][o], st.pd[4][o],
                           st.pd[5][o], best, h, nev);
     if (STAGED) {
         ans->best[o] = best;
@@ -200,7 +196,7 @@ __device__ __forceinline__ void store_tile(const Stage<P>& st, const Answers<P>&
 // A warp's share of a stage's FP64 tasks: it claims chunks of 32 tasks (one
 // bin-aligned chunk, so one solid kind) from the stage's counter until none
 // is left, and finishes their tracks.  Every lane of the warp takes part.
-template <bool SEGS, int P, bool STAGED, typename Index>
+template <int P, bool STAGED, typename Index>
 __device__ __forceinline__ void drain_tasks(const VolView& v, const ShapeRec64* __restrict__ tab64,
                                             const ShapeRec64& m64, Stage<P>& st,
                                             Answers<P>* ans, Index index, int64_t n, double* __restrict__ step,
@@ -215,7 +211,7 @@ __device__ __forceinline__ void drain_tasks(const VolView& v, const ShapeRec64* 
         const int e = st.task[q0 + lane];
         if (e >= 0) {
             const int o = e & ((1 << kOwnerBits) - 1), jj = (e >> kOwnerBits) - 1;
-            finish_track<SEGS, P, STAGED>(v, tab64, m64, st, ans, o, jj, index, n, step, hit);
+            finish_track<P, STAGED>(v, tab64, m64, st, ans, o, jj, index, n, step, hit);
         }
     }
 }
@@ -225,7 +221,7 @@ __device__ __forceinline__ void producer_barrier() { asm volatile("bar.sync 1, %
 template <int C>
 __device__ __forceinline__ void consumer_barrier() { asm volatile("bar.sync 2, %0;" ::"r"(C) : "memory"); }
 
-template <int P, int C, int SMEM, int TRAV, bool SEGS>
+template <int P, int C, int SMEM, int TRAV>
 __global__ void __launch_bounds__(P + C, 2) k_dist_refine(const __grid_constant__ VolView v, Basket b, double* __restrict__ step,
                                                              int32_t* __restrict__ hit,
                                                              double* __restrict__ bpoint,
@@ -287,12 +283,12 @@ __global__ void __launch_bounds__(P + C, 2) k_dist_refine(const __grid_constant_
             int h = -2, nev = 0;
             rs.status = 1;
             if (live)
-                refine_pass1<TRAV, SEGS>(v, f, GridTab{}, tab64, px, py, pz, qx, qy, qz, [&](int c) { return st_.pd[c][t]; }, rs, best,
+                refine_pass1<TRAV, true>(v, f, GridTab{}, tab64, px, py, pz, qx, qy, qz, [&](int c) { return st_.pd[c][t]; }, rs, best,
                                          h, nev);
             int task = 0, bin = -1;
             if (rs.status == 0) {
                 task = first_task(rs);
-                bin = task_bin<SEGS || TRAV == kTravGrid>(rs.tag, task, tab64);
+                bin = task_bin(rs.tag, task, tab64);
             }
             if (t < kTaskBins) st_.cnt[t] = 0;
             if (t == kTaskBins) st_.next = 0;
@@ -328,7 +324,7 @@ __global__ void __launch_bounds__(P + C, 2) k_dist_refine(const __grid_constant_
             const int64_t base = (int64_t(blockIdx.x) + int64_t(k) * gridDim.x) * P;
             const bool ok = __all_sync(0xffffffffu, healthy);   // a stage never filled is not read
             auto index = [base](int o) { return base + o; };
-            if (ok) drain_tasks<SEGS, P, true>(v, tab64, m64, S[k & 1], &A[k & 1], index, b.n, step, hit);
+            if (ok) drain_tasks<P, true>(v, tab64, m64, S[k & 1], &A[k & 1], index, b.n, step, hit);
             consumer_barrier<C>();   // every answer of the tile is in its answer buffer
             if (ok) store_tile<P, C>(S[k & 1], A[k & 1], c, index, b.n, step, hit, bpoint, nref);
             __syncwarp();
@@ -354,8 +350,6 @@ static cudaError_t launch_refine(K kernel, int smem, const VolView& v, const Bas
     return cudaGetLastError();
 }
 
-// SEGS: the instantiation with the tube segment's and the polycone's code
-// only for volumes that hold one, so the others keep the leaner kernel
 template <int P, int C>
 static cudaError_t launch_refine_cfg(const VolView& v, const Basket& b, double* step, int32_t* hit, double* bpoint,
                                      int32_t* nref, cudaStream_t s, int num_sms) {
@@ -367,16 +361,16 @@ static cudaError_t launch_refine_cfg(const VolView& v, const Basket& b, double* 
         // the grid walk needs registers: 12 + 2 warps at 72 registers beat
         // 12 + 4 at 64 (7.0 against 7.4 ms for 2^24 tracks in 512 daughters)
         constexpr int CV = P == kProd ? kVoxCons : C;
-        return launch_refine<P, CV>(k_dist_refine<P, CV, 0, kTravGrid, true>, stages, v, b, step, hit, bpoint, nref, s,
+        return launch_refine<P, CV>(k_dist_refine<P, CV, 0, kTravGrid>, stages, v, b, step, hit, bpoint, nref, s,
                                     num_sms);
     }
     if (v.smem_refine == 2)
-        return launch_refine<P, C>(k_dist_refine<P, C, 2, kTravAll, true>, stages + filt + v.nd * int(sizeof(ShapeRec64)), v,
+        return launch_refine<P, C>(k_dist_refine<P, C, 2, kTravAll>, stages + filt + v.nd * int(sizeof(ShapeRec64)), v,
                                    b, step, hit, bpoint, nref, s, num_sms);
     if (v.smem_refine == 1)
-        return launch_refine<P, C>(k_dist_refine<P, C, 1, kTravAll, true>, stages + filt, v, b, step, hit, bpoint, nref, s,
+        return launch_refine<P, C>(k_dist_refine<P, C, 1, kTravAll>, stages + filt, v, b, step, hit, bpoint, nref, s,
                                    num_sms);
-    return launch_refine<P, C>(k_dist_refine<P, C, 0, kTravAll, true>, stages, v, b, step, hit, bpoint, nref, s, num_sms);
+    return launch_refine<P, C>(k_dist_refine<P, C, 0, kTravAll>, stages, v, b, step, hit, bpoint, nref, s, num_sms);
 }
 
 }  // namespace geonav

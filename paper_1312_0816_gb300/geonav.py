@@ -609,7 +609,8 @@ def geo_dist_to_boundary_adjoint(vol: Volume, x, y, z, dx, dy, dz, hit, grad_ste
     nd = vol.n_daughters
     gp = torch.empty((3, n), dtype=f64, device=x.device)
     gd = torch.empty((3, n), dtype=f64, device=x.device)
-    # (the reduction writes every element; an empty basket launches nothing)
+    # (the reduction writes every row of the daughters and the mother's parameters, which
+    # is all that is returned; an empty basket launches nothing)
     make = torch.empty if n > 0 else torch.zeros
     gt = make((max(nd, 1), 3), dtype=f64, device=x.device) if want_geometry else None
     gprm = make((nd + 1, 5), dtype=f64, device=x.device) if want_geometry else None
