@@ -1041,6 +1041,8 @@ def main():
             "algorithmic_per_track": {"hbm_bytes": hbm_bytes, "fp64_dfma_equiv": ops64, "fp32_instr": ops32},
             "fp64_count": "the mother's exit on every track, the winning daughter's transform and "
                           "DistFromOutside, the boundary point",
+            "frac_note": "of the plain algorithm's operations: the kernel evaluates the one surface that "
+                         "decides, so the FP64 unit is less busy than frac says (63 % in the committed profile)",
             "winner_only": {"fp64_dfma_equiv": ops64_winner,
                             "frac": n * ops64_winner * 2 / launch_s / 1e12 / PEAK_FP64_TFLOPS,
                             "note": "the FP64 work the filter leaves: the winner's evaluation alone "

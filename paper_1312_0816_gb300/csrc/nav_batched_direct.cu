@@ -7,11 +7,12 @@
 // tables are read through L1.
 //
 // What bounds it: latency of the lanes' record gathers through L1 (a third of
-// the warps' time) with issue slots at 60 % and the FP64 unit at 55 %.  64
+// the warps' time) with issue slots at 62 % and the FP64 unit at 51 %.  64
 // volumes of 4 to 200 daughters, 2^22 tracks: 675 us with producer and consumer warps over
-// tables staged per tile, 616 us here (32 warps per SM 660, 24 657; two blocks of
-// 448 threads 641; parts of 192 tracks 630, of 64 644; chunks of 14 parts claimed by a block, so that an SM's
-// warps share a volume, 734: the last chunks run alone).
+// tables staged per tile, 617 us here (parts of 192 tracks 630, of 64 644).  Tracks that
+// start on a daughter's surface, where FP32 is certain of nothing, are the exception:
+// 524288 of them in the toy detector 276 us with the producers' lists, 405 here, where
+// about half of them take the FP32 pass twice (refine_again).
 #include <cuda_runtime.h>
 
 #include "geo_internal.h"

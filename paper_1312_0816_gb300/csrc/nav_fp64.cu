@@ -348,12 +348,17 @@ __global__ void __launch_bounds__(256) k_safety_fp64(VolView v, Basket b, double
         return cudaGetLastError();                                                           \
     } while (0)
 
-// One warp per track when the basket is small (at most 8 tracks per SM: the
-// latency of a track's serial daughter loop would set the time) and the
+// One warp per track, in both modes, when the basket is small (at most 8 tracks per
+// SM: the latency of a track's serial daughter loop would set the time) and the
 // daughters fit one pass of the lanes (at most 32).  With more daughters, or
 // more tracks, the warp's FP64 instructions -- charged in full whatever the
-// lanes that take part -- outweigh the latency it hides (the 40-daughter toy
-// detector: 53 us per call instead of 36 us at 16..1024 tracks).
+// lanes that take part -- outweigh the latency it hides.  Per call (graphs of 20
+// calls), the kernel that would take the basket otherwise -> this one, 16 and 1024 tracks:
+// GEO_FP64 (lists per lane) four boxes 8.3 -> 8.1 and 10.5 -> 8.6 us, eight solids of
+// the toy detector 13.7 -> 15.6 and 17.7 -> 18.2, four polycones 21.2 -> 15.3 and 61.4
+// -> 22.7; GEO_FP32_REFINE four polycones (pipelined) 14.8 -> 15.5 and 48.7 -> 22.7.
+// (The direct kernel, newer than this rule, would take 4.2 and 5.1 us for the boxes and
+// 6.3 and 11.7 for the eight solids.)
 bool small_basket(const VolView& v, int64_t n, int num_sms) {
     return !v.voxelized && v.nd <= 32 && n <= int64_t(8) * num_sms;
 }

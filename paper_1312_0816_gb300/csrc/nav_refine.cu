@@ -360,8 +360,8 @@ cudaError_t launch_dist_batched(const BatchView& bv, const Basket& b, double* st
 
 // A small basket in a volume of many daughters takes the split kernel
 // (split_basket()); otherwise volumes of boxes, tubes and cones without a grid
-// take the direct kernel whatever the size (per call against the pipelined
-// kernel: toy detector 19457 tracks 29.1 -> 21.8 us, 2^20 218 -> 140 us; with a
+// take the direct kernel whatever the size (against the pipelined kernel: toy
+// detector 19457 tracks 29.1 -> 21.8 us, 2^20 218 -> 138 us; with a
 // grid nav_refine_grid.cu), and
 // the others the pipelined one: its latency configuration for a basket of at
 // most two tiles of 256 tracks per resident block (two blocks per SM), else its

@@ -49,13 +49,10 @@ __global__ void __launch_bounds__(kGrid, kGridBlocks)
 }
 
 // What bounds it: issue slots (80 %) at 9 of 32 lanes, since a warp walks as long
-// as its longest track (22 cells, the mean is 7); FP64 36 warp instructions per
+// as its longest track (22 cells, the mean is 7); FP64 41 warp instructions per
 // 32 tracks (70 with one thread per track, whose unit was 67 % busy).  512
 // daughters, 2^22 tracks: 1745 us with the walk to the mother's exit in the
-// pipelined kernel, 754 with one thread per track, 702 here (768 threads 763;
-// equal shares per warp instead of strides of the grid gave 1.5 %).  Lanes that take
-// new tracks as theirs end walk with 15 lanes active, but their state does not fit 64
-// registers beside the bounds': 1132 us, 838 with 512 threads of 128 registers.
+// pipelined kernel, 754 with one thread per track, 698 here.
 constexpr int kStaged = 1024;   // threads: one block per SM, its tables staged once
 constexpr int kOnSheet = 128;   // tracks that a warp takes at a time
 

@@ -3,8 +3,8 @@
 // a block, daughter by daughter.
 //
 // A basket of a few thousand tracks leaves most of the GPU idle, and its time
-// is the latency of one tile: in the pipelined kernel a warp walks every
-// daughter of the volume for its 32 tracks, one after the other.  Here a block
+// is the latency of one warp's 32 tracks: in the kernels for large baskets a warp
+// tests every daughter of the volume for them, one after the other.  Here a block
 // takes 32 tracks (one per lane) and kSplitWarps warps; warp w bounds the
 // mother and daughters w, w + kSplitWarps, ... for all 32 tracks.  The warps'
 // candidate lists are merged per track, and each track's first FP64 task is
@@ -125,18 +125,17 @@ __global__ void __launch_bounds__(kSplitWarps * 32, kSplitBlocksPerSm)
     if (nref) nref[i] = nev;
 }
 
-// Volumes of more than 32 daughters (smaller volumes keep the warp-per-track
-// kernel or the pipelined one), baskets that fill at most one wave of blocks
+// Volumes of more than 32 daughters (smaller volumes take the warp-per-track
+// kernel, or those of large baskets), baskets that fill at most one wave of blocks
 // (four 256-thread blocks per SM at 64 registers), two waves from 128
 // daughters on in a volume without a uniform grid.  A volume with a grid is
 // walked here daughter by daughter all the same: for a small basket the
-// shared walk beats each lane's own walk through the cells.  Measured per
-// call (CUDA graph of one call), pipelined kernel -> this one: toy detector
-// (40 daughters) 16 tracks 21.8 -> 16.3 us, 1024 28.7 -> 18.3, 16384 30.7 ->
-// 26.5, 32768 32.7 -> 40.9; 512 daughters without the grid 16 tracks 126.9
-// -> 30.0 us, 16384 118.8 -> 34.8, 32768 118.8 -> 59.3, 65536 124.9 ->
-// 100.3; the same with the grid (the pipelined kernel walking it) 16 tracks
-// 45.0 -> 28.6 us, 16384 55.2 -> 34.8, 32768 55.3 -> 59.3.
+// shared walk beats each lane's own walk through the cells.  Per call (graphs of
+// 20 calls), the kernel that would take the basket otherwise -> this one: toy
+// detector (direct) 16 tracks 9.8 -> 10.3 us, 1024 12.0 -> 10.8, 4096 15.0 -> 11.0,
+// 16384 18.4 -> 21.3; 512 daughters without the grid (direct) 16 tracks 61.6 ->
+// 23.3, 16384 74.0 -> 30.9, 32768 74.2 -> 49.4; the same with the grid (k_dist_grid)
+// 16 tracks 23.4 -> 23.2, 1024 36.5 -> 30.4, 16384 34.8 -> 31.0.
 bool split_basket(const VolView& v, int64_t n, int num_sms) {
     const int64_t wave = int64_t(kSplitBlocksPerSm) * num_sms * 32;
     return v.nd > 32 && n <= (v.nd >= 128 && !v.voxelized ? 2 : 1) * wave;

@@ -71,8 +71,8 @@ __global__ void __launch_bounds__(256) k_shape(const __grid_constant__ ShapeArg 
 // distance, decides misses, and the zones keep margins that grow alike.  Directions
 // outside the FP32 range take the whole routine.
 //
-// What bounds it: the latency of the FP64 chains; 22 FP64 instructions per 32 tracks of
-// a placed cone, of which a quarter hit.  DistFromOutside of 2^20 tracks: k_shape 229 us
+// What bounds it: the latency of the FP64 chains (FP64 unit 64 %, issue 34 %); 26 FP64
+// instructions per 32 tracks of a placed cone, of which a quarter hit.  DistFromOutside of 2^20 tracks: k_shape 229 us
 // (113 FP64 instructions), 66 us so.  With whole batches of 128 dealt to the warps in turn
 // (1.7 for each), tracks that all need the whole routine took 15 to 30 % longer than
 // k_shape (cone, 30 radii away: 252 us and 397 for the safety against 225 and 317; 29 and

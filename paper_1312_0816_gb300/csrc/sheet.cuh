@@ -6,7 +6,7 @@
 // tracks are of both sorts pays for both.  So a warp runs the FP32 pass on up
 // to Q tracks first, keeps each track's first task and the least bound beside
 // it (8 bytes), and then evaluates them 32 at a time, the quadrics first, then
-// the planes (512 rotated solids: 36 FP64 instructions per 32 tracks instead of
+// the planes (512 rotated solids: 41 FP64 instructions per 32 tracks instead of
 // 70).  All of it is the warp's own: no barrier of the block.  The FP64 track is read
 // again from the basket (it is still in L2, and its latency is small beside
 // the FP32 pass).  Where nearly all surfaces are quadrics there is nothing to
@@ -28,9 +28,8 @@ constexpr int kTaskNone = -1;
 // A track that its first task (solid h, value s) does not settle (0.02 %, out of
 // line): the FP32 pass again, for its whole list of candidates.  This copy of the
 // pass may round a bound differently (the compiler contracts each copy's expressions
-// by itself) and name another first task; the loop over every daughter then decides.  (Marking such tracks and
-// taking them through the loop a second time: 748 us for 700 in the grid; two more
-// candidates kept per track: 709.)
+// by itself) and name another first task; the loop over every daughter then
+// decides.  (Two more candidates kept per track instead: the grid 709 us for 700.)
 template <int TRAV>
 static __device__ __noinline__ void refine_again(const VolView& v, double& s, double px, double py, double pz, double qx,
                                                  double qy, double qz, int& h, int& nev) {
