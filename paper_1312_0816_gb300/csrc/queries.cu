@@ -266,16 +266,44 @@ static __device__ __noinline__ double safety_cold(const VolView& v, int j, doubl
     const double p[3] = {px, py, pz};
     return safety_of<false>(v, j, p);
 }
-// the minimum over every candidate whose bound does not exceed the running one
-static __device__ __noinline__ double safety_all_cold(const VolView& v, double s, double px, double py, double pz, float tau) {
-    const double p[3] = {px, py, pz};
-    const float p32[3] = {f64_to_f32_trunc(px), f64_to_f32_trunc(py), f64_to_f32_trunc(pz)};
-    SafetyState st;
-    st.Lm = 0.f;
-    st.L2 = 0.f;
-    st.j1 = v.nd;   // no daughter is left out
-    int nev;
-    return safety_finish<false>(v, v.d32, p, p32, st, s, tau, &nev);
+// The points of a batch that their two nearest candidates do not settle (marked in
+// k2; L2: the bound above which no candidate matters), one after the other by the whole
+// warp: the least value of every candidate up to that bound, the mother or a daughter for
+// each lane.  They are rare (a few in 10^5), but one lane alone took 17 us over the 40
+// daughters of the toy detector, and its basket waited for it (60013 points 49 us, 27
+// without such a point).
+constexpr int kSafRest = -2;
+static __device__ __noinline__ void safety_rest(const VolView& v, SafetyBatch& B, int per, double* saf) {
+    const int lane = threadIdx.x & 31;
+    for (int base = 0; base < per; base += 32) {
+        const bool mine = base + lane < per && B.k2[base + lane] == kSafRest;
+        for (unsigned m = __ballot_sync(0xffffffffu, mine); m; m &= m - 1) {
+            const int q = base + __ffs(m) - 1;
+            const double p[3] = {B.p[0][q], B.p[1][q], B.p[2][q]};
+            const float p32[3] = {f64_to_f32_trunc(p[0]), f64_to_f32_trunc(p[1]), f64_to_f32_trunc(p[2])};
+            const float th = B.L2[q];
+            double s = d_inf();
+            for (int j = lane - 1; j < v.nd; j += 32) {
+                if (j >= 0) {
+                    const ShapeRec32& r = v.d32[j];
+                    float o[3], x[3];
+                    const float c2 = offset32(r, p32, o);
+                    if (beyond(r, c2, th)) continue;
+                    local32(r, o, x);
+                    if (safety_out_lb32(r, x) > th) continue;
+                }
+                s = fmin(s, safety_of<false>(v, j, p));
+            }
+            __syncwarp();
+#pragma unroll
+            for (int off = 16; off > 0; off >>= 1) s = fmin(s, __shfl_xor_sync(0xffffffffu, s, off));
+            if (lane == 0) {
+                saf[q] = s;
+                B.k2[q] = -1;
+            }
+        }
+    }
+    __syncwarp();
 }
 
 template <bool SMEM>
@@ -324,7 +352,10 @@ __global__ void __launch_bounds__(kSafWarps * 32, 4)
                         sort = per > 32 || zone == kZoneNone ? zone_sort(zone) : 0;
                     }
                 }
-                if (zone == kZoneInside) saf[i] = 0.0;
+                if (zone == kZoneInside) {
+                    saf[i] = 0.0;
+                    B.k2[o] = -1;
+                }
             }
 #pragma unroll
             for (int s = 0; s < kZoneSorts; ++s) {
@@ -334,6 +365,7 @@ __global__ void __launch_bounds__(kSafWarps * 32, 4)
             }
         }
         __syncwarp();
+        bool rest = false;
         // 32 points of one sort at a time (one copy of the code: c counts up through the sorts)
         for (int sort = 0, c = 0; sort < kZoneSorts;) {
             const int n = sort == 0 ? cnt[0] : (sort == 1 ? cnt[1] : (sort == 2 ? cnt[2] : cnt[3]));
@@ -352,13 +384,18 @@ __global__ void __launch_bounds__(kSafWarps * 32, 4)
                 if (!(B.L2[o] > above(r, tau))) {
                     const int k2 = B.k2[o];
                     r = fmin(r, safety_cold(v, k2 < 0 ? -1 : f.hvy[k2].id, px, py, pz));
-                    if (!(B.L3[o] > above(r, tau))) r = safety_all_cold(v, r, px, py, pz, tau);
+                    if (!(B.L3[o] > above(r, tau))) {
+                        B.k2[o] = kSafRest;
+                        B.L2[o] = above(r, tau);
+                        rest = true;
+                    }
                 }
                 saf[first + o] = r;
             }
             __syncwarp();
             c += 32;
         }
+        if (__any_sync(0xffffffffu, rest)) safety_rest(v, B, per, saf + first);
     }
 }
 

@@ -359,3 +359,24 @@ def test_starts_on_the_daughters_surfaces(g, scene):
         assert torch.equal(g.geo_contains(flat, *part, mode=g.GEO_FP64), g.geo_contains(flat, *part))
         a, b = g.geo_safety(flat, *part, mode=g.GEO_FP64), g.geo_safety(flat, *part)
         assert torch.equal(a.view(torch.int64), b.view(torch.int64))
+
+
+@pytest.mark.parametrize("n", [33, 5003, 170003])
+@pytest.mark.parametrize("daughters", [31, 32, 40, 70])
+def test_safety_of_points_with_many_nearest_solids(g, daughters, n):
+    """Points on and near the axis of a ring of equal solids, and anywhere: more
+    than two candidates are too close to tell apart in FP32."""
+    rng = np.random.default_rng(daughters + n)
+    rows = []
+    for k in range(daughters):
+        a = 2.0 * np.pi * k / daughters
+        at = (60.0 * np.cos(a), 60.0 * np.sin(a), 0.0)
+        solid = [(scenes.BOX, (1.0, 1.5, 9.0)), (scenes.TUBE, (0.4, 1.0, 9.0)), (scenes.CONE, (9.0, 0.2, 1.0, 0.3, 1.0))][k % 3]
+        rows.append((*solid, scenes._rot_z(a), at))
+    sc = scenes._scene("ring", scenes.TUBE, (0.0, 200.0, 150.0), rows)
+    vol = g.geo_build_volume(sc)
+    p = rng.normal(0.0, 1.0, (3, n)) * rng.choice([0.0, 1e-12, 1e-7, 1e-5, 1e-3, 50.0], n)
+    p[2] += rng.uniform(-8.0, 8.0, n) * rng.integers(0, 2, n)
+    t = cuda(*p)
+    a, b = g.geo_safety(vol, *t, mode=g.GEO_FP64), g.geo_safety(vol, *t)
+    assert torch.equal(a.view(torch.int64), b.view(torch.int64))
