@@ -171,7 +171,7 @@ __device__ __forceinline__ MotherExit mother_exit32(const V& v, const Ray32& r, 
 // The same for a track inside the mother that starts between her shrunk copy and
 // her surface: as one that has just entered.  (Without bounds of the exit such a
 // track has the mother evaluated in FP64 first and its list after that: 524288
-// tracks that all start there took 353 us in a batch of the toy detector, 110 so.)
+// tracks that all start there took 353 us in a batch of the toy detector, 101 so.)
 // Out of line: rare among points anywhere in the mother.
 static __device__ __noinline__ MotherExit mother_exit_near32(const VolView& v, Ray32 r) {
     return mother_exit32<true>(v, r, true);

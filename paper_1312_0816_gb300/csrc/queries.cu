@@ -250,7 +250,7 @@ __global__ void __launch_bounds__(256) k_contains_lists(const __grid_constant__ 
 //
 // What bounds it: issue slots (59 %) and the FP64 unit (54 %): 2290 warp
 // instructions and 38 FP64 instructions per 32 points of the toy detector.  2^21 +
-// 77 points: 236 us; k_safety32, whole solids binned by kind with block barriers,
+// 77 points: 238 us; k_safety32, whole solids binned by kind with block barriers,
 // took 514 us with 3950 and 101.
 constexpr int kSafWarps = 8;
 constexpr int kSafBatch = 128;

@@ -37,7 +37,7 @@ __device__ __forceinline__ float f_inf() { return __int_as_float(0x7f800000); }
 // flush subnormal operands to zero are one instruction each (the others test
 // and rescale their operand); a subnormal divisor then gives an infinity
 // and a subnormal square root 0.  Both stay within the margins because the pass
-// takes no direction shorter than dd_min (geo_abi.cu dd_limit) says.
+// takes no direction shorter than the volume's dd_min (dd_limit in geo_abi.cu).
 __device__ __forceinline__ float frcp(float a) {
     float r;
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(a));
